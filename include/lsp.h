@@ -245,6 +245,13 @@ typedef struct lsp_plan lsp_plan;
  * The ablation kernels (trig or staging non-zero) are FP32, scalar
  * (packed 0), k_reseed = freqs_per_thread = 16, standard periodogram only;
  * other combinations return LSP_E_UNSUPPORTED.
+ * reserved = 1: FP32 objects with enough observations get their trig sums
+ * from a nonuniform FFT per run of 2048 bins instead of pair by pair (the
+ * same sums; its error is below the pairwise kernel's), and the kernel the
+ * other fields name serves the rest.  It is the choice of every call whose
+ * lsp_opts leave the kernel options 0, and of a plan until lsp_plan_set_config
+ * says otherwise.  It needs block_threads x freqs_per_thread = 2048 (a single
+ * object: any) and no ablation; other configurations read it as 0.
  */
 typedef struct lsp_config {
   int32_t k_reseed;
@@ -254,7 +261,7 @@ typedef struct lsp_config {
   int32_t packed;      /* 1: packed f32x2 arithmetic across two reseed chains */
   int32_t trig;
   int32_t staging;
-  int32_t reserved;
+  int32_t reserved;    /* 1: objects of enough observations take the transform path (below) */
 } lsp_config;
 
 /*
@@ -370,8 +377,9 @@ lsp_status lsp_plan_autotune_ex(lsp_plan* plan, const double* t, const void* y, 
 /*
  * The last lsp_plan_autotune(_ex) error gate: its objects (batch indices,
  * into objects) and, for the configuration it chose, each object's
- * max |P_n - P_n(FP64)| (into max_err), at most cap of each; *n = the number
- * of gate objects (0 after a cache hit or for FP64 plans).  Host only.
+ * max |P_n - P_n(FP64)| with the direct kernel of that configuration (into
+ * max_err), at most cap of each; *n = the number of gate objects (0 after a
+ * cache hit or for FP64 plans).  Host only.
  */
 lsp_status lsp_plan_gate_report(const lsp_plan* plan, int64_t* objects, float* max_err, int32_t cap,
                                 int32_t* n);

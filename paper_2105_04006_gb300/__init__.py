@@ -419,6 +419,7 @@ class Plan:
     def set_config(self, **cfg):
         c = Config()
         _check(lib().lsp_plan_get_config(self._h, ctypes.byref(c)))
+        c.reserved = 0  # a named kernel configuration runs that kernel, not the transform
         for k, v in cfg.items():
             setattr(c, k, int(v))
         _check(lib().lsp_plan_set_config(self._h, ctypes.byref(c)))

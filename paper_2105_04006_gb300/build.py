@@ -43,15 +43,20 @@ def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
     srcs = sources()
     deps = srcs + [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cuh", ".h"))]
     deps.append(os.path.join(HERE, "..", "include", "lsp.h"))
-    deps.append(os.path.abspath(__file__))
+    gen = os.path.join(CSRC, "gen_transform_tables.py")
+    deps += [os.path.abspath(__file__), gen]
     if not force and not _stale(LIB, deps):
         return LIB
     nvcc = _nvcc()
     objs = []
+    tables = subprocess.run([sys.executable, gen, os.path.join(OUT_DIR, "lsp_transform_tables.inc")],
+                            capture_output=True, text=True)
+    if tables.returncode != 0:
+        raise RuntimeError(f"{gen} failed:\n{tables.stderr}")
 
     def compile_one(src):
         obj = os.path.join(OUT_DIR, os.path.basename(src)[:-3] + ".o")
-        cmd = [nvcc, *ARCH, *NVCC_FLAGS, *extra_flags, "-c", src, "-o", obj]
+        cmd = [nvcc, *ARCH, *NVCC_FLAGS, "-I", OUT_DIR, *extra_flags, "-c", src, "-o", obj]
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError(f"nvcc failed for {src}:\n{r.stdout}\n{r.stderr}")

@@ -67,6 +67,9 @@ int current_sm_count() {
 struct Layout {
   int prec, packed, k, fpt, threads, split, top_k, top, norm, center, gls;
   int abl = 0;  // ablation kernel code (lsp_config trig + 3 * staging)
+  int tf = 0;   // transform path (lsp_transform.cu) for objects of at least tf_min observations
+  int tf_min = 0, tf_grid = 0;
+  int cfg_split = 0;  // the direct kernel's split of a single object that takes the transform
   int64_t n_obj, total_nt, n_f;
   double f_min, df;
   int32_t n_chunks, n_res_chunks;
@@ -80,6 +83,12 @@ constexpr int kMinObsPerSplit = 32;
 constexpr int kMaxObsPerSplit = 8192;  // bounds each FP32 partial sum
 constexpr int kMaxSplit = 256;
 constexpr int kGateObjects = 8;  // objects the autotuner's error gate checks
+
+// Objects with at least this many observations take the transform path: its
+// cost per run of bins hardly depends on N_t, the direct kernel's is
+// proportional to it.  Measured (2000 objects of equal N_t, N_f = 1e5,
+// transform | direct, ms): N_t 32 2.2 | 1.9, 48 2.2 | 2.6, 100 2.4 | 5.0.
+constexpr int kTfMinObs = 40;
 
 lsp_status check_grid(const lsp_grid* g) {
   if (!g) return fail(LSP_E_ARG, "grid is NULL");
@@ -120,6 +129,11 @@ lsp_status resolve(int64_t n_obj, int64_t total_nt, const lsp_grid* g, const lsp
   l.gls = gls ? 1 : 0;
 
   int k, fpt, threads, packed, split_req, abl = 0;
+  // the transform is the library's own choice: a call that names a kernel
+  // option gets the direct kernel it names
+  bool tf = l.prec == LSP_FP32;
+  if (cfg) tf = tf && cfg->reserved == 1;
+  else tf = tf && !o.k_reseed && !o.freqs_per_thread && !o.block_threads && !o.obs_split;
   if (cfg) {
     k = cfg->k_reseed;
     fpt = cfg->freqs_per_thread;
@@ -177,7 +191,18 @@ lsp_status resolve(int64_t n_obj, int64_t total_nt, const lsp_grid* g, const lsp
     }
     if (split > kMaxSplit) split = kMaxSplit;
   }
+  tf = tf && !abl && n_obj > 0 && (n_obj == 1 ? total_nt >= kTfMinObs : chunk == kTfBins);
+  const int64_t tf_chunks = (l.n_f + kTfBins - 1) / kTfBins;
+  tf = tf && n_obj * tf_chunks < ((int64_t)1 << 31);  // 32-bit item numbers
+  l.tf = tf;
+  l.tf_min = kTfMinObs;
   l.split = split;
+  if (tf && n_obj == 1) {  // no direct kernel, no observation split
+    l.n_chunks = (int32_t)tf_chunks;
+    l.split = 1;
+    l.cfg_split = split;
+  }
+  split = l.split;
   const int64_t cchunk = (int64_t)kCombineThreads * kCombinePerThread;
   l.n_res_chunks = split > 1 ? (int32_t)((l.n_f + cchunk - 1) / cchunk) : l.n_chunks;
   l.n_items = n_obj * (int64_t)l.n_chunks * split;
@@ -192,7 +217,7 @@ lsp_status resolve(int64_t n_obj, int64_t total_nt, const lsp_grid* g, const lsp
   l.off_rec = take((size_t)total_nt * (l.prec ? sizeof(RecF64) : sizeof(RecF32)));
   l.off_order = take(n_obj > 1 ? (size_t)n_obj * sizeof(int32_t) : 0);
   l.off_hist = take(n_obj > 1 ? (LSP_HIST_BINS + 1) * sizeof(uint32_t) : 0);
-  l.off_queue = take(16);
+  l.off_queue = take(24);
   l.off_best = take((size_t)n_obj * l.n_res_chunks * sizeof(ChunkBest));
   l.off_cand = take(l.top ? (size_t)n_obj * l.n_res_chunks * sizeof(ChunkCand) : 0);
   // partial sums: 4 per frequency, the generalized periodogram's 6 in slots of 8
@@ -208,6 +233,16 @@ lsp_status resolve(int64_t n_obj, int64_t total_nt, const lsp_grid* g, const lsp
   int64_t grid = (int64_t)bps * current_sm_count();
   if (grid > l.n_items) grid = l.n_items;
   l.grid = (int)(grid < 1 ? 1 : grid);
+  if (l.tf) {
+    int tb = transform_blocks_per_sm(l.gls);
+    if (tb <= 0) {
+      cudaGetLastError();
+      tb = 1;
+    }
+    int64_t tg = (int64_t)tb * current_sm_count();
+    if (tg > l.n_items) tg = l.n_items;
+    l.tf_grid = (int)(tg < 1 ? 1 : tg);
+  }
   return LSP_OK;
 }
 
@@ -240,14 +275,45 @@ lsp_status run(const Layout& L, const double* t, const void* y, const int64_t* o
                                     st, L.gls != 0, dy),
              "prologue");
   } else {
-    LSP_CUDA(cudaMemsetAsync(queue, 0, 16, st), "queue reset");
+    LSP_CUDA(cudaMemsetAsync(queue, 0, 24, st), "queue reset");
     LSP_CUDA(launch_stats(t, y, y64, offsets, L.n_obj, L.total_nt, L.center, L.norm, obj, st, L.gls != 0,
                           dy, L.n_obj == 1 ? ws + L.off_stats : nullptr, queue + 1),
              "prologue (statistics)");
     LSP_CUDA(launch_records(t, y, y64, obj, L.n_obj, L.total_nt, L.f_min, L.df, y64, rec, st, L.gls != 0, dy),
              "prologue (records)");
   }
-  if (order) LSP_CUDA(launch_lpt_order(obj, L.n_obj, hist, order, st), "work-queue order");
+  // queue[3]: the transform's work counter; queue[4], queue[5]: list lengths
+  if (order && L.tf)
+    LSP_CUDA(launch_split_order(obj, L.n_obj, L.tf_min, L.n_chunks, hist, order, queue + 4, st), "work lists");
+  else if (order)
+    LSP_CUDA(launch_lpt_order(obj, L.n_obj, hist, order, st), "work-queue order");
+  const bool tf_peak = L.tf && !order && !L.top && peaks;  // the transform kernel writes the peak
+  if (L.tf) {
+    TransformParams tp;
+    tp.rec = (const RecF32*)rec;
+    tp.obj = obj;
+    tp.order_back = order ? order + (L.n_obj - 1) : nullptr;
+    tp.power_out = (float*)power_out;
+    tp.best = best;
+    tp.cand = cand;
+    tp.queue = queue + 3;
+    tp.n_items_dev = order ? queue + 4 : nullptr;
+    tp.n_items = (uint32_t)L.n_items;
+    tp.n_chunks = L.n_chunks;
+    tp.n_f = L.n_f;
+    tp.peaks = tf_peak ? peaks : nullptr;
+    tp.f_min = L.f_min;
+    tp.df = L.df;
+    tp.ticket = queue + 2;
+    if (ev_main0) LSP_CUDA(cudaEventRecordWithFlags(ev_main0, st, cudaEventRecordExternal), "timing event");
+    LSP_CUDA(launch_transform(tp, L.gls, L.tf_grid, st), "transform kernel");
+    if (!order) {
+      if (ev_main1) LSP_CUDA(cudaEventRecordWithFlags(ev_main1, st, cudaEventRecordExternal), "timing event");
+      if (peaks && !tf_peak)
+        LSP_CUDA(launch_finalize(obj, best, cand, 1, L.n_chunks, L.top_k, L.f_min, L.df, peaks, st), "finalize");
+      return LSP_OK;
+    }
+  }
   MainLaunch ml;
   ml.prec = L.prec;
   ml.packed = L.packed;
@@ -270,8 +336,9 @@ lsp_status run(const Layout& L, const double* t, const void* y, const int64_t* o
   ml.n_chunks = L.n_chunks;
   ml.split = L.split;
   ml.n_items = L.n_items;
+  if (L.tf) ml.n_items_dev = queue + 5;  // the objects the transform left
   // External records become event-record nodes when captured into a graph.
-  if (ev_main0) LSP_CUDA(cudaEventRecordWithFlags(ev_main0, st, cudaEventRecordExternal), "timing event");
+  if (ev_main0 && !L.tf) LSP_CUDA(cudaEventRecordWithFlags(ev_main0, st, cudaEventRecordExternal), "timing event");
   LSP_CUDA(launch_main(ml, st), "main kernel");
   if (ev_main1) LSP_CUDA(cudaEventRecordWithFlags(ev_main1, st, cudaEventRecordExternal), "timing event");
   // one object, first maximum: the combine kernel writes the peak itself
@@ -491,7 +558,8 @@ lsp_config config_of(const Layout& L) {
   c.k_reseed = L.k;
   c.freqs_per_thread = L.fpt;
   c.block_threads = L.threads;
-  c.obs_split = L.split;
+  c.obs_split = L.tf && L.n_obj == 1 ? L.cfg_split : L.split;
+  c.reserved = L.tf;
   c.packed = L.packed;
   c.trig = L.abl % 3;
   c.staging = L.abl / 3;
@@ -589,6 +657,7 @@ bool cache_lookup(const char* path, const std::string& key, lsp_config* c) {
         get("block_threads", &t.block_threads) && get("obs_split", &t.obs_split) &&
         get("packed", &t.packed)) {
       get("trig", &t.trig);        // absent in older entries: 0
+      get("transform", &t.reserved);
       get("staging", &t.staging);
       *c = t;
       found = true;
@@ -603,7 +672,7 @@ void cache_store(const char* path, const std::string& key, const lsp_config& c, 
   f << "{\"key\": \"" << key << "\", \"k_reseed\": " << c.k_reseed << ", \"freqs_per_thread\": "
     << c.freqs_per_thread << ", \"block_threads\": " << c.block_threads << ", \"obs_split\": "
     << c.obs_split << ", \"packed\": " << c.packed << ", \"trig\": " << c.trig << ", \"staging\": "
-    << c.staging << ", \"ms\": " << ms << ", \"max_err\": " << err
+    << c.staging << ", \"transform\": " << c.reserved << ", \"ms\": " << ms << ", \"max_err\": " << err
     << "}\n";
 }
 
@@ -831,9 +900,13 @@ lsp_status lsp_plan_kernel_count(const lsp_plan* p, int32_t* count) {
   // (+ 3 for the LPT order) (+ combine) (+ finalize, which a split single
   // object with a first-maximum output folds into the combine); peaks
   // requested; plans of one object run without offsets
-  const bool fused = L.split > 1 && !L.top;
   const bool one_prologue = L.n_obj == 1 && L.total_nt <= kFusedMaxNt;
-  *count = (one_prologue ? 2 : 3) + (L.n_obj > 1 ? 3 : 0) + (L.split > 1 ? 1 : 0) + (fused ? 0 : 1);
+  if (L.tf && L.n_obj == 1) {  // prologue + transform (+ finalize for the top-k)
+    *count = (one_prologue ? 1 : 2) + 1 + (L.top ? 1 : 0);
+    return LSP_OK;
+  }
+  const bool fused = L.split > 1 && !L.top;
+  *count = (one_prologue ? 2 : 3) + (L.tf ? 1 : 0) + (L.n_obj > 1 ? 3 : 0) + (L.split > 1 ? 1 : 0) + (fused ? 0 : 1);
   return LSP_OK;
 }
 
@@ -1064,6 +1137,15 @@ lsp_status lsp_plan_autotune_ex(lsp_plan* p, const double* t, const void* y, con
     }
   }
 
+  // The transform path, where the plan's options leave the choice to the
+  // library: one more candidate, its configuration that of the direct kernel
+  // for the objects it leaves (so it comes after that candidate itself).
+  {
+    Layout Ld;
+    if ((st = resolve(p->n_obj, p->total_nt, &p->grid, &p->opts, nullptr, &Ld))) return st;
+    if (Ld.tf) cands.push_back(config_of(Ld));
+  }
+
   // Error gate (FP32): each candidate's periodograms of a few objects against
   // the FP64 path -- the first object, the one with the most observations
   // (the longest FP32 sums), the worst-conditioned one of a pool (the largest
@@ -1222,7 +1304,7 @@ lsp_status lsp_plan_autotune_ex(lsp_plan* p, const double* t, const void* y, con
     if (e != cudaSuccess) { cleanup(); return cuda_fail(e, "autotune gate inputs"); }
     if ((st = run(L64, gt, y64, g_nobj > 1 ? goff : nullptr, ref, nullptr, gws, s))) { cleanup(); return st; }
   }
-  std::vector<double> cur_err((size_t)g_rows), best_obj_err;
+  std::vector<double> cur_err((size_t)g_rows), best_obj_err, direct_err;
 
   float best_ms = 1e30f;
   double best_err = 0.0;
@@ -1275,6 +1357,13 @@ lsp_status lsp_plan_autotune_ex(lsp_plan* p, const double* t, const void* y, con
     p->L = saved;
     if (st) { cleanup(); return st; }
     record(config_of(Lc), ms, err, true, worst_obj);
+    // the report describes the direct kernel of the configuration, also
+    // where the transform, gated above like every candidate, is chosen
+    const lsp_config cc = config_of(Lc), ct = cands.back();
+    if (ct.reserved && !cc.reserved && cc.k_reseed == ct.k_reseed && cc.freqs_per_thread == ct.freqs_per_thread &&
+        cc.block_threads == ct.block_threads && cc.packed == ct.packed && !cc.trig && !cc.staging)
+      direct_err = cur_err;
+    if (cc.reserved && !direct_err.empty()) cur_err = direct_err;
     if (ms < best_ms) {
       best_ms = ms;
       best = config_of(Lc);

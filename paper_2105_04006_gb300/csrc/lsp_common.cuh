@@ -427,6 +427,34 @@ __device__ __forceinline__ void fix_ill_conditioned(float (&pv)[F], uint32_t bad
   }
 }
 
+// One thread's F consecutive powers into the object's row of the periodogram.
+template <int F>
+__device__ __forceinline__ void store_row(float* row, int64_t k0, const float (&pv)[F], int64_t n_f) {
+  if (k0 + F <= n_f && ((reinterpret_cast<uintptr_t>(row + k0) & 15) == 0)) {
+    float4* d = reinterpret_cast<float4*>(row + k0);
+#pragma unroll
+    for (int q = 0; q < F / 4; ++q)
+      __stcs(d + q, make_float4(pv[4 * q], pv[4 * q + 1], pv[4 * q + 2], pv[4 * q + 3]));
+  } else {
+#pragma unroll
+    for (int m = 0; m < F; ++m)
+      if (k0 + m < n_f) row[k0 + m] = pv[m];
+  }
+}
+
+template <int F>
+__device__ __forceinline__ void store_row(double* row, int64_t k0, const double (&pv)[F], int64_t n_f) {
+  if (k0 + F <= n_f && ((reinterpret_cast<uintptr_t>(row + k0) & 15) == 0)) {
+    double2* d = reinterpret_cast<double2*>(row + k0);
+#pragma unroll
+    for (int q = 0; q < F / 2; ++q) __stcs(d + q, make_double2(pv[2 * q], pv[2 * q + 1]));
+  } else {
+#pragma unroll
+    for (int m = 0; m < F; ++m)
+      if (k0 + m < n_f) row[k0 + m] = pv[m];
+  }
+}
+
 // ------------------------------------------------------ chunk reductions
 // (p, k) pair ordering: higher power first, lower index on ties.
 __device__ __forceinline__ bool better(double pa, int64_t ka, double pb, int64_t kb) {

@@ -85,6 +85,36 @@ int main_blocks_per_sm(int prec, int packed, int k_reseed, int fpt, int threads,
                       int abl = 0);
 size_t main_dyn_smem(int prec, int fpt, int threads, int top);
 
+// Transform path (lsp_transform.cu): the trig sums of runs of kTfBins bins by
+// a nonuniform FFT; FP32, standard and generalized periodogram.
+constexpr int kTfBins = 2048;
+struct TransformParams {
+  const RecF32* rec;
+  const ObjInfo* obj;
+  const int32_t* order_back;  // last word of the object list, read backwards (nullptr: identity)
+  float* power_out;      // nullable, n_obj x n_f
+  ChunkBest* best;
+  ChunkCand* cand;       // nullable: only with top_k > 1
+  uint32_t* queue;       // zeroed work counter
+  const uint32_t* n_items_dev;  // device item count (overrides n_items)
+  uint32_t n_items;
+  int32_t n_chunks;      // runs per object
+  int64_t n_f;
+  // one object, first maximum only: the peak is written by the last CTA
+  // (ticket: a zeroed word); NULL: a finalize launch follows
+  lsp_peak* peaks;
+  double f_min, df;
+  uint32_t* ticket;
+};
+cudaError_t launch_transform(const TransformParams& p, int gls, int grid, cudaStream_t stream);
+int transform_blocks_per_sm(int gls);
+// The work lists of a batch that takes both paths: objects of at least
+// `n_min` observations (the transform) from the back of order[], the others
+// (the direct kernel) from its front, each list by decreasing N_t;
+// items[0] and items[1] receive the two lists' lengths times n_chunks.
+cudaError_t launch_split_order(const ObjInfo* obj, int64_t n_obj, int n_min, int n_chunks, uint32_t* hist,
+                               int32_t* order, uint32_t* items, cudaStream_t stream);
+
 // Split-N_t combine (single object; gls: the generalized periodogram's six
 // sums in stride-8 slots): sums the partial sums in a fixed order,
 // evaluates the power, stores it (optional) and reduces chunk results; with

@@ -385,8 +385,11 @@ __global__ void hist_kernel(const ObjInfo* __restrict__ obj, int64_t n_obj, uint
   }
 }
 
-// Exclusive scan of LSP_HIST_BINS counters by one CTA of 1024 threads.
-__global__ void scan_kernel(uint32_t* hist) {
+// Exclusive scan of LSP_HIST_BINS counters by one CTA of 1024 threads.  With
+// items, also the lengths of launch_split_order's two work lists: the scanned
+// counter past the bins of n >= n_min is the number of those objects.
+__global__ void scan_kernel(uint32_t* hist, int64_t n_obj = 0, int n_min = 0, int n_chunks = 0,
+                            uint32_t* __restrict__ items = nullptr) {
   __shared__ uint32_t part[1024];
   constexpr int per = LSP_HIST_BINS / 1024;
   uint32_t loc[per];
@@ -406,7 +409,23 @@ __global__ void scan_kernel(uint32_t* hist) {
   uint32_t run = part[threadIdx.x] - s;
   for (int i = 0; i < per; ++i) {
     hist[threadIdx.x * per + i] = run;
+    if (items && threadIdx.x * per + i == LSP_HIST_BINS - n_min) {
+      items[0] = run * (uint32_t)n_chunks;
+      items[1] = ((uint32_t)n_obj - run) * (uint32_t)n_chunks;
+    }
     run += loc[i];
+  }
+}
+
+__global__ void split_scatter_kernel(const ObjInfo* __restrict__ obj, int64_t n_obj, int n_min, int n_chunks,
+                                     uint32_t* start, const uint32_t* __restrict__ items, int32_t* order) {
+  const int64_t n_long = items[0] / (uint32_t)n_chunks;
+  for (int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o < n_obj;
+       o += (int64_t)gridDim.x * blockDim.x) {
+    const int n = obj[o].n;
+    const int bin = LSP_HIST_BINS - 1 - (n < LSP_HIST_BINS - 1 ? n : LSP_HIST_BINS - 1);
+    const int64_t pos = atomicAdd(&start[bin], 1u);
+    order[n >= n_min ? n_obj - 1 - pos : pos - n_long] = (int32_t)o;
   }
 }
 
@@ -547,6 +566,20 @@ cudaError_t launch_lpt_order(const ObjInfo* obj, int64_t n_obj, uint32_t* hist, 
   hist_kernel<<<blocks, 256, 0, stream>>>(obj, n_obj, hist);
   scan_kernel<<<1, 1024, 0, stream>>>(hist);
   scatter_kernel<<<blocks, 256, 0, stream>>>(obj, n_obj, hist, order);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_split_order(const ObjInfo* obj, int64_t n_obj, int n_min, int n_chunks, uint32_t* hist,
+                               int32_t* order, uint32_t* items, cudaStream_t stream) {
+  if (n_obj <= 0) return cudaSuccess;
+  if (n_min < 1 || n_min >= LSP_HIST_BINS) return cudaErrorInvalidValue;
+  cudaError_t err = cudaMemsetAsync(hist, 0, sizeof(uint32_t) * LSP_HIST_BINS, stream);
+  if (err != cudaSuccess) return err;
+  int blocks = (int)((n_obj + 255) / 256);
+  if (blocks > 4096) blocks = 4096;
+  hist_kernel<<<blocks, 256, 0, stream>>>(obj, n_obj, hist);
+  scan_kernel<<<1, 1024, 0, stream>>>(hist, n_obj, n_min, n_chunks, items);
+  split_scatter_kernel<<<blocks, 256, 0, stream>>>(obj, n_obj, n_min, n_chunks, hist, items, order);
   return cudaGetLastError();
 }
 

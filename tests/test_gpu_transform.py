@@ -1,0 +1,115 @@
+"""The transform path (trig sums of a run of bins by a nonuniform FFT) against
+the FP64 CPU oracle, at the sizes where it can go wrong: either side of the
+rule that selects it, of the observation tile (256) and of the run (2048
+bins), one bin, clustered and unsorted times, spans longer than 1 / df (the
+grid wraps), and many observations in few cells.
+
+Tolerance on P_n: the sums' relative error is at most the window's aliasing
+(1.6e-7) plus the FP32 transform's and weights' rounding (about 2^-24 log2 4096
++ a few ulp, under 1e-6); a power doubles it, and dividing by N^2 - R^2 >=
+0.0975 N^2 magnifies the denominator's part by up to 10: 1.2e-5 in all.
+"""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+pytestmark = pytest.mark.gpu
+TOL = 1.2e-5
+
+
+@pytest.fixture(scope="module")
+def env():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.fail("GPU tests need CUDA")
+    from paper_2105_04006_gb300 import build
+    build.build()
+    oracle.build()
+    import paper_2105_04006_gb300 as lsp
+    return lsp, torch, torch.device("cuda", 0)
+
+
+def _segments(counts, cadence, seed):
+    r = np.random.default_rng(seed)
+    segs = []
+    for n in counts:
+        if cadence == "uniform":
+            t = np.sort(60000 + r.uniform(0, 3650, n))
+        elif cadence == "unsorted":
+            t = 60000 + r.uniform(0, 3650, n)
+        elif cadence == "one_night":
+            t = 60000.3 + r.uniform(0, 0.1, n)
+        elif cadence == "nightly":
+            t = 60000.3 + r.integers(0, 3000, n) + r.uniform(0, 1 / 24, n)
+        else:  # long: the span exceeds 1 / df many times over
+            t = np.sort(60000 + r.uniform(0, 2e5, n))
+        segs.append((t, 0.4 * np.sin(2 * np.pi * r.uniform(0.3, 5.0) * t) + r.normal(0, 0.2, n) + 3.0))
+    off = np.concatenate([[0], np.cumsum(counts)]).astype(np.int64)
+    return np.concatenate([s[0] for s in segs]), np.concatenate([s[1] for s in segs]), off
+
+
+@pytest.mark.parametrize("cadence,n_f", [("uniform", 6007), ("unsorted", 2049), ("one_night", 2048),
+                                         ("nightly", 4111), ("long", 2047), ("uniform", 1)])
+@pytest.mark.parametrize("gls", [False, True])
+def test_batch_both_sides_of_every_edge(env, cadence, n_f, gls):
+    lsp, torch, dev = env
+    counts = [3, 31, 39, 40, 41, 63, 64, 65, 255, 256, 257, 511, 513, 2600]
+    t, y, off = _segments(counts, cadence, 7)
+    y32 = y.astype(np.float32)
+    dy = np.random.default_rng(5).uniform(0.05, 0.3, t.size).astype(np.float32)
+    g = lsp.Grid(0.24, 12.0, n_f)
+    td, od = torch.tensor(t, device=dev), torch.tensor(off, device=dev)
+    yd, ed = torch.tensor(y32, device=dev), torch.tensor(dy, device=dev)
+    if gls:
+        p, pk = lsp.batch_gls(td, yd, ed, od, g, return_power=True)
+        ref = oracle.gls_batch(t, y32.astype(np.float64), dy.astype(np.float64), off, g.f_min, g.f_max, n_f)
+        tol = 1e-4  # the generalized determinant is inverted down to 0.002 W^2
+        if cadence == "one_night":
+            # a fraction of a cycle of data: the fit is near singular on every bin and FP32 magnitudes
+            # do not fix its power to 1e-4; both paths re-evaluate such bins in FP64, so they must agree
+            q, _ = lsp.batch_gls(td, yd, ed, od, g, return_power=True, k_reseed=8)
+            ref = {"power": q.cpu().numpy().astype(np.float64)}
+    else:
+        p, pk = lsp.batch(td, yd, od, g, return_power=True)
+        ref = oracle.lsp_batch(t, y32.astype(np.float64), off, g.f_min, g.f_max, n_f, return_power=True)
+        tol = TOL
+    torch.cuda.synchronize()
+    p, pk = p.cpu().numpy(), lsp.peaks_to_numpy(pk)
+    assert np.isfinite(p).all()
+    err = np.abs(p - ref["power"]).max(axis=1)
+    # three observations determine the generalized fit's three parameters:
+    # its power is 1 or, where the determinant is dropped, 0 (direct kernel)
+    err = err[1:] if gls else err
+    assert err.max() <= tol, dict(zip(counts[-len(err):], err))
+    np.testing.assert_array_equal(pk["idx"], np.argmax(p, axis=1))
+
+
+@pytest.mark.parametrize("n_t", [39, 40, 300, 2049])
+@pytest.mark.parametrize("top_k", [1, 3])
+def test_single_object(env, n_t, top_k):
+    lsp, torch, dev = env
+    b = synth.single_small(n_t=n_t, grid=synth.Grid(0.1, 10.0, 10_007))
+    t, y = torch.tensor(b.t, device=dev), torch.tensor(b.y.astype(np.float32), device=dev)
+    p, pk = lsp.periodogram(t, y, lsp.Grid(0.1, 10.0, 10_007), top_k=top_k)
+    p, pk = p.cpu().numpy(), lsp.peaks_to_numpy(pk)
+    ref, _ = oracle.lsp_single(b.t, b.y.astype(np.float32).astype(np.float64), 0.1, 10.0, 10_007)
+    assert np.max(np.abs(p - ref)) <= TOL
+    idx = [int(np.argmax(p))] if top_k == 1 else list(oracle.top_local_maxima(p.astype(np.float64), 3)[0])
+    assert list(pk["idx"]) == idx
+
+
+def test_plan_uses_the_transform_until_told_otherwise(env):
+    lsp, torch, dev = env
+    b = synth.ragged_survey(6, seed=3, grid=synth.Grid(0.24, 12.0, 3001))
+    g = lsp.Grid(0.24, 12.0, 3001)
+    args = (torch.tensor(b.t, device=dev), torch.tensor(b.y.astype(np.float32), device=dev),
+            torch.tensor(b.offsets, device=dev))
+    plan = lsp.Plan(b.n_obj, b.t.size, g)
+    _, want = lsp.batch(*args, g)
+    assert torch.equal(plan.execute(*args), want)
+    plan.set_config(k_reseed=8, freqs_per_thread=16, block_threads=128)
+    _, direct = lsp.batch(*args, g, k_reseed=8, freqs_per_thread=16, block_threads=128)
+    assert torch.equal(plan.execute(*args), direct) and not torch.equal(direct, want)
+    plan.close()

@@ -97,9 +97,10 @@ def main(path):
         # kTfPoly[d][r]: coefficient of u^d for the cell r - 3 cells from the observation's own
         emit(out, "__device__ const float kTfPoly[%d * %d]" % (deg + 1, w),
              [polys[r][d] for d in range(deg + 1) for r in range(w)], f32)
-        # kTfDeconv[i]: 1 / psi^ at offset i - m/4 of the run's centre
+        # kTfDeconv[256 s + t]: 1 / psi^ at the offset of thread t's s-th output, t/16 + 16 (t%16) + 256 s - m/4
         emit(out, "__device__ const float kTfDeconv[%d]" % (m // 2),
-             [1.0 / psi_hat((i - m // 4) / m, w, beta) for i in range(m // 2)], f32)
+             [1.0 / psi_hat((t // 16 + 16 * (t % 16) + 256 * s - m // 4) / m, w, beta)
+              for s in range(8) for t in range(256)], f32)
         # twiddles of the 4096-point transform's first two radix-16 passes
         emit(out, "__device__ const float2 kTfTw1[15 * 256]",
              [unit(p * b, 4096) for p in range(1, 16) for b in range(256)], c32, 4)

@@ -279,7 +279,8 @@ lsp_status run(const Layout& L, const double* t, const void* y, const int64_t* o
     LSP_CUDA(launch_stats(t, y, y64, offsets, L.n_obj, L.total_nt, L.center, L.norm, obj, st, L.gls != 0,
                           dy, L.n_obj == 1 ? ws + L.off_stats : nullptr, queue + 1),
              "prologue (statistics)");
-    LSP_CUDA(launch_records(t, y, y64, obj, L.n_obj, L.total_nt, L.f_min, L.df, y64, rec, st, L.gls != 0, dy),
+    LSP_CUDA(launch_records(t, y, y64, obj, L.n_obj, L.total_nt, L.f_min, L.df, y64, rec, st, L.gls != 0, dy,
+                            L.tf && L.n_obj > 1 ? L.tf_min : 0),
              "prologue (records)");
   }
   // queue[3]: the transform's work counter; queue[4], queue[5]: list lengths
@@ -300,6 +301,7 @@ lsp_status run(const Layout& L, const double* t, const void* y, const int64_t* o
     tp.n_items_dev = order ? queue + 4 : nullptr;
     tp.n_items = (uint32_t)L.n_items;
     tp.n_chunks = L.n_chunks;
+    tp.have_scale = L.n_obj > 1;
     tp.n_f = L.n_f;
     tp.peaks = tf_peak ? peaks : nullptr;
     tp.f_min = L.f_min;

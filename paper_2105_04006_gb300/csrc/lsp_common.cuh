@@ -880,4 +880,73 @@ __device__ __forceinline__ float lsp_power_f32(float xc, float xs, float cc, flo
   return den > 0.0f ? __fdividef(fmaxf(num, 0.0f), den) : 0.0f;
 }
 
+// ------------------------------------------- transform path: fixed-point scales
+// The transform (lsp_transform.cu) accumulates its grid cells in 32-bit fixed
+// point.  An observation's window covers 8 cells, so at most two neighbouring
+// groups of 8, and window values are <= 1: a cell's magnitude is at most the
+// largest count of two neighbouring groups times the largest weight.  The
+// scales put that at 2^30, half the range, and are capped so that their
+// inverses stay normal numbers.  W's observations sit at twice the phase.
+constexpr int kTfGroups = 512;
+struct TfScale {
+  float y, w, c;  // Z, W and (generalized) C
+};
+__device__ __forceinline__ void tf_count(uint32_t* count, uint32_t y_bits, uint32_t w_bits, uint32_t b_hi,
+                                         uint32_t b_lo, uint32_t& ymax, uint32_t& wmax) {
+  const uint32_t ya = y_bits & 0x7fffffffu;  // magnitudes' bits order like integers
+  ymax = ya > ymax ? ya : ymax;
+  wmax = w_bits > wmax ? w_bits : wmax;
+  const uint32_t b2 = (b_hi << 1) | (b_lo >> 31);
+  atomicAdd(&count[b_hi >> 23], 1u);
+  atomicAdd(&count[kTfGroups + (b2 >> 23)], 1u);
+}
+// The scales from the CTA's counts (complete) and each thread's largest
+// weights; every thread of the NW warps gets them.
+template <int NW>
+__device__ __forceinline__ TfScale tf_scale_block(const uint32_t* count, uint32_t ymax, uint32_t wmax,
+                                                  uint32_t (*s_max)[NW]) {
+  uint32_t cz = 1u, cw = 1u;
+  for (int g = threadIdx.x; g < kTfGroups; g += 32 * NW) {
+    const int g1 = (g + 1) & (kTfGroups - 1);
+    cz = max(cz, count[g] + count[g1]);
+    cw = max(cw, count[kTfGroups + g] + count[kTfGroups + g1]);
+  }
+  cz = __reduce_max_sync(0xffffffffu, cz);
+  cw = __reduce_max_sync(0xffffffffu, cw);
+  ymax = __reduce_max_sync(0xffffffffu, ymax);
+  wmax = __reduce_max_sync(0xffffffffu, wmax);
+  const int warp = threadIdx.x >> 5;
+  if ((threadIdx.x & 31) == 0) {
+    s_max[0][warp] = cz;
+    s_max[1][warp] = cw;
+    s_max[2][warp] = ymax;
+    s_max[3][warp] = wmax;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < NW; ++i) {
+    cz = max(cz, s_max[0][i]);
+    cw = max(cw, s_max[1][i]);
+    ymax = max(ymax, s_max[2][i]);
+    wmax = max(wmax, s_max[3][i]);
+  }
+  const float top = 1073741824.0f;
+  TfScale s;
+  s.y = fminf(top / __uint_as_float(ymax) / (float)cz, 1e37f);
+  s.w = fminf(top / __uint_as_float(wmax) / (float)cw, 1e37f);
+  s.c = fminf(top / __uint_as_float(wmax) / (float)cz, 1e37f);
+  return s;
+}
+// Once the records are written an object's t0 and mean are not read again:
+// the records kernel leaves the scales in their place.
+__device__ __forceinline__ void tf_scale_put(ObjInfo* oi, TfScale s) {
+  reinterpret_cast<float2*>(&oi->t0)[0] = make_float2(s.y, s.w);
+  reinterpret_cast<float2*>(&oi->ymean)[0] = make_float2(s.c, 0.0f);
+}
+__device__ __forceinline__ TfScale tf_scale_of(const ObjInfo& oi) {
+  const unsigned long long a = (unsigned long long)__double_as_longlong(oi.t0);
+  const unsigned long long b = (unsigned long long)__double_as_longlong(oi.ymean);
+  return TfScale{__uint_as_float((uint32_t)a), __uint_as_float((uint32_t)(a >> 32)), __uint_as_float((uint32_t)b)};
+}
+
 }  // namespace lsp

@@ -34,10 +34,12 @@ cudaError_t launch_stats(const double* t, const void* y, bool y64, const int64_t
 // it, and a zeroed ticket word, one object without offsets is reduced by
 // many CTAs; without it by one.
 size_t stats_slices_bytes(int64_t total_nt);
-cudaError_t launch_records(const double* t, const void* y, bool y64, const ObjInfo* obj,
+// tf_min > 0 (batches, FP32 records of float magnitudes): also the transform
+// path's scales of objects of at least tf_min observations (tf_scale_of).
+cudaError_t launch_records(const double* t, const void* y, bool y64, ObjInfo* obj,
                            int64_t n_obj, int64_t max_nt_single, double f_min, double df,
                            bool rec64, void* rec, cudaStream_t stream, bool gls = false,
-                           const void* dy = nullptr);
+                           const void* dy = nullptr, int tf_min = 0);
 // One object of at most kFusedMaxNt observations: statistics and records in
 // one launch, which also clears the four work-counter words at `queue` (no
 // memset, no ticket).  Every CTA redoes the object's FP64 statistics, about
@@ -99,6 +101,7 @@ struct TransformParams {
   const uint32_t* n_items_dev;  // device item count (overrides n_items)
   uint32_t n_items;
   int32_t n_chunks;      // runs per object
+  int32_t have_scale;    // the records kernel left the scales (batches)
   int64_t n_f;
   // one object, first maximum only: the peak is written by the last CTA
   // (ticket: a zeroed word); NULL: a finalize launch follows

@@ -280,8 +280,9 @@ __device__ __forceinline__ uint64_t frac_fixed64(double f, double x) {
 }
 
 // The record of observation j of an object (statistics oi).
+constexpr int kRecThreads = 128;
 template <typename YT, typename Rec, bool GLS>
-__device__ __forceinline__ void make_record(const double* __restrict__ t, const YT* __restrict__ y,
+__device__ __forceinline__ Rec make_record(const double* __restrict__ t, const YT* __restrict__ y,
                                             const YT* __restrict__ dy, int64_t j, const ObjInfo& oi, double f_min,
                                             double df, Rec* __restrict__ rec) {
   const double tp = t[j] - oi.t0;
@@ -329,19 +330,43 @@ __device__ __forceinline__ void make_record(const double* __restrict__ t, const 
     r.pad = GLS ? (uint64_t)__double_as_longlong(w) : 0ull;
   }
   rec[j] = r;
+  return r;
 }
 
 // grid.x: object; grid.y: slices of a single large object's observations.
-template <typename YT, typename Rec, bool GLS>
+// TF (batches, one CTA of 128 threads per object): also the fixed-point scales
+// of the transform path for objects of at least tf_min observations, left in
+// the object's record in place of its t0 and mean.
+template <typename YT, typename Rec, bool GLS, bool TF>
 __global__ void records_kernel(const double* __restrict__ t, const YT* __restrict__ y,
-                               const YT* __restrict__ dy, const ObjInfo* __restrict__ obj,
-                               int64_t slice, double f_min, double df, Rec* __restrict__ rec) {
+                               const YT* __restrict__ dy, ObjInfo* __restrict__ obj,
+                               int64_t slice, double f_min, double df, Rec* __restrict__ rec, int tf_min) {
   const ObjInfo oi = obj[blockIdx.x];
   if (oi.flags & (LSP_FLAG_BAD_OFFSETS | LSP_FLAG_NONFINITE)) return;
   const int64_t lo = oi.begin + (int64_t)blockIdx.y * slice;
   int64_t hi = lo + slice;
   if (hi > oi.begin + oi.n) hi = oi.begin + oi.n;
-  for (int64_t j = lo + threadIdx.x; j < hi; j += blockDim.x) make_record<YT, Rec, GLS>(t, y, dy, j, oi, f_min, df, rec);
+  if constexpr (!TF) {
+    for (int64_t j = lo + threadIdx.x; j < hi; j += blockDim.x)
+      make_record<YT, Rec, GLS>(t, y, dy, j, oi, f_min, df, rec);
+  } else {
+    __shared__ uint32_t count[2 * kTfGroups];
+    __shared__ uint32_t s_max[4][kRecThreads / 32];
+    const bool scaled = oi.n >= tf_min;
+    if (scaled)
+      for (int i = threadIdx.x; i < 2 * kTfGroups; i += kRecThreads) count[i] = 0u;
+    __syncthreads();
+    uint32_t ymax = 0u, wmax = GLS ? 0u : 0x3f800000u;
+    for (int64_t j = lo + threadIdx.x; j < hi; j += kRecThreads) {
+      const Rec r = make_record<YT, Rec, GLS>(t, y, dy, j, oi, f_min, df, rec);
+      if (scaled)
+        tf_count(count, __float_as_uint(r.y), GLS ? r.pad : 0x3f800000u, r.b_hi, r.b_lo, ymax, wmax);
+    }
+    if (!scaled) return;
+    __syncthreads();
+    const TfScale s = tf_scale_block<kRecThreads / 32>(count, ymax, wmax, s_max);
+    if (threadIdx.x == 0) tf_scale_put(obj + blockIdx.x, s);
+  }
 }
 
 // One object of at most kFusedMaxNt observations in one launch: every CTA
@@ -497,35 +522,33 @@ cudaError_t launch_stats(const double* t, const void* y, bool y64, const int64_t
   return cudaGetLastError();
 }
 
-cudaError_t launch_records(const double* t, const void* y, bool y64, const ObjInfo* obj,
+cudaError_t launch_records(const double* t, const void* y, bool y64, ObjInfo* obj,
                            int64_t n_obj, int64_t max_nt_single, double f_min, double df,
-                           bool rec64, void* rec, cudaStream_t stream, bool gls, const void* dy) {
+                           bool rec64, void* rec, cudaStream_t stream, bool gls, const void* dy, int tf_min) {
   if (n_obj <= 0) return cudaSuccess;
   int64_t slice = INT64_MAX / 4;
   unsigned gy = 1;
-  int threads = 128;
   if (n_obj == 1) {  // spread one object over many CTAs (FP64 work is slow per SM)
     slice = 256;
     gy = (unsigned)((max_nt_single + slice - 1) / slice);
     if (gy == 0) gy = 1;
-    threads = 128;
   }
   dim3 grid((unsigned)n_obj, gy);
-#define LSP_REC(YT, REC, G)                                                                        \
-  records_kernel<YT, REC, G><<<grid, threads, 0, stream>>>(t, (const YT*)y, (const YT*)dy, obj, slice, \
-                                                            f_min, df, (REC*)rec)
+#define LSP_REC(YT, REC, G, TF)                                                                          \
+  records_kernel<YT, REC, G, TF><<<grid, kRecThreads, 0, stream>>>(t, (const YT*)y, (const YT*)dy, obj, slice, \
+                                                                   f_min, df, (REC*)rec, tf_min)
   if (rec64) {
     if (y64) {
-      if (gls) LSP_REC(double, RecF64, true); else LSP_REC(double, RecF64, false);
+      if (gls) LSP_REC(double, RecF64, true, false); else LSP_REC(double, RecF64, false, false);
     } else {
-      if (gls) LSP_REC(float, RecF64, true); else LSP_REC(float, RecF64, false);
+      if (gls) LSP_REC(float, RecF64, true, false); else LSP_REC(float, RecF64, false, false);
     }
+  } else if (y64) {
+    if (gls) LSP_REC(double, RecF32, true, false); else LSP_REC(double, RecF32, false, false);
+  } else if (tf_min > 0 && gy == 1) {
+    if (gls) LSP_REC(float, RecF32, true, true); else LSP_REC(float, RecF32, false, true);
   } else {
-    if (y64) {
-      if (gls) LSP_REC(double, RecF32, true); else LSP_REC(double, RecF32, false);
-    } else {
-      if (gls) LSP_REC(float, RecF32, true); else LSP_REC(float, RecF32, false);
-    }
+    if (gls) LSP_REC(float, RecF32, true, false); else LSP_REC(float, RecF32, false, false);
   }
 #undef LSP_REC
   return cudaGetLastError();

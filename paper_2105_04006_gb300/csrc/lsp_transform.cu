@@ -55,9 +55,9 @@ namespace {
 
 constexpr int kM = 4096;                 // grid cells
 constexpr int kThreads = 256;
-constexpr int kTile = 256;               // observations staged at a time
-constexpr int kGroups = kM / 8;          // cells counted in groups of 8 for the scale
-static_assert(kTfBins == kM / 2 && kTfBins == kThreads * 8, "run length");
+constexpr int kWarps = kThreads / 32;
+constexpr size_t kPowers = kTfBins + kTfBins / 16;  // a word of padding per 16 powers
+static_assert(kTfBins == kM / 2 && kTfBins == kThreads * 8 && kTfGroups == kM / 8, "run length");
 
 // ------------------------------------------------------------ arithmetic on
 // f32x2 pairs (two transforms at once) or single floats
@@ -151,10 +151,13 @@ __device__ __forceinline__ Cx<float> get(const float* buf, int i) {
 }
 
 // The 4096-point transform of the CTA: on entry thread b holds cells
-// 256 a + b (a = 0 .. 15); on return out[s] holds the value at offset
-// m = tid + 256 s - 1024 from the run's centre, s = 0 .. 7.  buf: 4096
-// complex words, free on entry once every thread has passed the first
-// barrier here; free again only after a barrier of the caller.
+// 256 a + b (a = 0 .. 15); on return, with p = tid >> 4 and r = tid & 15,
+// out[s] holds the value at offset p + 16 r + 256 s - 1024 from the run's
+// centre, s = 0 .. 7.  buf: 4096 complex words, free once every thread has
+// passed the first barrier here; free again only after a barrier of the
+// caller.  The second exchange stays within the 16 threads of one p, in the
+// 256 words that only they read in the first one, so it needs no barrier of
+// the whole CTA.
 template <typename T>
 __device__ __forceinline__ void fft4096(Cx<T> (&x)[16], T* buf, Cx<T> (&out)[8]) {
   const int tid = threadIdx.x;
@@ -169,9 +172,10 @@ __device__ __forceinline__ void fft4096(Cx<T> (&x)[16], T* buf, Cx<T> (&out)[8])
 #pragma unroll
   for (int p = 0; p < 16; ++p) put(buf, p * 256 + tid, x[4 * (p & 3) + (p >> 2)]);
   __syncthreads();
-  const int p = tid >> 4, d = tid & 15;
+  T* const own = buf + (tid >> 4) * 512;  // 256 complex words
+  const int d = tid & 15;
 #pragma unroll
-  for (int c = 0; c < 16; ++c) x[c] = get(buf, p * 256 + 16 * c + d);
+  for (int c = 0; c < 16; ++c) x[c] = get(own, 16 * c + d);
   dft16(x);
 #pragma unroll
   for (int r = 1; r < 16; ++r) {
@@ -179,22 +183,20 @@ __device__ __forceinline__ void fft4096(Cx<T> (&x)[16], T* buf, Cx<T> (&out)[8])
     const int q = 4 * (r & 3) + (r >> 2);
     x[q] = cmul(x[q], w.x, w.y);
   }
-  __syncthreads();
-  // word (p, r, d) at r 256 + p 16 + (d ^ (p & 7)): eight lanes of either
-  // the writing order (d runs) or the reading order (p runs) touch the eight
-  // 16-byte bank groups once each
+  __syncwarp();
+  // word (r, d) at 16 r + (d ^ r): the lanes of either the writing order (d
+  // runs) or the reading order (r runs) fall on distinct banks
 #pragma unroll
-  for (int r = 0; r < 16; ++r) put(buf, r * 256 + p * 16 + (d ^ (p & 7)), x[4 * (r & 3) + (r >> 2)]);
-  __syncthreads();
-  const int p2 = tid & 15, r2 = tid >> 4;  // this thread's outputs: k = tid + 256 s
+  for (int r = 0; r < 16; ++r) put(own, 16 * r + (d ^ r), x[4 * (r & 3) + (r >> 2)]);
+  __syncwarp();
 #pragma unroll
-  for (int e = 0; e < 16; ++e) x[e] = get(buf, r2 * 256 + p2 * 16 + (e ^ (p2 & 7)));
+  for (int e = 0; e < 16; ++e) x[e] = get(own, 16 * d + (e ^ d));
   dft16_first(x);
 #pragma unroll
   for (int k1 = 0; k1 < 4; ++k1) {
     const Cx<T> x0 = x[4 * k1], x1 = x[4 * k1 + 1], x2 = x[4 * k1 + 2], x3 = x[4 * k1 + 3];
-    out[4 + k1] = (x0 + x2) + (x1 + x3);    // s = k1:      m = tid + 256 k1
-    out[k1] = sub_i(x0 - x2, x1 - x3);      // s = 12 + k1: m = tid + 256 k1 - 1024
+    out[4 + k1] = (x0 + x2) + (x1 + x3);    // s = k1 of the transform's 16
+    out[k1] = sub_i(x0 - x2, x1 - x3);      // s = 12 + k1
   }
 }
 
@@ -203,16 +205,15 @@ __device__ __forceinline__ f2_t cells_f2(const int32_t* a, const int32_t* b, int
 }
 
 // Shared memory: grid planes (the exchange buffer after the grid is read),
-// staged observations (the run's powers later), group counts.
+// staged observations (group counts before, the run's powers after them).
 template <bool GLS>
 struct Smem {
   static constexpr int kPlanes = GLS ? 6 : 4;
   static constexpr int kStage = GLS ? 48 : 32;  // bytes per staged observation
   static constexpr size_t grid = (size_t)kPlanes * kM * 4;
-  static constexpr size_t stage = (size_t)kTile * kStage;
-  static constexpr size_t counts = (size_t)2 * kGroups * 4;
-  static constexpr size_t total = grid + stage + counts;
-  static_assert(stage >= kTfBins * 4, "the run's powers use the staging area");
+  static constexpr size_t stage = (size_t)kThreads * kStage > kPowers * 4 ? (size_t)kThreads * kStage : kPowers * 4;
+  static constexpr size_t total = grid + stage;
+  static_assert(stage >= 2 * kTfGroups * 4, "the counts use the staging area");
 };
 
 // Eq. 2 from Z and W (lsp_power_f32 with its sums already combined).
@@ -234,19 +235,27 @@ __global__ void __launch_bounds__(kThreads, 2) transform_kernel(TransformParams 
   extern __shared__ __align__(128) unsigned char dyn_smem[];
   int32_t* const plane = reinterpret_cast<int32_t*>(dyn_smem);
   unsigned char* const stage = dyn_smem + S::grid;
-  uint32_t* const count = reinterpret_cast<uint32_t*>(dyn_smem + S::grid + S::stage);
   __shared__ unsigned long long red[32];
-  __shared__ float s_edge[4 * (kThreads / 32) + 2];
-  __shared__ uint32_t s_max[4][kThreads / 32];
+  __shared__ float s_edge[4 * kWarps + 2];
+  __shared__ uint32_t s_max[4][kWarps];
   __shared__ uint32_t s_item;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t n_items = p.n_items_dev ? *p.n_items_dev : p.n_items;
   const uint32_t n_chunks = (uint32_t)p.n_chunks;
+  f2_t poly[9];  // of this lane's cell, lane & 7
+#pragma unroll
+  for (int d = 0; d < 9; ++d) poly[d] = dup_<f2_t>(__ldg(&kTfPoly[d * 8 + (lane & 7)]));
+  auto clear_grid = [&]() {
+    int4* g4 = reinterpret_cast<int4*>(plane);
+#pragma unroll
+    for (int i = 0; i < S::kPlanes * kM / 4 / kThreads; ++i) g4[tid + i * kThreads] = make_int4(0, 0, 0, 0);
+  };
+  clear_grid();
 
   uint32_t ticket = blockIdx.x;  // first item static, then one ticket ahead (as in main_f32_packed_body)
   for (;;) {
     if (tid == 0) s_item = ticket;
-    __syncthreads();
+    __syncthreads();  // also: the grid is clear
     const uint32_t item = s_item;
     if (item >= n_items) break;
     if (tid == 0) ticket = gridDim.x + atomicAdd(p.queue, 1u);
@@ -259,110 +268,80 @@ __global__ void __launch_bounds__(kThreads, 2) transform_kernel(TransformParams 
     const int n = oi.flags ? 0 : oi.n;  // flagged objects: zero power
     const uint4* rec = reinterpret_cast<const uint4*>(p.rec + oi.begin);
 
-    // ---- group counts and largest weights, for the fixed-point scales
-    for (int i = tid; i < 2 * kGroups; i += kThreads) count[i] = 0u;
-    {
-      int4* g4 = reinterpret_cast<int4*>(plane);
-#pragma unroll
-      for (int i = 0; i < S::kPlanes * kM / 4 / kThreads; ++i) g4[tid + i * kThreads] = make_int4(0, 0, 0, 0);
-    }
-    __syncthreads();
-    uint32_t ymax = 0u, wmax = GLS ? 0u : 0x3f800000u;  // magnitudes' bits order like integers
-    for (int j = tid; j < n; j += kThreads) {
-      const uint4 r0 = __ldg(rec + 2 * j), r1 = __ldg(rec + 2 * j + 1);
-      const uint32_t ya = r0.x & 0x7fffffffu;
-      ymax = ya > ymax ? ya : ymax;
-      if (GLS) wmax = r1.w > wmax ? r1.w : wmax;
-      const uint32_t b2 = (r1.x << 1) | (r1.y >> 31);
-      atomicAdd(&count[r1.x >> 23], 1u);
-      atomicAdd(&count[kGroups + (b2 >> 23)], 1u);
-    }
-    __syncthreads();
-    uint32_t cz = 0u, cw = 0u;
-#pragma unroll
-    for (int i = 0; i < kGroups / kThreads; ++i) {
-      const int g = tid + i * kThreads, g1 = (g + 1) & (kGroups - 1);
-      cz = max(cz, count[g] + count[g1]);
-      cw = max(cw, count[kGroups + g] + count[kGroups + g1]);
-    }
-    cz = __reduce_max_sync(0xffffffffu, cz);
-    cw = __reduce_max_sync(0xffffffffu, cw);
-    ymax = __reduce_max_sync(0xffffffffu, ymax);
-    wmax = __reduce_max_sync(0xffffffffu, wmax);
-    if (lane == 0) {
-      s_max[0][warp] = cz;
-      s_max[1][warp] = cw;
-      s_max[2][warp] = ymax;
-      s_max[3][warp] = wmax;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < kThreads / 32; ++i) {
-      cz = max(cz, s_max[0][i]);
-      cw = max(cw, s_max[1][i]);
-      ymax = max(ymax, s_max[2][i]);
-      wmax = max(wmax, s_max[3][i]);
-    }
-    // |cell| <= (observations in two neighbouring groups) x (largest weight)
-    // <= 2^30, a factor of two under the overflow; capped so that the
-    // scale's inverse stays a normal number
-    const float y_sc = fminf(1073741824.0f / __uint_as_float(ymax) / (float)(cz ? cz : 1u), 1e37f);
-    const float w_sc = fminf(1073741824.0f / __uint_as_float(wmax) / (float)(cw ? cw : 1u), 1e37f);
-    const float c_sc = GLS ? fminf(1073741824.0f / __uint_as_float(wmax) / (float)(cz ? cz : 1u), 1e37f) : 0.0f;
-
-    // ---- spread
-    float poly[9];
-#pragma unroll
-    for (int d = 0; d < 9; ++d) poly[d] = __ldg(&kTfPoly[d * 8 + (lane & 7)]);
-    for (int ts = 0; ts < n; ts += kTile) {
-      const int j = ts + tid;
-      if (j < n) {
+    // ---- fixed-point scales: the records kernel's, or counted here
+    TfScale sc;
+    if (p.have_scale) {
+      sc = tf_scale_of(oi);
+    } else {
+      uint32_t* const count = reinterpret_cast<uint32_t*>(stage);
+      for (int i = tid; i < 2 * kTfGroups; i += kThreads) count[i] = 0u;
+      __syncthreads();
+      uint32_t ymax = 0u, wmax = GLS ? 0u : 0x3f800000u;
+      for (int j = tid; j < n; j += kThreads) {
         const uint4 r0 = __ldg(rec + 2 * j), r1 = __ldg(rec + 2 * j + 1);
-        const uint32_t ph = phase_hi32(r0.w, r1.x, r1.y, kc);
-        float s, c;
-        sincospif(__int2float_rn((int)ph) * 4.656612873077393e-10f, &s, &c);  // 2^-31 half-cycles
-        const float ys = __uint_as_float(r0.x) * y_sc;
-        const float ws = GLS ? __uint_as_float(r1.w) * w_sc : w_sc;
-        // position in cells, 12 bits of cell and 32 of fraction
-        const uint32_t fz = (r1.x << 12) | (r1.y >> 20), b2 = (r1.x << 1) | (r1.y >> 31), lo2 = r1.y << 1;
-        const uint32_t fw = (b2 << 12) | (lo2 >> 20);
-        const float uz = fmaf(__uint2float_rn(fz), 2.3283064365386963e-10f, -0.5f);
-        const float uw = fmaf(__uint2float_rn(fw), 2.3283064365386963e-10f, -0.5f);
-        float4* st = reinterpret_cast<float4*>(stage + (size_t)tid * S::kStage);
-        st[0] = make_float4(__uint_as_float((r1.x >> 20) - 3u), uz, __uint_as_float((b2 >> 20) - 3u), uw);
-        st[1] = make_float4(ys * c, ys * s, ws * (c - s) * (c + s), ws * 2.0f * c * s);
-        if (GLS) {
-          const float cs = __uint_as_float(r1.w) * c_sc;
-          st[2] = make_float4(cs * c, cs * s, 0.0f, 0.0f);
-        }
+        tf_count(count, r0.x, GLS ? r1.w : 0x3f800000u, r1.x, r1.y, ymax, wmax);
       }
       __syncthreads();
-      const int nt = min(kTile, n - ts);
-#pragma unroll 2
-      for (int i = 4 * warp + (lane >> 3); i < nt; i += kThreads / 8) {
-        const float4* st = reinterpret_cast<const float4*>(stage + (size_t)i * S::kStage);
-        const float4 at = st[0], v = st[1];
-        const float uz = at.y, uw = at.w;
-        float wz = poly[8], ww = poly[8];
-#pragma unroll
-        for (int d = 7; d >= 0; --d) {
-          wz = fmaf(wz, uz, poly[d]);
-          ww = fmaf(ww, uw, poly[d]);
-        }
-        const int lz = (int)(__float_as_uint(at.x) + (uint32_t)(lane & 7)) & (kM - 1);
-        const int lw = (int)(__float_as_uint(at.z) + (uint32_t)(lane & 7)) & (kM - 1);
-        atomicAdd(&plane[0 * kM + lz], __float2int_rn(wz * v.x));
-        atomicAdd(&plane[1 * kM + lz], __float2int_rn(wz * v.y));
-        atomicAdd(&plane[kW * kM + lw], __float2int_rn(ww * v.z));
-        atomicAdd(&plane[(kW + 1) * kM + lw], __float2int_rn(ww * v.w));
-        if (GLS) {
-          const float4 q = st[2];
-          atomicAdd(&plane[2 * kM + lz], __float2int_rn(wz * q.x));
-          atomicAdd(&plane[3 * kM + lz], __float2int_rn(wz * q.y));
-        }
-      }
-      __syncthreads();
+      sc = tf_scale_block<kWarps>(count, ymax, wmax, s_max);  // its barriers end the use of the counts
     }
+    const float y_sc = sc.y, w_sc = sc.w, c_sc = sc.c;
+
+    // ---- spread: each warp takes an eighth of the observations, 32 at a
+    // time: a lane each for the phase, then an octet of lanes each for the 8
+    // cells
+    {
+      const int j1 = (int)((int64_t)n * (warp + 1) / kWarps);
+      unsigned char* const mine = stage + (size_t)warp * 32 * S::kStage;
+      for (int jb = (int)((int64_t)n * warp / kWarps); jb < j1; jb += 32) {
+        const int j = jb + lane;
+        if (j < j1) {
+          const uint4 r0 = __ldg(rec + 2 * j), r1 = __ldg(rec + 2 * j + 1);
+          const uint32_t ph = phase_hi32(r0.w, r1.x, r1.y, kc);
+          float s, c;
+          sincospif(__int2float_rn((int)ph) * 4.656612873077393e-10f, &s, &c);  // 2^-31 half-cycles
+          const float ys = __uint_as_float(r0.x) * y_sc;
+          const float ws = GLS ? __uint_as_float(r1.w) * w_sc : w_sc;
+          // position in cells, 12 bits of cell and 32 of fraction
+          const uint32_t fz = (r1.x << 12) | (r1.y >> 20), b2 = (r1.x << 1) | (r1.y >> 31), lo2 = r1.y << 1;
+          const uint32_t fw = (b2 << 12) | (lo2 >> 20);
+          const float uz = fmaf(__uint2float_rn(fz), 2.3283064365386963e-10f, -0.5f);
+          const float uw = fmaf(__uint2float_rn(fw), 2.3283064365386963e-10f, -0.5f);
+          float4* st = reinterpret_cast<float4*>(mine + (size_t)lane * S::kStage);
+          st[0] = make_float4(uz, uw, __uint_as_float((r1.x >> 20) - 3u), __uint_as_float((b2 >> 20) - 3u));
+          st[1] = make_float4(ys * c, ys * s, ws * (c - s) * (c + s), ws * 2.0f * c * s);
+          if (GLS) {
+            const float cs = __uint_as_float(r1.w) * c_sc;
+            st[2] = make_float4(cs * c, cs * s, 0.0f, 0.0f);
+          }
+        }
+        __syncwarp();
+        const int nt = min(32, j1 - jb);
+#pragma unroll 2
+        for (int i = lane >> 3; i < nt; i += 4) {
+          const float4* st = reinterpret_cast<const float4*>(mine + (size_t)i * S::kStage);
+          const float4 at = st[0], v = st[1];
+          const f2_t u = f2_pack(at.x, at.y);
+          f2_t w2 = poly[8];
+#pragma unroll
+          for (int d = 7; d >= 0; --d) w2 = f2_fma(w2, u, poly[d]);
+          float wz, ww;
+          f2_unpack(w2, wz, ww);
+          const int lz = (int)(__float_as_uint(at.z) + (uint32_t)(lane & 7)) & (kM - 1);
+          const int lw = (int)(__float_as_uint(at.w) + (uint32_t)(lane & 7)) & (kM - 1);
+          atomicAdd(&plane[0 * kM + lz], __float2int_rn(wz * v.x));
+          atomicAdd(&plane[1 * kM + lz], __float2int_rn(wz * v.y));
+          atomicAdd(&plane[kW * kM + lw], __float2int_rn(ww * v.z));
+          atomicAdd(&plane[(kW + 1) * kM + lw], __float2int_rn(ww * v.w));
+          if (GLS) {
+            const float4 q = st[2];
+            atomicAdd(&plane[2 * kM + lz], __float2int_rn(wz * q.x));
+            atomicAdd(&plane[3 * kM + lz], __float2int_rn(wz * q.y));
+          }
+        }
+        __syncwarp();
+      }
+    }
+    __syncthreads();
 
     // ---- transform, power
     float* const pw = reinterpret_cast<float*>(stage);
@@ -379,8 +358,8 @@ __global__ void __launch_bounds__(kThreads, 2) transform_kernel(TransformParams 
       const float nf = (float)oi.n;
 #pragma unroll
       for (int s = 0; s < 8; ++s) {
-        const int i = tid + 256 * s;
-        const float dc = __ldg(&kTfDeconv[i]);
+        const int i = (tid >> 4) + 17 * (tid & 15) + 272 * s;  // bin p + 16 r + 256 s, padded
+        const float dc = __ldg(&kTfDeconv[256 * s + tid]);
         const f2_t f = f2_mul(inv, f2_pack(dc, dc));
         float zr, wr, zi, wi;
         f2_unpack(f2_mul(out[s].re, f), zr, wr);
@@ -416,8 +395,8 @@ __global__ void __launch_bounds__(kThreads, 2) transform_kernel(TransformParams 
       const float inv_w = 1.0f / w_sc, wsum = oi.wsum_f, yy = (float)oi.sum_y2;
 #pragma unroll
       for (int s = 0; s < 8; ++s) {
-        const int i = tid + 256 * s;
-        const float dc = __ldg(&kTfDeconv[i]);
+        const int i = (tid >> 4) + 17 * (tid & 15) + 272 * s;  // bin p + 16 r + 256 s, padded
+        const float dc = __ldg(&kTfDeconv[256 * s + tid]);
         const f2_t f = f2_mul(inv, f2_pack(dc, dc));
         float yr, cr, yi, ci;
         f2_unpack(f2_mul(out[s].re, f), yr, cr);
@@ -433,11 +412,9 @@ __global__ void __launch_bounds__(kThreads, 2) transform_kernel(TransformParams 
 
     // ---- eight consecutive bins per thread from here on
     float pv[8];
-    {
-      const float4 a = reinterpret_cast<const float4*>(pw)[2 * tid], b = reinterpret_cast<const float4*>(pw)[2 * tid + 1];
-      pv[0] = a.x; pv[1] = a.y; pv[2] = a.z; pv[3] = a.w;
-      pv[4] = b.x; pv[5] = b.y; pv[6] = b.z; pv[7] = b.w;
-    }
+#pragma unroll
+    for (int m = 0; m < 8; ++m) pv[m] = pw[8 * tid + (tid >> 1) + m];
+    clear_grid();  // for the next item: every thread is past the transform
     const uint32_t k0 = (uint32_t)kc0 + 8u * (uint32_t)tid;
     uint32_t bad = 0u;
 #pragma unroll

@@ -139,7 +139,9 @@ lsp_status lsp_workspace_size(int64_t n_obj, int64_t total_nt, const lsp_grid* g
  * paper's "return the periodogram or not" option; leaving it NULL keeps the
  * periodogram out of HBM entirely.  peaks (nullable) receives opts->top_k
  * lsp_peak entries.  workspace must hold lsp_workspace_size(1, n_t, ...)
- * bytes and be 256-byte aligned; the call may use all of it.
+ * bytes and be 256-byte aligned; the call may use all of it.  (Less is
+ * enough where a path with less scratch runs: what lsp_workspace_size gives
+ * for options that name a direct kernel always is.)
  */
 lsp_status lsp_periodogram(const double* t, const void* y, int64_t n_t, const lsp_grid* grid,
                            const lsp_opts* opts, void* power_out, lsp_peak* peaks,
@@ -169,7 +171,7 @@ lsp_status lsp_batch(const double* t, const void* y, const int64_t* offsets, int
  * counterpart: this is a deployment convenience of this library.
  * Arguments and results are those of lsp_batch; the scratch memory is a
  * fixed device array of LSP_NOALLOC_SCRATCH_BYTES inside the library.  A
- * shape whose lsp_workspace_size exceeds it returns LSP_E_WORKSPACE,
+ * shape that no path of lsp_batch runs within it returns LSP_E_WORKSPACE,
  * launching nothing; an empty batch returns LSP_OK at once.  The call
  * allocates nothing itself.  The CUDA runtime reserves the array in a
  * device's memory when it loads the library's module there -- with lazy
@@ -245,10 +247,10 @@ typedef struct lsp_plan lsp_plan;
  * The ablation kernels (trig or staging non-zero) are FP32, scalar
  * (packed 0), k_reseed = freqs_per_thread = 16, standard periodogram only;
  * other combinations return LSP_E_UNSUPPORTED.
- * reserved = 1: FP32 objects with enough observations get their trig sums
- * from a nonuniform FFT per run of 2048 bins instead of pair by pair (the
- * same sums; its error is below the pairwise kernel's), and the kernel the
- * other fields name serves the rest.  It is the choice of every call whose
+ * reserved = 1: objects with enough observations (FP32 40, FP64 8) get their
+ * trig sums from a nonuniform FFT, per run of 2048 bins or, one object, of
+ * its whole grid, instead of pair by pair (the same sums, no less exact), and
+ * the kernel the other fields name serves the rest.  It is the choice of every call whose
  * lsp_opts leave the kernel options 0, and of a plan until lsp_plan_set_config
  * says otherwise.  It needs block_threads x freqs_per_thread = 2048 (a single
  * object: any) and no ablation; other configurations read it as 0.

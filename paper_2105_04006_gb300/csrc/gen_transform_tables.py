@@ -17,6 +17,7 @@ kernels) and 4.8e-15 and 1.1e-15 (w = 16, FP64) for |xi| <= 1/4, beta being
 the minimiser of the former.
 """
 import math
+import struct
 import sys
 
 
@@ -63,6 +64,51 @@ def window_polys(w, beta, deg):
     return rows
 
 
+def window_sub_polys(w, beta, deg, n_sub):
+    """[s][r][d]: monomial coefficients in v of psi(r - (w/2 - 1) - (s + 1/2 + v) / n_sub), |v| <= 1/2."""
+    n = 12
+    th = [math.pi * (k + 0.5) / n for k in range(n)]
+    cosj = [[math.cos(j * a) for a in th] for j in range(deg + 1)]
+    # Chebyshev polynomials in monomials of x = 2v
+    mono = [[1.0], [0.0, 1.0]]
+    while len(mono) <= deg:
+        nxt = [0.0] + [2.0 * v for v in mono[-1]]
+        for d, v in enumerate(mono[-2]):
+            nxt[d] -= v
+        mono.append(nxt)
+    out = []
+    for s in range(n_sub):
+        rows = []
+        for r in range(w):
+            f = [psi(r - (w // 2 - 1) - (s + 0.5 + 0.5 * c) / n_sub, w, beta) for c in cosj[1]]
+            cheb = [(2.0 if j else 1.0) / n * math.fsum(v * c for v, c in zip(f, cosj[j])) for j in range(deg + 1)]
+            rows.append([math.fsum(cheb[j] * mono[j][d] for j in range(deg + 1) if d < len(mono[j])) * 2.0 ** d
+                         for d in range(deg + 1)])
+        out.append(rows)
+    return out
+
+
+def deconv_poly(w, beta, deg):
+    """Monomial coefficients in z = (4 xi)^2, 0 <= z <= 1, of 1 / psi^(xi)."""
+    n = 64
+    th = [math.pi * (k + 0.5) / n for k in range(n)]
+    f = [1.0 / psi_hat(0.25 * math.sqrt(0.5 * math.cos(a) + 0.5), w, beta) for a in th]
+    cheb = [(2.0 if j else 1.0) / n * math.fsum(v * math.cos(j * a) for v, a in zip(f, th)) for j in range(deg + 1)]
+    # T_j(2z - 1) in powers of z
+    t0, t1, c = [1.0], [-1.0, 2.0], [0.0] * (deg + 1)
+    for j in range(deg + 1):
+        for d, v in enumerate(t0):
+            c[d] += cheb[j] * v
+        t2 = [0.0] * (len(t1) + 1)
+        for d, v in enumerate(t1):
+            t2[d] -= 2.0 * v
+            t2[d + 1] += 4.0 * v
+        for d, v in enumerate(t0):
+            t2[d] -= v
+        t0, t1 = t1, t2
+    return c
+
+
 def emit(out, decl, values, fmt, per_line=8):
     out.write("%s = {\n" % decl)
     for i in range(0, len(values), per_line):
@@ -80,13 +126,38 @@ def f64(v):
     return s if any(c in s for c in ".en") else s + ".0"
 
 
+def single(v):
+    return struct.unpack("f", struct.pack("f", v))[0]
+
+
+def two(v):
+    """A double as a two-float pair (48 of its bits)."""
+    h = single(v)
+    return "%s, %s" % (f32(h), f32(single(v - h)))
+
+
+def dd(v):
+    return "{%s}" % two(v)
+
+
+def dd2(v):
+    return "{%s, %s}" % (two(v[0]), two(v[1]))
+
+
 def c32(v):
     return "{%s, %s}" % (f32(v[0]), f32(v[1]))
 
 
 def unit(num, den):
-    a = 2.0 * math.pi * num / den
-    return math.cos(a), math.sin(a)
+    """(cos, sin) of 2 pi num / den, the angle reduced to the first octant first."""
+    num %= den
+    q, r = divmod(8 * num, den)  # octant and remainder / den
+    s = r if q % 2 == 0 else den - r
+    a = 2.0 * math.pi * s / (8 * den)
+    c, v = math.cos(a), math.sin(a)
+    if q in (1, 2, 5, 6):
+        c, v = v, c
+    return (-c if q in (2, 3, 4, 5) else c), (-v if q >= 4 else v)
 
 
 def main(path):
@@ -94,9 +165,12 @@ def main(path):
     with open(path, "w") as out:
         out.write("// written by gen_transform_tables.py\n")
         polys = window_polys(w, beta, deg)
+        out.write("#if defined(LSP_TF_TABLES_F32) || defined(LSP_TF_TABLES_LONG)\n")
         # kTfPoly[d][r]: coefficient of u^d for the cell r - 3 cells from the observation's own
         emit(out, "__device__ const float kTfPoly[%d * %d]" % (deg + 1, w),
              [polys[r][d] for d in range(deg + 1) for r in range(w)], f32)
+        out.write("#endif\n")
+        out.write("#ifdef LSP_TF_TABLES_F32\n")
         # kTfDeconv[256 s + t]: 1 / psi^ at the offset of thread t's s-th output, t/16 + 16 (t%16) + 256 s - m/4
         emit(out, "__device__ const float kTfDeconv[%d]" % (m // 2),
              [1.0 / psi_hat((t // 16 + 16 * (t % 16) + 256 * s - m // 4) / m, w, beta)
@@ -106,6 +180,32 @@ def main(path):
              [unit(p * b, 4096) for p in range(1, 16) for b in range(256)], c32, 4)
         emit(out, "__device__ const float2 kTfTw2[15 * 16]",
              [unit(r * d, 256) for r in range(1, 16) for d in range(16)], c32, 4)
+        out.write("#endif\n")
+        # one long object: e^{2 pi i n / 4096}, e^{2 pi i n / 2^24}, and 1 / psi^ as a polynomial in (4 xi)^2
+        out.write("#ifdef LSP_TF_TABLES_LONG\n")
+        emit(out, "__device__ const float2 kUnit[4096]", [unit(k, 4096) for k in range(4096)], c32, 4)
+        emit(out, "__device__ const float2 kFine[4096]", [unit(k, 1 << 24) for k in range(4096)], c32, 4)
+        emit(out, "__device__ const float4 kUnitD[4096]", [unit(k, 4096) for k in range(4096)], dd2, 2)
+        emit(out, "__device__ const float4 kFineD[4096]", [unit(k, 1 << 24) for k in range(4096)], dd2, 2)
+        emit(out, "__device__ const float kDeconvPoly[9]", deconv_poly(w, beta, 8), f32)
+        emit(out, "__device__ const float2 kDeconvPolyD[17]", deconv_poly(16, 0.741 * 16 * math.pi, 16), dd, 4)
+        out.write("#endif\n")
+        out.write("#ifdef LSP_TF_TABLES_F64\n")
+        w, beta, deg, n_sub = 16, 0.741 * 16 * math.pi, 5, 64
+        polys = window_sub_polys(w, beta, deg, n_sub)
+        # kTfPolyD[(6 sub + d) 16 + r]: coefficient of v^d, sub-interval sub of a cell, cell r - 7
+        out.write("#endif\n#if defined(LSP_TF_TABLES_F64) || defined(LSP_TF_TABLES_LONG)\n")
+        emit(out, "__device__ const float2 kTfPolyD[%d]" % (n_sub * (deg + 1) * w),
+             [polys[s][r][d] for s in range(n_sub) for d in range(deg + 1) for r in range(w)], dd, 4)
+        out.write("#endif\n#ifdef LSP_TF_TABLES_F64\n")
+        emit(out, "__device__ const float2 kTfDeconvD[%d]" % (m // 2),
+             [1.0 / psi_hat((t // 16 + 16 * (t % 16) + 256 * s - m // 4) / m, w, beta)
+              for s in range(8) for t in range(256)], dd, 4)
+        emit(out, "__device__ const float4 kTfTwD1[15 * 256]",
+             [unit(p * b, 4096) for p in range(1, 16) for b in range(256)], dd2, 2)
+        emit(out, "__device__ const float4 kTfTwD2[15 * 16]",
+             [unit(r * d, 256) for r in range(1, 16) for d in range(16)], dd2, 2)
+        out.write("#endif\n")
 
 
 if __name__ == "__main__":

@@ -75,7 +75,10 @@ struct Layout {
   int32_t n_chunks, n_res_chunks;
   int64_t n_items;
   int grid;  // persistent CTAs
-  size_t off_obj, off_rec, off_order, off_hist, off_queue, off_best, off_cand, off_part, off_stats, total;
+  int lng = 0;      // one object by one transform of its whole grid (lsp_long.cu)
+  LongPlan lp;
+  size_t off_obj, off_rec, off_order, off_hist, off_queue, off_best, off_cand, off_part, off_stats, off_cells, off_t,
+      off_row, total;
 };
 
 constexpr int64_t kMaxNf = (int64_t)1 << 31;  // k0 + F must fit in 32 bits
@@ -89,6 +92,21 @@ constexpr int kGateObjects = 8;  // objects the autotuner's error gate checks
 // proportional to it.  Measured (2000 objects of equal N_t, N_f = 1e5,
 // transform | direct, ms): N_t 32 2.2 | 1.9, 48 2.2 | 2.6, 100 2.4 | 5.0.
 constexpr int kTfMinObs = 40;
+constexpr int kTfMinObs64 = 8;
+// One FP32 object goes run by run or by one transform of its whole grid,
+// whichever a model of their times (us, GB300, fitted to N_t 1e3 .. 1e5, N_f
+// 3e3 .. 1e6) puts first: a run costs 12 + N_t / 150 per wave of CTAs, the
+// whole grid 30 + N_f / 12500.  Measured, runs | whole grid: N_t 3000, N_f 1e5
+// 41 | 43; N_t 1e4, N_f 1e5 78 | 43; N_t 3000, N_f 4e5 49 | 65; N_t 1e5, N_f 1e6
+// 1480 | 127.  In FP64 the whole grid is always the faster (N_t 1000, N_f 1e5:
+// 208 | 88; the direct kernel takes 1400).
+bool long_is_faster(int64_t n_t, int64_t n_f, int64_t runs, int64_t slots) {
+  const double waves = (double)((runs + slots - 1) / slots);
+  return waves * (12.0 + (double)n_t / 150.0) > 30.0 + (double)n_f / 12500.0;
+}
+// The paths a call may take, by the workspace they need: everything; without
+// the whole-grid transform; the direct kernels alone.
+constexpr int kLevels = 3;
 
 lsp_status check_grid(const lsp_grid* g) {
   if (!g) return fail(LSP_E_ARG, "grid is NULL");
@@ -101,7 +119,7 @@ lsp_status check_grid(const lsp_grid* g) {
 }
 
 lsp_status resolve(int64_t n_obj, int64_t total_nt, const lsp_grid* g, const lsp_opts* opts_in,
-                   const lsp_config* cfg, Layout* L, bool gls = false) {
+                   const lsp_config* cfg, Layout* L, bool gls = false, int level = 0) {
   lsp_status st = check_grid(g);
   if (st) return st;
   if (n_obj < 0 || n_obj > INT32_MAX) return fail(LSP_E_ARG, "n_obj out of range");
@@ -131,7 +149,8 @@ lsp_status resolve(int64_t n_obj, int64_t total_nt, const lsp_grid* g, const lsp
   int k, fpt, threads, packed, split_req, abl = 0;
   // the transform is the library's own choice: a call that names a kernel
   // option gets the direct kernel it names
-  bool tf = l.prec == LSP_FP32;
+  bool tf = l.prec == LSP_FP32 || !gls;
+  const int tf_min = l.prec == LSP_FP32 ? kTfMinObs : kTfMinObs64;
   if (cfg) tf = tf && cfg->reserved == 1;
   else tf = tf && !o.k_reseed && !o.freqs_per_thread && !o.block_threads && !o.obs_split;
   if (cfg) {
@@ -191,16 +210,18 @@ lsp_status resolve(int64_t n_obj, int64_t total_nt, const lsp_grid* g, const lsp
     }
     if (split > kMaxSplit) split = kMaxSplit;
   }
-  tf = tf && !abl && n_obj > 0 && (n_obj == 1 ? total_nt >= kTfMinObs : chunk == kTfBins);
+  tf = tf && level < 2 && !abl && n_obj > 0 && (n_obj == 1 ? total_nt >= tf_min : chunk == kTfBins);
   const int64_t tf_chunks = (l.n_f + kTfBins - 1) / kTfBins;
   tf = tf && n_obj * tf_chunks < ((int64_t)1 << 31);  // 32-bit item numbers
   l.tf = tf;
-  l.tf_min = kTfMinObs;
+  l.tf_min = tf_min;
   l.split = split;
   if (tf && n_obj == 1) {  // no direct kernel, no observation split
     l.n_chunks = (int32_t)tf_chunks;
     l.split = 1;
     l.cfg_split = split;
+    l.lng = level < 1 && !gls && (l.prec || long_is_faster(total_nt, l.n_f, tf_chunks, 2 * (int64_t)current_sm_count())) &&
+            long_plan(l.prec, l.n_f, &l.lp);
   }
   split = l.split;
   const int64_t cchunk = (int64_t)kCombineThreads * kCombinePerThread;
@@ -223,6 +244,9 @@ lsp_status resolve(int64_t n_obj, int64_t total_nt, const lsp_grid* g, const lsp
   // partial sums: 4 per frequency, the generalized periodogram's 6 in slots of 8
   l.off_part = take(split > 1 ? (size_t)split * l.n_f * (gls ? 8 : 4) * (l.prec ? 8 : 4) : 0);
   l.off_stats = take(n_obj == 1 ? stats_slices_bytes(total_nt) : 0);
+  l.off_cells = take(l.lng ? l.lp.cell_bytes : 0);
+  l.off_t = take(l.lng ? l.lp.t_bytes : 0);
+  l.off_row = take(l.lng ? l.lp.row_bytes : 0);
   l.total = off;
 
   int bps = main_blocks_per_sm(l.prec, l.packed, l.k, l.fpt, l.threads, l.top, l.gls, l.abl);
@@ -234,7 +258,7 @@ lsp_status resolve(int64_t n_obj, int64_t total_nt, const lsp_grid* g, const lsp
   if (grid > l.n_items) grid = l.n_items;
   l.grid = (int)(grid < 1 ? 1 : grid);
   if (l.tf) {
-    int tb = transform_blocks_per_sm(l.gls);
+    int tb = transform_blocks_per_sm(l.prec, l.gls);
     if (tb <= 0) {
       cudaGetLastError();
       tb = 1;
@@ -290,25 +314,50 @@ lsp_status run(const Layout& L, const double* t, const void* y, const int64_t* o
     LSP_CUDA(launch_lpt_order(obj, L.n_obj, hist, order, st), "work-queue order");
   const bool tf_peak = L.tf && !order && !L.top && peaks;  // the transform kernel writes the peak
   if (L.tf) {
-    TransformParams tp;
-    tp.rec = (const RecF32*)rec;
-    tp.obj = obj;
-    tp.order_back = order ? order + (L.n_obj - 1) : nullptr;
-    tp.power_out = (float*)power_out;
-    tp.best = best;
-    tp.cand = cand;
-    tp.queue = queue + 3;
-    tp.n_items_dev = order ? queue + 4 : nullptr;
-    tp.n_items = (uint32_t)L.n_items;
-    tp.n_chunks = L.n_chunks;
-    tp.have_scale = L.n_obj > 1;
-    tp.n_f = L.n_f;
-    tp.peaks = tf_peak ? peaks : nullptr;
-    tp.f_min = L.f_min;
-    tp.df = L.df;
-    tp.ticket = queue + 2;
+    auto fill = [&](auto& tp) {
+      tp.order_back = order ? order + (L.n_obj - 1) : nullptr;
+      tp.obj = obj;
+      tp.best = best;
+      tp.cand = cand;
+      tp.queue = queue + 3;
+      tp.n_items_dev = order ? queue + 4 : nullptr;
+      tp.n_items = (uint32_t)L.n_items;
+      tp.n_chunks = L.n_chunks;
+      tp.have_scale = L.n_obj > 1;
+      tp.n_f = L.n_f;
+      tp.peaks = tf_peak ? peaks : nullptr;
+      tp.f_min = L.f_min;
+      tp.df = L.df;
+      tp.ticket = queue + 2;
+    };
     if (ev_main0) LSP_CUDA(cudaEventRecordWithFlags(ev_main0, st, cudaEventRecordExternal), "timing event");
-    LSP_CUDA(launch_transform(tp, L.gls, L.tf_grid, st), "transform kernel");
+    if (L.lng && L.prec == LSP_FP64) {
+      TransformParams64 tp;
+      fill(tp);
+      tp.rec = (const RecF64*)rec;
+      tp.power_out = (double*)power_out;
+      LSP_CUDA(launch_long64(L.lp, tp, L.total_nt, ws + L.off_cells, ws + L.off_t, ws + L.off_row, st),
+               "whole-grid transform");
+    } else if (L.lng) {
+      TransformParams tp;
+      fill(tp);
+      tp.rec = (const RecF32*)rec;
+      tp.power_out = (float*)power_out;
+      LSP_CUDA(launch_long32(L.lp, tp, L.total_nt, ws + L.off_cells, ws + L.off_t, ws + L.off_row, st),
+               "whole-grid transform");
+    } else if (L.prec == LSP_FP64) {
+      TransformParams64 tp;
+      fill(tp);
+      tp.rec = (const RecF64*)rec;
+      tp.power_out = (double*)power_out;
+      LSP_CUDA(launch_transform64(tp, L.tf_grid, st), "transform kernel");
+    } else {
+      TransformParams tp;
+      fill(tp);
+      tp.rec = (const RecF32*)rec;
+      tp.power_out = (float*)power_out;
+      LSP_CUDA(launch_transform(tp, L.gls, L.tf_grid, st), "transform kernel");
+    }
     if (!order) {
       if (ev_main1) LSP_CUDA(cudaEventRecordWithFlags(ev_main1, st, cudaEventRecordExternal), "timing event");
       if (peaks && !tf_peak)
@@ -364,6 +413,19 @@ lsp_status check_ws(const Layout& L, void* ws, size_t ws_bytes) {
   return LSP_OK;
 }
 
+// The layout of a one-shot call: the first level whose scratch fits the
+// caller's workspace (a workspace sized for the direct kernels stays enough).
+lsp_status resolve_for(int64_t n_obj, int64_t total_nt, const lsp_grid* g, const lsp_opts* opts, bool gls, size_t ws_bytes,
+                       Layout* L) {
+  lsp_status st = resolve(n_obj, total_nt, g, opts, nullptr, L, gls);
+  for (int level = 1; !st && L->total > ws_bytes && level < kLevels; ++level) {
+    Layout M;
+    if (resolve(n_obj, total_nt, g, opts, nullptr, &M, gls, level)) break;
+    if (M.total <= ws_bytes) *L = M;
+  }
+  return st;
+}
+
 lsp_status check_io(int64_t n, const double* t, const void* y) {
   if (n > 0 && (!t || !y)) return fail(LSP_E_ARG, "t and y must not be NULL");
   return LSP_OK;
@@ -374,6 +436,16 @@ lsp_status check_io(int64_t n, const double* t, const void* y) {
 namespace lsp {
 // Lets other translation units of the library report through lsp_last_error.
 void set_last_error(const char* msg) { g_err = msg ? msg : ""; }
+// The least workspace with which lsp_batch runs this shape.
+lsp_status least_workspace(int64_t n_obj, int64_t total_nt, const lsp_grid* grid, const lsp_opts* opts, size_t* bytes) {
+  for (int level = 0; level < kLevels; ++level) {
+    Layout L;
+    lsp_status st = resolve(n_obj, total_nt, grid, opts, nullptr, &L, false, level);
+    if (st) return st;
+    if (level == 0 || L.total < *bytes) *bytes = L.total;
+  }
+  return LSP_OK;
+}
 }  // namespace lsp
 
 // ======================================================================= C ABI
@@ -436,7 +508,7 @@ lsp_status lsp_periodogram(const double* t, const void* y, int64_t n_t, const ls
                            size_t ws_bytes, lsp_stream_t stream) {
   g_err.clear();
   Layout L;
-  lsp_status st = resolve(1, n_t, grid, opts, nullptr, &L);
+  lsp_status st = resolve_for(1, n_t, grid, opts, false, ws_bytes, &L);
   if (st) return st;
   if ((st = check_io(n_t, t, y))) return st;
   if ((st = check_ws(L, workspace, ws_bytes))) return st;
@@ -448,7 +520,7 @@ lsp_status lsp_batch(const double* t, const void* y, const int64_t* offsets, int
                      lsp_peak* peaks, void* workspace, size_t ws_bytes, lsp_stream_t stream) {
   g_err.clear();
   Layout L;
-  lsp_status st = resolve(n_obj, total_nt, grid, opts, nullptr, &L);
+  lsp_status st = resolve_for(n_obj, total_nt, grid, opts, false, ws_bytes, &L);
   if (st) return st;
   if (n_obj == 0) return LSP_OK;
   if (!offsets) return fail(LSP_E_ARG, "offsets must not be NULL");
@@ -473,7 +545,7 @@ lsp_status lsp_batch_gls(const double* t, const void* y, const void* dy, const i
                          lsp_stream_t stream) {
   g_err.clear();
   Layout L;
-  lsp_status st = resolve(n_obj, total_nt, grid, opts, nullptr, &L, true);
+  lsp_status st = resolve_for(n_obj, total_nt, grid, opts, true, ws_bytes, &L);
   if (st) return st;
   if (n_obj == 0) return LSP_OK;
   if (!offsets) return fail(LSP_E_ARG, "offsets must not be NULL");
@@ -487,7 +559,7 @@ lsp_status lsp_periodogram_gls(const double* t, const void* y, const void* dy, i
                                lsp_peak* peaks, void* workspace, size_t ws_bytes, lsp_stream_t stream) {
   g_err.clear();
   Layout L;
-  lsp_status st = resolve(1, n_t, grid, opts, nullptr, &L, true);
+  lsp_status st = resolve_for(1, n_t, grid, opts, true, ws_bytes, &L);
   if (st) return st;
   if ((st = check_io(n_t, t, y))) return st;
   if ((st = check_ws(L, workspace, ws_bytes))) return st;
@@ -521,6 +593,7 @@ struct lsp_plan {
   lsp_opts opts;
   lsp_config cfg;
   int64_t n_obj = 0, total_nt = 0;
+  int level = 0;  // paths its workspace has room for (kLevels)
   int device = 0;
   char* ws = nullptr;
   size_t ws_cap = 0;
@@ -595,7 +668,7 @@ lsp_status ensure_ws(lsp_plan* p, size_t bytes) {
 
 lsp_status apply_config(lsp_plan* p, const lsp_config* c) {
   Layout L;
-  lsp_status st = resolve(p->n_obj, p->total_nt, &p->grid, &p->opts, c, &L);
+  lsp_status st = resolve(p->n_obj, p->total_nt, &p->grid, &p->opts, c, &L, false, p->level);
   if (st) return st;
   if ((st = ensure_ws(p, L.total))) return st;
   p->L = L;
@@ -743,7 +816,8 @@ lsp_status execute_host_parts(lsp_plan* p, int parts, const double* t, const voi
   for (int j = 0; j < parts; ++j) {
     const int64_t a = first[(size_t)j], b = first[(size_t)j + 1];
     for (int64_t i = a; i <= b; ++i) p->h_rel[(size_t)(i + j)] = offsets[i] - offsets[a];
-    lsp_status st = resolve(b - a, offsets[b] - offsets[a], &p->grid, &p->opts, &p->cfg, &G[(size_t)j]);
+    lsp_status st = resolve(b - a, offsets[b] - offsets[a], &p->grid, &p->opts, &p->cfg, &G[(size_t)j],
+                            false, p->level);
     if (st) return st;
     if (G[(size_t)j].total > ws_need) ws_need = G[(size_t)j].total;
   }
@@ -837,10 +911,16 @@ lsp_status lsp_plan_create(lsp_plan** plan, int64_t n_obj, int64_t total_nt, con
   p->n_obj = n_obj;
   p->total_nt = total_nt;
   cudaGetDevice(&p->device);
-  if ((st = ensure_ws(p, L.total))) {
+  // without room for the larger paths' scratch the plan takes a smaller one
+  while ((st = ensure_ws(p, L.total)) && ++p->level < kLevels)
+    if (resolve(n_obj, total_nt, grid, opts, nullptr, &L, false, p->level)) break;
+  if (st) {
     delete p;
     return st;
   }
+  g_err.clear();
+  p->L = L;
+  p->cfg = config_of(L);
   if (cudaStreamCreateWithFlags(&p->cap_stream, cudaStreamNonBlocking) != cudaSuccess) {
     cudaGetLastError();
     lsp_plan_destroy(p);
@@ -904,7 +984,7 @@ lsp_status lsp_plan_kernel_count(const lsp_plan* p, int32_t* count) {
   // requested; plans of one object run without offsets
   const bool one_prologue = L.n_obj == 1 && L.total_nt <= kFusedMaxNt;
   if (L.tf && L.n_obj == 1) {  // prologue + transform (+ finalize for the top-k)
-    *count = (one_prologue ? 1 : 2) + 1 + (L.top ? 1 : 0);
+    *count = (one_prologue ? 1 : 2) + (L.lng ? 4 : 1) + (L.top ? 1 : 0);
     return LSP_OK;
   }
   const bool fused = L.split > 1 && !L.top;
@@ -1144,7 +1224,7 @@ lsp_status lsp_plan_autotune_ex(lsp_plan* p, const double* t, const void* y, con
   // for the objects it leaves (so it comes after that candidate itself).
   {
     Layout Ld;
-    if ((st = resolve(p->n_obj, p->total_nt, &p->grid, &p->opts, nullptr, &Ld))) return st;
+    if ((st = resolve(p->n_obj, p->total_nt, &p->grid, &p->opts, nullptr, &Ld, false, p->level))) return st;
     if (Ld.tf) cands.push_back(config_of(Ld));
   }
 

@@ -393,6 +393,26 @@ __device__ __forceinline__ void fix_ill_conditioned_gls(float (&pv)[F], uint32_t
   }
 }
 
+// exact_power_warp on FP64 records.
+static __device__ __noinline__ double exact_power_warp64(const RecF64* __restrict__ rec, int64_t begin, int n,
+                                                         uint32_t k, double norm_scale) {
+  double xc = 0.0, xs = 0.0, cc = 0.0, cs = 0.0;
+  for (int j = threadIdx.x & 31; j < n; j += 32) {
+    const RecF64 r = rec[begin + j];
+    double c, s;
+    seed_sincos_f64(r.a + (uint64_t)k * r.b, c, s);
+    xc = fma(r.y, c, xc);
+    xs = fma(r.y, s, xs);
+    cc = fma(c, c, cc);
+    cs = fma(c, s, cs);
+  }
+  xc = warp_sum_d(xc);
+  xs = warp_sum_d(xs);
+  cc = warp_sum_d(cc);
+  cs = warp_sum_d(cs);
+  return norm_scale * lsp_power<double>(xc, xs, cc, cs, (double)n, EpsRel<double>::v);
+}
+
 // Replace the ill-conditioned bins (bit m of `bad`: bin k0 + m) of every lane
 // of the warp by their FP64 re-evaluation.  Called by all 32 lanes.
 template <int F>

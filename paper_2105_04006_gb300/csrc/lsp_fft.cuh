@@ -1,0 +1,241 @@
+// lsp_fft.cuh -- the 4096-point transform of the transform kernels (internal).
+//
+// One CTA of 256 threads, 16 points per thread, 4096 = 16^3: three register
+// passes with two exchanges through shared memory, e^{+2 pi i jk / 4096},
+// outputs only for the half of the frequencies inside a run of bins.  The
+// element type T is f2_t (two FP32 transforms side by side in packed f32x2
+// halves, sharing every twiddle), float, or dd (two-float numbers of about 48
+// bits, the FP64 path).
+#pragma once
+
+#include <cstring>
+#include <type_traits>
+
+#include "lsp_common.cuh"
+
+namespace lsp {
+
+// ------------------------------------------------------------ arithmetic on
+// f32x2 pairs (two transforms at once) or single floats
+__device__ __forceinline__ f2_t add_(f2_t a, f2_t b) {
+  f2_t d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ f2_t sub_(f2_t a, f2_t b) { return f2_fma(b, 0xbf800000bf800000ull, a); }
+__device__ __forceinline__ float add_(float a, float b) { return a + b; }
+__device__ __forceinline__ float sub_(float a, float b) { return a - b; }
+__device__ __forceinline__ f2_t mul_(f2_t a, f2_t b) { return f2_mul(a, b); }
+__device__ __forceinline__ float mul_(float a, float b) { return a * b; }
+__device__ __forceinline__ f2_t fma_(f2_t a, f2_t b, f2_t c) { return f2_fma(a, b, c); }
+__device__ __forceinline__ float fma_(float a, float b, float c) { return fmaf(a, b, c); }
+template <typename T> __device__ __forceinline__ T dup_(float v);
+template <> __device__ __forceinline__ f2_t dup_<f2_t>(float v) { return f2_pack(v, v); }
+template <> __device__ __forceinline__ float dup_<float>(float v) { return v; }
+__device__ __forceinline__ f2_t neg1_(f2_t a) { return mul_(a, 0xbf800000bf800000ull); }
+__device__ __forceinline__ float neg1_(float a) { return -a; }
+
+// ----------------------------------------------------------- two-float numbers
+// hi + lo with |lo| <= ulp(hi)/2: Dekker's arithmetic (1971), products by FMA.
+// GB300 runs FP64 at 1/64 of the FP32 rate, so 11 FP32 operations for a sum
+// and 7 for a product are 6 to 9 times faster than one FP64 operation each.
+// The sum's error is relative to |a| + |b| (2^-47), not to the result, which
+// is what a transform needs.
+struct __align__(8) dd {
+  float hi, lo;
+};
+__device__ __forceinline__ dd dd_fast(float s, float e) {  // |s| >= |e|
+  const float h = __fadd_rn(s, e);
+  return {h, __fsub_rn(e, __fsub_rn(h, s))};
+}
+__device__ __forceinline__ dd add_(dd a, dd b) {
+  const float s = __fadd_rn(a.hi, b.hi);
+  const float t = __fsub_rn(s, a.hi);
+  float e = __fadd_rn(__fsub_rn(a.hi, __fsub_rn(s, t)), __fsub_rn(b.hi, t));
+  e = __fadd_rn(e, __fadd_rn(a.lo, b.lo));
+  return dd_fast(s, e);
+}
+__device__ __forceinline__ dd neg1_(dd a) { return {-a.hi, -a.lo}; }
+__device__ __forceinline__ dd sub_(dd a, dd b) { return add_(a, neg1_(b)); }
+__device__ __forceinline__ dd mul_(dd a, dd b) {
+  const float p = __fmul_rn(a.hi, b.hi);
+  float e = __fmaf_rn(a.hi, b.hi, -p);
+  e = __fmaf_rn(a.hi, b.lo, e);
+  e = __fmaf_rn(a.lo, b.hi, e);
+  return dd_fast(p, e);
+}
+__device__ __forceinline__ dd dd_of(double v) {
+  const float h = (float)v;
+  return {h, (float)(v - (double)h)};
+}
+__device__ __forceinline__ double dd_double(dd v) { return (double)v.hi + (double)v.lo; }
+
+// Twiddle factors (cos, sin) as a table holds them.
+template <typename T> struct Twiddle { typedef float2 type; };
+template <> struct Twiddle<dd> { typedef float4 type; };  // cos hi, lo, sin hi, lo
+template <typename T>
+__device__ __forceinline__ typename Twiddle<T>::type twiddle(double c, double s) {
+  if constexpr (sizeof(typename Twiddle<T>::type) == 8) {
+    return make_float2((float)c, (float)s);
+  } else {
+    const float ch = (float)c, sh = (float)s;
+    return make_float4(ch, (float)(c - (double)ch), sh, (float)(s - (double)sh));
+  }
+}
+
+template <typename T>
+struct Cx {
+  T re, im;
+};
+template <typename T>
+__device__ __forceinline__ Cx<T> operator+(Cx<T> a, Cx<T> b) { return {add_(a.re, b.re), add_(a.im, b.im)}; }
+template <typename T>
+__device__ __forceinline__ Cx<T> operator-(Cx<T> a, Cx<T> b) { return {sub_(a.re, b.re), sub_(a.im, b.im)}; }
+// a + i b and a - i b
+template <typename T>
+__device__ __forceinline__ Cx<T> add_i(Cx<T> a, Cx<T> b) { return {sub_(a.re, b.im), add_(a.im, b.re)}; }
+template <typename T>
+__device__ __forceinline__ Cx<T> sub_i(Cx<T> a, Cx<T> b) { return {add_(a.re, b.im), sub_(a.im, b.re)}; }
+template <typename T>
+__device__ __forceinline__ Cx<T> cmul(Cx<T> a, float2 w) {
+  const T r = dup_<T>(w.x), i = dup_<T>(w.y), ni = dup_<T>(-w.y);
+  return {fma_(a.im, ni, mul_(a.re, r)), fma_(a.re, i, mul_(a.im, r))};
+}
+__device__ __forceinline__ Cx<dd> cmul(Cx<dd> a, float4 w) {
+  const dd r{w.x, w.y}, i{w.z, w.w};
+  return {sub_(mul_(a.re, r), mul_(a.im, i)), add_(mul_(a.im, r), mul_(a.re, i))};
+}
+
+// In-place transform of 4 points with e^{+2 pi i jk/4}.
+template <typename T>
+__device__ __forceinline__ void dft4(Cx<T>& x0, Cx<T>& x1, Cx<T>& x2, Cx<T>& x3) {
+  const Cx<T> a = x0 + x2, b = x0 - x2, c = x1 + x3, d = x1 - x3;
+  x0 = a + c;
+  x1 = add_i(b, d);
+  x2 = a - c;
+  x3 = sub_i(b, d);
+}
+
+// First half of the 16-point transform: afterwards x[4 k1 + n2] holds the
+// k1-th output of the n2-th inner transform, times e^{2 pi i n2 k1 / 16}.
+template <typename T>
+__device__ __forceinline__ void dft16_first(Cx<T> (&x)[16]) {
+#pragma unroll
+  for (int n2 = 0; n2 < 4; ++n2) dft4(x[n2], x[4 + n2], x[8 + n2], x[12 + n2]);
+  constexpr double c1 = 0.92387953251128675613, s1 = 0.38268343236508977173, h = 0.70710678118654752440;
+  x[4 * 1 + 1] = cmul(x[4 * 1 + 1], twiddle<T>(c1, s1));    // W^1
+  x[4 * 2 + 1] = cmul(x[4 * 2 + 1], twiddle<T>(h, h));      // W^2
+  x[4 * 3 + 1] = cmul(x[4 * 3 + 1], twiddle<T>(s1, c1));    // W^3
+  x[4 * 1 + 2] = cmul(x[4 * 1 + 2], twiddle<T>(h, h));      // W^2
+  x[4 * 2 + 2] = Cx<T>{neg1_(x[4 * 2 + 2].im), x[4 * 2 + 2].re};  // W^4 = i
+  x[4 * 3 + 2] = cmul(x[4 * 3 + 2], twiddle<T>(-h, h));     // W^6
+  x[4 * 1 + 3] = cmul(x[4 * 1 + 3], twiddle<T>(s1, c1));    // W^3
+  x[4 * 2 + 3] = cmul(x[4 * 2 + 3], twiddle<T>(-h, h));     // W^6
+  x[4 * 3 + 3] = cmul(x[4 * 3 + 3], twiddle<T>(-c1, -s1));  // W^9
+}
+// The whole 16-point transform; output k sits at x[4 (k & 3) + (k >> 2)].
+template <typename T>
+__device__ __forceinline__ void dft16(Cx<T> (&x)[16]) {
+  dft16_first(x);
+#pragma unroll
+  for (int k1 = 0; k1 < 4; ++k1) dft4(x[4 * k1], x[4 * k1 + 1], x[4 * k1 + 2], x[4 * k1 + 3]);
+}
+
+// One complex word of the exchange buffer: 16 bytes (f2_t, dd) or 8 (float).
+template <typename T>
+__device__ __forceinline__ void put(Cx<T>* buf, int i, Cx<T> v) {
+  typedef typename std::conditional<sizeof(T) == 8, uint4, uint2>::type Word;
+  Word w;
+  memcpy(&w, &v, sizeof w);
+  reinterpret_cast<Word*>(buf)[i] = w;
+}
+template <typename T>
+__device__ __forceinline__ Cx<T> get(const Cx<T>* buf, int i) {
+  typedef typename std::conditional<sizeof(T) == 8, uint4, uint2>::type Word;
+  const Word w = reinterpret_cast<const Word*>(buf)[i];
+  Cx<T> v;
+  memcpy(&v, &w, sizeof w);
+  return v;
+}
+
+// The 4096-point transform of the CTA: on entry thread b holds cells
+// 256 a + b (a = 0 .. 15); on return, with p = tid >> 4 and r = tid & 15,
+// out[s] holds the value at offset p + 16 r + 256 s - 1024 from the run's
+// centre, s = 0 .. 7.  buf: 4096 complex words, free once every thread has
+// passed the first barrier here; free again only after a barrier of the
+// caller.  The second exchange stays within the 16 threads of one p, in the
+// 256 words that only they read in the first one, so it needs no barrier of
+// the whole CTA.
+// tw1[256 (p - 1) + b] = e^{2 pi i p b / 4096}, tw2[16 (r - 1) + d] = e^{2 pi i r d / 256}.
+template <typename T>
+__device__ __forceinline__ void fft4096(Cx<T> (&x)[16], Cx<T>* buf, const typename Twiddle<T>::type* __restrict__ tw1,
+                                        const typename Twiddle<T>::type* __restrict__ tw2, Cx<T> (&out)[8]) {
+  const int tid = threadIdx.x;
+  dft16(x);
+#pragma unroll
+  for (int p = 1; p < 16; ++p) {
+    const int q = 4 * (p & 3) + (p >> 2);
+    x[q] = cmul(x[q], __ldg(&tw1[(p - 1) * 256 + tid]));
+  }
+  __syncthreads();  // every thread has read its cells
+#pragma unroll
+  for (int p = 0; p < 16; ++p) put(buf, p * 256 + tid, x[4 * (p & 3) + (p >> 2)]);
+  __syncthreads();
+  Cx<T>* const own = buf + (tid >> 4) * 256;
+  const int d = tid & 15;
+#pragma unroll
+  for (int c = 0; c < 16; ++c) x[c] = get(own, 16 * c + d);
+  dft16(x);
+#pragma unroll
+  for (int r = 1; r < 16; ++r) {
+    const int q = 4 * (r & 3) + (r >> 2);
+    x[q] = cmul(x[q], __ldg(&tw2[(r - 1) * 16 + d]));
+  }
+  __syncwarp();
+  // word (r, d) at 16 r + (d ^ r): the lanes of either the writing order (d
+  // runs) or the reading order (r runs) fall on distinct banks
+#pragma unroll
+  for (int r = 0; r < 16; ++r) put(own, 16 * r + (d ^ r), x[4 * (r & 3) + (r >> 2)]);
+  __syncwarp();
+#pragma unroll
+  for (int e = 0; e < 16; ++e) x[e] = get(own, 16 * d + (e ^ d));
+  dft16_first(x);
+#pragma unroll
+  for (int k1 = 0; k1 < 4; ++k1) {
+    const Cx<T> x0 = x[4 * k1], x1 = x[4 * k1 + 1], x2 = x[4 * k1 + 2], x3 = x[4 * k1 + 3];
+    out[4 + k1] = (x0 + x2) + (x1 + x3);    // s = k1 of the transform's 16
+    out[k1] = sub_i(x0 - x2, x1 - x3);      // s = 12 + k1
+  }
+}
+
+// -------------------------------------------------------------------- power
+// Eq. 2 from Z and W (lsp_power_f32 with its sums already combined).
+__device__ __forceinline__ float power_zw(float zr, float zi, float wr, float wi, float n, bool& ill) {
+  const float r2 = fmaf(wr, wr, wi * wi);
+  const float nn = n * n;
+  const float z2 = fmaf(zr, zr, zi * zi);
+  const float re = fmaf((zr - zi) * (zr + zi), wr, 2.0f * zr * zi * wi);
+  const float num = fmaf(n, z2, -re);
+  const float den = nn - r2;
+  ill = r2 > kIllR2 * nn;
+  return den > 0.0f ? __fdividef(fmaxf(num, 0.0f), den) : 0.0f;
+}
+
+// (N |Z|^2 - Re(Z^2 conj W)) / (N^2 - |W|^2), as lsp_power_f32.
+__device__ __forceinline__ dd power_dd(Cx<dd> z, Cx<dd> w, dd n, bool& ill) {
+  const dd w2 = add_(mul_(w.re, w.re), mul_(w.im, w.im));
+  const dd nn = mul_(n, n);
+  const dd zr2 = mul_(z.re, z.re), zi2 = mul_(z.im, z.im);
+  dd b = mul_(z.re, z.im);
+  b = dd{2.0f * b.hi, 2.0f * b.lo};
+  const dd re = add_(mul_(sub_(zr2, zi2), w.re), mul_(b, w.im));
+  const dd num = sub_(mul_(n, add_(zr2, zi2)), re);
+  const dd den = sub_(nn, w2);
+  ill = w2.hi > kIllR2 * nn.hi;
+  if (!(den.hi > 0.0f) || !(num.hi > 0.0f)) return dd{0.0f, 0.0f};
+  const float q = __fdiv_rn(num.hi, den.hi);
+  const dd r = sub_(num, mul_(den, dd{q, 0.0f}));
+  return dd_fast(q, __fdiv_rn(r.hi, den.hi));
+}
+
+}  // namespace lsp

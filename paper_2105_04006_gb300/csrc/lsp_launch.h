@@ -15,11 +15,23 @@ namespace lsp {
 // and dynamic shared memory together pass the 48 KB available by default.
 template <typename Kern>
 inline cudaError_t allow_dyn_smem(Kern kern, size_t dyn) {
-  cudaFuncAttributes a{};
-  cudaError_t e = cudaFuncGetAttributes(&a, kern);
-  if (e != cudaSuccess) return e;
-  if (dyn + a.sharedSizeBytes <= 48 * 1024) return cudaSuccess;
+  if (dyn == 0) return cudaSuccess;  // static shared memory alone never passes it
+  if (dyn <= 48 * 1024) {
+    cudaFuncAttributes a{};
+    cudaError_t e = cudaFuncGetAttributes(&a, kern);
+    if (e != cudaSuccess) return e;
+    if (dyn + a.sharedSizeBytes <= 48 * 1024) return cudaSuccess;
+  }
   return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+}
+
+// CTAs of a kernel resident per SM (0 on an error), asked of the runtime once
+// per device, kernel and shape: the query costs several microseconds, as much
+// as the smallest calls' kernels.
+int cached_blocks_per_sm(const void* kern, int threads, size_t dyn);
+template <typename Kern>
+inline int blocks_per_sm(Kern* kern, int threads, size_t dyn) {
+  return cached_blocks_per_sm(reinterpret_cast<const void*>(kern), threads, dyn);
 }
 
 // Prologue, Section 2 (zero-mean magnitudes) and the per-observation phase
@@ -88,13 +100,15 @@ int main_blocks_per_sm(int prec, int packed, int k_reseed, int fpt, int threads,
 size_t main_dyn_smem(int prec, int fpt, int threads, int top);
 
 // Transform path (lsp_transform.cu): the trig sums of runs of kTfBins bins by
-// a nonuniform FFT; FP32, standard and generalized periodogram.
+// a nonuniform FFT; FP32 (standard and generalized periodogram) and FP64
+// (standard).
 constexpr int kTfBins = 2048;
-struct TransformParams {
-  const RecF32* rec;
+template <typename Rec, typename Real>
+struct TransformParamsOf {
+  const Rec* rec;
   const ObjInfo* obj;
   const int32_t* order_back;  // last word of the object list, read backwards (nullptr: identity)
-  float* power_out;      // nullable, n_obj x n_f
+  Real* power_out;      // nullable, n_obj x n_f
   ChunkBest* best;
   ChunkCand* cand;       // nullable: only with top_k > 1
   uint32_t* queue;       // zeroed work counter
@@ -109,8 +123,25 @@ struct TransformParams {
   double f_min, df;
   uint32_t* ticket;
 };
+typedef TransformParamsOf<RecF32, float> TransformParams;
+typedef TransformParamsOf<RecF64, double> TransformParams64;
 cudaError_t launch_transform(const TransformParams& p, int gls, int grid, cudaStream_t stream);
-int transform_blocks_per_sm(int gls);
+cudaError_t launch_transform64(const TransformParams64& p, int grid, cudaStream_t stream);
+int transform_blocks_per_sm(int prec, int gls);  // 0: no such kernel
+// One object on its whole grid by one large transform (lsp_long.cu).
+constexpr int kLongMaxLog2 = 22;
+struct LongPlan {
+  int lg, lg2;   // log2 of the transform's length and of its second pass's
+  int32_t kc;    // the bin at offset 0
+  size_t cell_bytes, t_bytes, row_bytes;  // scratch
+};
+bool long_plan(int prec, int64_t n_f, LongPlan* lp);  // false: the grid is too long
+// p: rec, obj, power_out, best, cand, n_chunks, n_f, peaks, f_min, df, ticket;
+// max_n: an upper bound of the object's observations.
+cudaError_t launch_long32(const LongPlan& lp, const TransformParams& p, int64_t max_n, void* cells, void* t, void* row,
+                          cudaStream_t stream);
+cudaError_t launch_long64(const LongPlan& lp, const TransformParams64& p, int64_t max_n, void* cells, void* t,
+                          void* row, cudaStream_t stream);
 // The work lists of a batch that takes both paths: objects of at least
 // `n_min` observations (the transform) from the back of order[], the others
 // (the direct kernel) from its front, each list by decreasing N_t;

@@ -14,14 +14,6 @@ cudaError_t launch_kernel(Kern kern, const MainLaunch& ml, const P& p, cudaStrea
   return cudaGetLastError();
 }
 
-template <typename Kern>
-int occupancy(Kern kern, int threads, size_t dyn) {
-  int nb = 0;
-  if (allow_dyn_smem(kern, dyn) != cudaSuccess) return 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, threads, dyn) != cudaSuccess) return 0;
-  return nb;
-}
-
 // abl: ablation code trig + 3 * staging (0: the production kernels); the
 // ablation kernels are scalar, K = 16, standard periodogram only.
 template <typename Fn>
@@ -82,7 +74,7 @@ bool main_variant_exists_f32(int packed, int k, int fpt, int gls, int abl) {
 int main_blocks_per_sm_f32(int packed, int k, int fpt, int threads, int top, int gls, int abl) {
   int nb = 0;
   size_t dyn = main_dyn_smem(0, fpt, threads, top);
-  dispatch_f32(packed, k, gls, abl, threads, [&](auto kern) { nb = occupancy(kern, threads, dyn); });
+  dispatch_f32(packed, k, gls, abl, threads, [&](auto kern) { nb = blocks_per_sm(kern, threads, dyn); });
   return nb;
 }
 

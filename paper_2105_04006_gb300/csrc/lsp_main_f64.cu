@@ -31,10 +31,7 @@ bool main_variant_exists_f64(int k, int fpt, int gls) {
 int main_blocks_per_sm_f64(int k, int fpt, int threads, int top, int gls) {
   int nb = 0;
   size_t dyn = main_dyn_smem(1, fpt, threads, top);
-  dispatch_f64(k, gls, [&](auto kern) {
-    if (allow_dyn_smem(kern, dyn) != cudaSuccess || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, threads, dyn) != cudaSuccess)
-      nb = 0;
-  });
+  dispatch_f64(k, gls, [&](auto kern) { nb = blocks_per_sm(kern, threads, dyn); });
   return nb;
 }
 

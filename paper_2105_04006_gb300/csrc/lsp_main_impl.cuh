@@ -692,12 +692,13 @@ __global__ void __launch_bounds__(256) main_scalar(MainParams<Rec, Real> p) {
   const int tid = threadIdx.x;
   const Rec* srec = reinterpret_cast<const Rec*>(s_rec);
 
+  const int64_t n_items = p.n_items_dev ? (int64_t)*p.n_items_dev : p.n_items;
   for (;;) {
     if (tid == 0) s_item = atomicAdd(p.queue, 1u);
     __syncthreads();
     const int64_t item = s_item;
     __syncthreads();
-    if (item >= p.n_items) break;
+    if (item >= n_items) break;
     const Item it = decode_item(p, item);
     const ObjInfo oi = p.obj[it.o];
     const int64_t kc0 = (int64_t)it.chunk * blockDim.x * F;

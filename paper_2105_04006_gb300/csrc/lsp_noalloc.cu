@@ -11,7 +11,7 @@
 //
 // Limits and sharing:
 //   - The scratch array holds LSP_NOALLOC_SCRATCH_BYTES (32 MiB).  A shape
-//     whose lsp_workspace_size exceeds it is rejected with LSP_E_WORKSPACE
+//     that no path of lsp_batch runs within it is rejected with LSP_E_WORKSPACE
 //     before anything is launched.
 //   - When the array is reserved: the CUDA runtime places it in device
 //     memory when it loads this file's module on a device.  With lazy module
@@ -38,6 +38,7 @@
 
 namespace lsp {
 void set_last_error(const char* msg);
+lsp_status least_workspace(int64_t n_obj, int64_t total_nt, const lsp_grid* grid, const lsp_opts* opts, size_t* bytes);
 }
 
 namespace {
@@ -98,7 +99,7 @@ extern "C" lsp_status lsp_batch_noalloc(const double* t, const void* y, const in
                                         const lsp_opts* opts, void* power_out, lsp_peak* peaks,
                                         lsp_stream_t stream) {
   size_t need = 0;
-  lsp_status st = lsp_workspace_size(n_obj, total_nt, grid, opts, &need);
+  lsp_status st = lsp::least_workspace(n_obj, total_nt, grid, opts, &need);
   if (st != LSP_OK) return st;
   if (n_obj == 0) return LSP_OK;  // nothing to do: no lookup, no module load
   if (need > (size_t)LSP_NOALLOC_SCRATCH_BYTES) {

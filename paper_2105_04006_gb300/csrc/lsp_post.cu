@@ -1,5 +1,6 @@
 // lsp_post.cu -- split-N_t combine, per-object peaks, stored-periodogram argmax.
 #include <cmath>
+#include <mutex>
 #include <type_traits>
 
 #include "../../include/lsp.h"
@@ -7,6 +8,34 @@
 #include "lsp_peak.cuh"
 
 namespace lsp {
+
+int cached_blocks_per_sm(const void* kern, int threads, size_t dyn) {
+  struct Entry {
+    const void* kern;
+    int dev, threads, blocks;
+    size_t dyn;
+  };
+  constexpr int kMost = 256;  // kernels x shapes in use; past it the runtime is asked again
+  static std::mutex mu;
+  static Entry known[kMost];
+  static int n_known = 0;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  {
+    std::lock_guard<std::mutex> lk(mu);
+    for (int i = 0; i < n_known; ++i) {
+      const Entry& e = known[i];
+      if (e.kern == kern && e.dev == dev && e.threads == threads && e.dyn == dyn) return e.blocks;
+    }
+  }
+  int nb = 0;
+  if (allow_dyn_smem(kern, dyn) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, threads, dyn) != cudaSuccess)
+    return 0;
+  std::lock_guard<std::mutex> lk(mu);
+  if (n_known < kMost) known[n_known++] = Entry{kern, dev, threads, nb, dyn};
+  return nb;
+}
 
 bool main_variant_exists_f32(int packed, int k, int fpt, int gls, int abl);
 bool main_variant_exists_f64(int k, int fpt, int gls);

@@ -44,6 +44,7 @@
 #include <type_traits>
 
 #include "../../include/lsp.h"
+#include "lsp_fft.cuh"
 #include "lsp_launch.h"
 #include "lsp_peak.cuh"
 
@@ -51,6 +52,7 @@ namespace lsp {
 
 namespace {
 
+#define LSP_TF_TABLES_F32
 #include "lsp_transform_tables.inc"
 
 constexpr int kM = 4096;                 // grid cells
@@ -58,147 +60,6 @@ constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 constexpr size_t kPowers = kTfBins + kTfBins / 16;  // a word of padding per 16 powers
 static_assert(kTfBins == kM / 2 && kTfBins == kThreads * 8 && kTfGroups == kM / 8, "run length");
-
-// ------------------------------------------------------------ arithmetic on
-// f32x2 pairs (two transforms at once) or single floats
-__device__ __forceinline__ f2_t add_(f2_t a, f2_t b) {
-  f2_t d;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ f2_t sub_(f2_t a, f2_t b) { return f2_fma(b, 0xbf800000bf800000ull, a); }
-__device__ __forceinline__ float add_(float a, float b) { return a + b; }
-__device__ __forceinline__ float sub_(float a, float b) { return a - b; }
-__device__ __forceinline__ f2_t mul_(f2_t a, f2_t b) { return f2_mul(a, b); }
-__device__ __forceinline__ float mul_(float a, float b) { return a * b; }
-__device__ __forceinline__ f2_t fma_(f2_t a, f2_t b, f2_t c) { return f2_fma(a, b, c); }
-__device__ __forceinline__ float fma_(float a, float b, float c) { return fmaf(a, b, c); }
-template <typename T> __device__ __forceinline__ T dup_(float v);
-template <> __device__ __forceinline__ f2_t dup_<f2_t>(float v) { return f2_pack(v, v); }
-template <> __device__ __forceinline__ float dup_<float>(float v) { return v; }
-
-template <typename T>
-struct Cx {
-  T re, im;
-};
-template <typename T>
-__device__ __forceinline__ Cx<T> operator+(Cx<T> a, Cx<T> b) { return {add_(a.re, b.re), add_(a.im, b.im)}; }
-template <typename T>
-__device__ __forceinline__ Cx<T> operator-(Cx<T> a, Cx<T> b) { return {sub_(a.re, b.re), sub_(a.im, b.im)}; }
-// a + i b and a - i b
-template <typename T>
-__device__ __forceinline__ Cx<T> add_i(Cx<T> a, Cx<T> b) { return {sub_(a.re, b.im), add_(a.im, b.re)}; }
-template <typename T>
-__device__ __forceinline__ Cx<T> sub_i(Cx<T> a, Cx<T> b) { return {add_(a.re, b.im), sub_(a.im, b.re)}; }
-template <typename T>
-__device__ __forceinline__ Cx<T> cmul(Cx<T> a, float wr, float wi) {
-  const T r = dup_<T>(wr), i = dup_<T>(wi), ni = dup_<T>(-wi);
-  return {fma_(a.im, ni, mul_(a.re, r)), fma_(a.re, i, mul_(a.im, r))};
-}
-
-// In-place transform of 4 points with e^{+2 pi i jk/4}.
-template <typename T>
-__device__ __forceinline__ void dft4(Cx<T>& x0, Cx<T>& x1, Cx<T>& x2, Cx<T>& x3) {
-  const Cx<T> a = x0 + x2, b = x0 - x2, c = x1 + x3, d = x1 - x3;
-  x0 = a + c;
-  x1 = add_i(b, d);
-  x2 = a - c;
-  x3 = sub_i(b, d);
-}
-
-// First half of the 16-point transform: afterwards x[4 k1 + n2] holds the
-// k1-th output of the n2-th inner transform, times e^{2 pi i n2 k1 / 16}.
-template <typename T>
-__device__ __forceinline__ void dft16_first(Cx<T> (&x)[16]) {
-#pragma unroll
-  for (int n2 = 0; n2 < 4; ++n2) dft4(x[n2], x[4 + n2], x[8 + n2], x[12 + n2]);
-  constexpr float c1 = 0.92387953251128676f, s1 = 0.38268343236508977f, h = 0.70710678118654752f;
-  x[4 * 1 + 1] = cmul(x[4 * 1 + 1], c1, s1);   // W^1
-  x[4 * 2 + 1] = cmul(x[4 * 2 + 1], h, h);     // W^2
-  x[4 * 3 + 1] = cmul(x[4 * 3 + 1], s1, c1);   // W^3
-  x[4 * 1 + 2] = cmul(x[4 * 1 + 2], h, h);     // W^2
-  {
-    const Cx<T> v = x[4 * 2 + 2];              // W^4 = i
-    x[4 * 2 + 2] = Cx<T>{mul_(v.im, dup_<T>(-1.0f)), v.re};
-  }
-  x[4 * 3 + 2] = cmul(x[4 * 3 + 2], -h, h);    // W^6
-  x[4 * 1 + 3] = cmul(x[4 * 1 + 3], s1, c1);   // W^3
-  x[4 * 2 + 3] = cmul(x[4 * 2 + 3], -h, h);    // W^6
-  x[4 * 3 + 3] = cmul(x[4 * 3 + 3], -c1, -s1); // W^9
-}
-// The whole 16-point transform; output k sits at x[4 (k & 3) + (k >> 2)].
-template <typename T>
-__device__ __forceinline__ void dft16(Cx<T> (&x)[16]) {
-  dft16_first(x);
-#pragma unroll
-  for (int k1 = 0; k1 < 4; ++k1) dft4(x[4 * k1], x[4 * k1 + 1], x[4 * k1 + 2], x[4 * k1 + 3]);
-}
-
-// One 16-byte (f2_t) or 8-byte (float) complex word of the exchange buffer.
-__device__ __forceinline__ void put(f2_t* buf, int i, Cx<f2_t> v) {
-  reinterpret_cast<ulonglong2*>(buf)[i] = make_ulonglong2(v.re, v.im);
-}
-__device__ __forceinline__ Cx<f2_t> get(const f2_t* buf, int i) {
-  const ulonglong2 v = reinterpret_cast<const ulonglong2*>(buf)[i];
-  return {v.x, v.y};
-}
-__device__ __forceinline__ void put(float* buf, int i, Cx<float> v) {
-  reinterpret_cast<float2*>(buf)[i] = make_float2(v.re, v.im);
-}
-__device__ __forceinline__ Cx<float> get(const float* buf, int i) {
-  const float2 v = reinterpret_cast<const float2*>(buf)[i];
-  return {v.x, v.y};
-}
-
-// The 4096-point transform of the CTA: on entry thread b holds cells
-// 256 a + b (a = 0 .. 15); on return, with p = tid >> 4 and r = tid & 15,
-// out[s] holds the value at offset p + 16 r + 256 s - 1024 from the run's
-// centre, s = 0 .. 7.  buf: 4096 complex words, free once every thread has
-// passed the first barrier here; free again only after a barrier of the
-// caller.  The second exchange stays within the 16 threads of one p, in the
-// 256 words that only they read in the first one, so it needs no barrier of
-// the whole CTA.
-template <typename T>
-__device__ __forceinline__ void fft4096(Cx<T> (&x)[16], T* buf, Cx<T> (&out)[8]) {
-  const int tid = threadIdx.x;
-  dft16(x);
-#pragma unroll
-  for (int p = 1; p < 16; ++p) {
-    const float2 w = __ldg(&kTfTw1[(p - 1) * 256 + tid]);
-    const int q = 4 * (p & 3) + (p >> 2);
-    x[q] = cmul(x[q], w.x, w.y);
-  }
-  __syncthreads();  // every thread has read its cells
-#pragma unroll
-  for (int p = 0; p < 16; ++p) put(buf, p * 256 + tid, x[4 * (p & 3) + (p >> 2)]);
-  __syncthreads();
-  T* const own = buf + (tid >> 4) * 512;  // 256 complex words
-  const int d = tid & 15;
-#pragma unroll
-  for (int c = 0; c < 16; ++c) x[c] = get(own, 16 * c + d);
-  dft16(x);
-#pragma unroll
-  for (int r = 1; r < 16; ++r) {
-    const float2 w = __ldg(&kTfTw2[(r - 1) * 16 + d]);
-    const int q = 4 * (r & 3) + (r >> 2);
-    x[q] = cmul(x[q], w.x, w.y);
-  }
-  __syncwarp();
-  // word (r, d) at 16 r + (d ^ r): the lanes of either the writing order (d
-  // runs) or the reading order (r runs) fall on distinct banks
-#pragma unroll
-  for (int r = 0; r < 16; ++r) put(own, 16 * r + (d ^ r), x[4 * (r & 3) + (r >> 2)]);
-  __syncwarp();
-#pragma unroll
-  for (int e = 0; e < 16; ++e) x[e] = get(own, 16 * d + (e ^ d));
-  dft16_first(x);
-#pragma unroll
-  for (int k1 = 0; k1 < 4; ++k1) {
-    const Cx<T> x0 = x[4 * k1], x1 = x[4 * k1 + 1], x2 = x[4 * k1 + 2], x3 = x[4 * k1 + 3];
-    out[4 + k1] = (x0 + x2) + (x1 + x3);    // s = k1 of the transform's 16
-    out[k1] = sub_i(x0 - x2, x1 - x3);      // s = 12 + k1
-  }
-}
 
 __device__ __forceinline__ f2_t cells_f2(const int32_t* a, const int32_t* b, int i) {
   return f2_pack(__int2float_rn(a[i]), __int2float_rn(b[i]));
@@ -215,18 +76,6 @@ struct Smem {
   static constexpr size_t total = grid + stage;
   static_assert(stage >= 2 * kTfGroups * 4, "the counts use the staging area");
 };
-
-// Eq. 2 from Z and W (lsp_power_f32 with its sums already combined).
-__device__ __forceinline__ float power_zw(float zr, float zi, float wr, float wi, float n, bool& ill) {
-  const float r2 = fmaf(wr, wr, wi * wi);
-  const float nn = n * n;
-  const float z2 = fmaf(zr, zr, zi * zi);
-  const float re = fmaf((zr - zi) * (zr + zi), wr, 2.0f * zr * zi * wi);
-  const float num = fmaf(n, z2, -re);
-  const float den = nn - r2;
-  ill = r2 > kIllR2 * nn;
-  return den > 0.0f ? __fdividef(fmaxf(num, 0.0f), den) : 0.0f;
-}
 
 template <bool GLS>
 __global__ void __launch_bounds__(kThreads, 2) transform_kernel(TransformParams p) {
@@ -353,7 +202,7 @@ __global__ void __launch_bounds__(kThreads, 2) transform_kernel(TransformParams 
         const int i = 256 * a + tid;
         x[a] = Cx<f2_t>{cells_f2(plane, plane + 2 * kM, i), cells_f2(plane + kM, plane + 3 * kM, i)};
       }
-      fft4096(x, reinterpret_cast<f2_t*>(plane), out);
+      fft4096(x, reinterpret_cast<Cx<f2_t>*>(plane), kTfTw1, kTfTw2, out);
       const f2_t inv = f2_pack(1.0f / y_sc, 1.0f / w_sc);
       const float nf = (float)oi.n;
 #pragma unroll
@@ -380,7 +229,7 @@ __global__ void __launch_bounds__(kThreads, 2) transform_kernel(TransformParams 
           const int i = 256 * a + tid;
           x[a] = Cx<f2_t>{cells_f2(plane, plane + 2 * kM, i), cells_f2(plane + kM, plane + 3 * kM, i)};
         }
-        fft4096(x, reinterpret_cast<f2_t*>(plane), out);
+        fft4096(x, reinterpret_cast<Cx<f2_t>*>(plane), kTfTw1, kTfTw2, out);
       }
       {
         Cx<float> x[16];
@@ -389,7 +238,7 @@ __global__ void __launch_bounds__(kThreads, 2) transform_kernel(TransformParams 
           const int i = kW * kM + 256 * a + tid;
           x[a] = Cx<float>{__int2float_rn(plane[i]), __int2float_rn(plane[kM + i])};
         }
-        fft4096(x, reinterpret_cast<float*>(plane), outw);
+        fft4096(x, reinterpret_cast<Cx<float>*>(plane), kTfTw1, kTfTw2, outw);
       }
       const f2_t inv = f2_pack(1.0f / y_sc, 1.0f / c_sc);
       const float inv_w = 1.0f / w_sc, wsum = oi.wsum_f, yy = (float)oi.sum_y2;
@@ -458,18 +307,12 @@ __global__ void __launch_bounds__(kThreads, 2) transform_kernel(TransformParams 
 
 }  // namespace
 
-int transform_blocks_per_sm(int gls) {
-  int nb = 0;
-  auto occ = [&](auto kern, size_t dyn) {
-    if (allow_dyn_smem(kern, dyn) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, kThreads, dyn) != cudaSuccess)
-      nb = 0;
-  };
-  if (gls)
-    occ(transform_kernel<true>, Smem<true>::total);
-  else
-    occ(transform_kernel<false>, Smem<false>::total);
-  return nb;
+int transform_blocks_per_sm64();
+
+int transform_blocks_per_sm(int prec, int gls) {
+  if (prec) return gls ? 0 : transform_blocks_per_sm64();
+  return gls ? blocks_per_sm(transform_kernel<true>, kThreads, Smem<true>::total)
+             : blocks_per_sm(transform_kernel<false>, kThreads, Smem<false>::total);
 }
 
 cudaError_t launch_transform(const TransformParams& p, int gls, int grid, cudaStream_t stream) {

@@ -113,3 +113,83 @@ def test_plan_uses_the_transform_until_told_otherwise(env):
     _, direct = lsp.batch(*args, g, k_reseed=8, freqs_per_thread=16, block_threads=128)
     assert torch.equal(plan.execute(*args), direct) and not torch.equal(direct, want)
     plan.close()
+
+
+@pytest.mark.parametrize("n_t,n_f", [(8, 1), (9, 2047), (33, 32737), (300, 32738), (1000, 65505), (7001, 20_011)])
+@pytest.mark.parametrize("cadence", ["uniform", "nightly", "long"])
+def test_single_object_fp64(env, n_t, n_f, cadence):
+    """The FP64 path's two-float transform of the whole grid, on either side of its grid's powers of two
+    (2 (N_f + 32) cells), at the FP64 path's own tolerance."""
+    lsp, torch, dev = env
+    t, y, _ = _segments([n_t], cadence, 11)
+    g = lsp.Grid(0.24, 12.0, n_f)
+    p, pk = lsp.periodogram(torch.tensor(t, device=dev), torch.tensor(y, device=dev), g, precision="fp64")
+    p, pk = p.cpu().numpy(), lsp.peaks_to_numpy(pk)
+    ks = np.unique(np.concatenate([np.linspace(0, n_f - 1, 300).astype(np.int64), np.arange(max(0, n_f - 5), n_f)]))
+    if cadence == "long":
+        # 2.4e6 cycles: the oracle's FP64 phases are good to 2.4e6 x 2^-53 cycle only, the library's fixed-point
+        # ones are exact; the direct kernel has the same phases
+        ref = lsp.periodogram(torch.tensor(t, device=dev), torch.tensor(y, device=dev), g, precision="fp64",
+                              k_reseed=16)[0].cpu().numpy()[ks]
+    else:
+        ref, _ = oracle.lsp_single(t, y, 0.24, 12.0, n_f, k_sel=ks)
+    assert np.isfinite(p).all() and np.max(np.abs(p[ks] - ref)) <= 1e-10
+    assert pk["idx"][0] == int(np.argmax(p)) and pk["power"][0] == p.max()
+
+
+@pytest.mark.parametrize("n_t,n_f", [(6000, 1), (9001, 16_352), (20_000, 16_353), (30_000, 600_000)])
+@pytest.mark.parametrize("top_k", [1, 3])
+def test_single_object_of_many_observations(env, n_t, n_f, top_k):
+    """FP32, the whole grid in one transform (its second pass of 256, 512 points)."""
+    lsp, torch, dev = env
+    b = synth.single_large(n_t=n_t, grid=synth.Grid(0.05, 25.0, n_f))
+    t, y = torch.tensor(b.t, device=dev), torch.tensor(b.y.astype(np.float32), device=dev)
+    p, pk = lsp.periodogram(t, y, lsp.Grid(0.05, 25.0, n_f), top_k=top_k)
+    p, pk = p.cpu().numpy(), lsp.peaks_to_numpy(pk)
+    ks = np.unique(np.concatenate([np.linspace(0, n_f - 1, 200).astype(np.int64), np.arange(max(0, n_f - 5), n_f)]))
+    ref, _ = oracle.lsp_single(b.t, b.y.astype(np.float32).astype(np.float64), 0.05, 25.0, n_f, k_sel=ks)
+    assert np.isfinite(p).all() and np.max(np.abs(p[ks] - ref)) <= TOL
+    if top_k == 1 or n_f > 1:
+        idx = [int(np.argmax(p))] if top_k == 1 else list(oracle.top_local_maxima(p.astype(np.float64), 3)[0])
+        assert list(pk["idx"]) == idx
+
+
+@pytest.mark.parametrize("cadence", ["uniform", "one_night", "nightly", "long"])
+def test_fp64_batch_both_sides_of_every_edge(env, cadence):
+    lsp, torch, dev = env
+    counts = [3, 7, 8, 9, 31, 64, 255, 256, 257, 511, 513, 2600]
+    t, y, off = _segments(counts, cadence, 9)
+    g = lsp.Grid(0.24, 12.0, 4099)
+    args = [torch.tensor(a, device=dev) for a in (t, y, off)]
+    p, pk = lsp.batch(*args, g, precision="fp64", return_power=True)
+    direct = lsp.batch(*args, g, precision="fp64", return_power=True, k_reseed=16)[0].cpu().numpy()
+    if cadence == "long":  # as in test_single_object_fp64
+        ref = direct
+    else:
+        ref = oracle.lsp_batch(t, y, off, 0.24, 12.0, 4099, return_power=True)["power"]
+    p = p.cpu().numpy()
+    np.testing.assert_array_equal(p[:2], direct[:2])  # 3 and 7 observations: left to the direct kernel
+    err = np.abs(p - ref).max(axis=1)[2:]
+    assert err.max() <= 1e-10, dict(zip(counts[2:], err))
+    np.testing.assert_array_equal(lsp.peaks_to_numpy(pk)["idx"], np.argmax(p, axis=1))
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_smaller_workspaces_take_smaller_paths(env, precision):
+    """A workspace that holds only what the direct kernel needs is enough: the call takes that kernel."""
+    lsp, torch, dev = env
+    b = synth.single_small(n_t=9000, grid=synth.Grid(0.1, 10.0, 3001))
+    dt = torch.float32 if precision == "fp32" else torch.float64
+    t, y = torch.tensor(b.t, device=dev), torch.tensor(b.y, dtype=dt, device=dev)
+    g = lsp.Grid(0.1, 10.0, 3001)
+    k = 8 if precision == "fp32" else 16
+    need = lsp.workspace_size(1, 9000, g, lsp.make_opts(precision=precision, k_reseed=k))
+    full = lsp.workspace_size(1, 9000, g, lsp.make_opts(precision=precision))
+    want, _ = lsp.periodogram(t, y, g, precision=precision)
+    direct, _ = lsp.periodogram(t, y, g, precision=precision, k_reseed=k)
+    ws = torch.empty(need, dtype=torch.uint8, device=dev)
+    got, _ = lsp.periodogram(t, y, g, precision=precision, workspace=ws)
+    assert torch.equal(got, direct if need < full else want)
+    assert torch.allclose(want, direct, rtol=0, atol=TOL if precision == "fp32" else 1e-10)
+    with pytest.raises(lsp.LSPError):
+        lsp.periodogram(t, y, g, precision=precision, workspace=torch.empty(1024, dtype=torch.uint8, device=dev))

@@ -107,7 +107,8 @@ template <typename Rec, typename Real>
 struct TransformParamsOf {
   const Rec* rec;
   const ObjInfo* obj;
-  const int32_t* order_back;  // last word of the object list, read backwards (nullptr: identity)
+  const int32_t* order = nullptr;       // object list, read forwards, or
+  const int32_t* order_back = nullptr;  // its last word, read backwards (neither: identity)
   Real* power_out;      // nullable, n_obj x n_f
   ChunkBest* best;
   ChunkCand* cand;       // nullable: only with top_k > 1
@@ -116,6 +117,10 @@ struct TransformParamsOf {
   uint32_t n_items;
   int32_t n_chunks;      // runs per object
   int32_t have_scale;    // the records kernel left the scales (batches)
+  // FP32: per-object windows instead of runs from 0 (n_chunks = 1, one item
+  // per object): bins [win_start[o], win_start[o] + win_len) of the grid
+  const int32_t* win_start = nullptr;
+  int32_t win_len = 0;
   int64_t n_f;
   // one object, first maximum only: the peak is written by the last CTA
   // (ticket: a zeroed word); NULL: a finalize launch follows

@@ -389,7 +389,7 @@ lsp_status gemm(const Gemm& q, cudaStream_t s) {
   // Columns per CTA: 256, or fewer where that leaves SMs without a CTA (a
   // training batch of 4096 rows is 32 tiles: 32 columns make 256 of them).
   // The K order of every output, and so its bits, does not depend on it.
-  // Measured: train step of 4096 rows 494 -> 240 us together with the
+  // Measured: train step of 4096 rows 499 -> 228 us together with the
   // epilogue's transposed copy.
   const int row_tiles = (q.M + umma::BM - 1) / umma::BM * (q.splits < 1 ? 1 : q.splits);
   int n_tile = q.N >= umma::MAX_BN ? umma::MAX_BN : (q.N + 15) / 16 * 16;
@@ -644,10 +644,76 @@ __global__ void items_from_count(const uint32_t* count, uint32_t per, uint32_t* 
   *items = *count * per;
 }
 
+// The fallback's full grid by the transform, then the direct kernel on the
+// runs that can hold the maximum: P_n of either kernel is within 1e-4 of exact
+// (the library's FP32 tolerance), so the direct kernel's first maximum lies
+// in a run whose transform maximum is within 2e-4 of the largest one.  Those
+// runs become pseudo-objects (a copy of the object's record and a window
+// start) for one more launch of the direct kernel: the result is the one the
+// direct kernel gives on the whole grid, bit for bit, from one or two runs.
+// An object with more than kMaxRuns such runs, or past the room for them,
+// goes to the direct kernel's full grid.
+constexpr double kRunMargin = 2.5e-4;
+constexpr int kMaxRuns = 4;
+
+// One warp per listed object.  cand_of[o] = (first pseudo-object, count).
+__global__ void select_runs(const uint32_t* __restrict__ n_list, const int32_t* __restrict__ list, int n_chunks, int norm,
+                            const ObjInfo* __restrict__ obj, const ChunkBest* __restrict__ full, int cap,
+                            ObjInfo* __restrict__ cand_obj, int32_t* __restrict__ cand_win,
+                            int2* __restrict__ cand_of, uint32_t* n_cand, int32_t* __restrict__ list2, uint32_t* n_list2) {
+  const uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (i >= *n_list) return;
+  const int32_t o = list[i];
+  const ObjInfo oi = obj[o];
+  const ChunkBest* row = full + (int64_t)o * n_chunks;
+  double top = 0.0;
+  for (int c = lane; c < n_chunks; c += 32) top = fmax(top, row[c].p);
+  for (int off = 16; off > 0; off >>= 1) top = fmax(top, __shfl_xor_sync(0xffffffffu, top, off));
+  const double least = top - kRunMargin * (norm == LSP_NORM_STANDARD ? 1.0 : 0.5 * oi.sum_y2);
+  int count = 0;
+  for (int c = lane; c < n_chunks; c += 32) count += row[c].p >= least;
+  for (int off = 16; off > 0; off >>= 1) count += __shfl_xor_sync(0xffffffffu, count, off);
+  int first = 0;
+  if (lane == 0 && count <= kMaxRuns) first = (int)atomicAdd(n_cand, (uint32_t)count);
+  first = __shfl_sync(0xffffffffu, first, 0);
+  const bool fits = count <= kMaxRuns && first + count <= cap;
+  if (!fits) {
+    if (lane == 0) {
+      list2[atomicAdd(n_list2, 1u)] = o;
+      cand_of[o] = make_int2(0, 0);
+      // slots claimed inside the room hold no work
+      for (int q = first; count <= kMaxRuns && q < first + count && q < cap; ++q) {
+        ObjInfo none = oi;
+        none.n = 0;
+        none.flags = LSP_FLAG_FEW_OBS;
+        cand_obj[q] = none;
+        cand_win[q] = 0;
+      }
+    }
+    return;
+  }
+  if (lane == 0) cand_of[o] = make_int2(first, count);
+  int at = first;
+  for (int c0 = 0; c0 < n_chunks; c0 += 32) {
+    const bool hit = c0 + lane < n_chunks && row[c0 + lane].p >= least;
+    const unsigned m = __ballot_sync(0xffffffffu, hit);
+    if (hit) {
+      const int q = at + __popc(m & ((1u << lane) - 1u));
+      cand_obj[q] = oi;
+      cand_win[q] = (c0 + lane) * kTfBins;
+    }
+    at += __popc(m);
+  }
+}
+
+__global__ void capped_count(const uint32_t* count, uint32_t cap, uint32_t* items) { *items = min(*count, cap); }
+
 __global__ void refine_finalize(int64_t n_obj, const ObjInfo* __restrict__ obj,
                                 const RefineState* __restrict__ st, float fallback_power, int inconclusive,
-                                const ChunkBest* __restrict__ full_best, int n_chunks, double f_min,
-                                double df, lsp_peak* __restrict__ peaks, int32_t* __restrict__ info) {
+                                const ChunkBest* __restrict__ full_best, int n_chunks,
+                                const int2* __restrict__ cand_of, const ChunkBest* __restrict__ cand_best,
+                                double f_min, double df, lsp_peak* __restrict__ peaks, int32_t* __restrict__ info) {
   const int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (o >= n_obj) return;
   const RefineState s = st[o];
@@ -658,8 +724,11 @@ __global__ void refine_finalize(int64_t n_obj, const ObjInfo* __restrict__ obj,
   if (fb) {  // full grid: first maximum over the chunks
     p = 0.0;
     k = -1;
-    for (int c = 0; c < n_chunks; ++c) {
-      const ChunkBest b = full_best[o * n_chunks + c];
+    const int2 cand = cand_of ? cand_of[o] : make_int2(0, 0);
+    const ChunkBest* from = cand.y ? cand_best + cand.x : full_best + o * n_chunks;
+    const int n_from = cand.y ? cand.y : n_chunks;
+    for (int c = 0; c < n_from; ++c) {
+      const ChunkBest b = from[c];
       if (b.k >= 0 && (k < 0 || b.p > p || (b.p == p && b.k < k))) {
         p = b.p;
         k = b.k;
@@ -1043,8 +1112,11 @@ lsp_status lsp_top_classes(const float* logits, int64_t rows, int32_t n_classes,
 // lives here with its own workspace layout.
 namespace {
 struct RefineLayout {
-  size_t off_obj, off_rec, off_state, off_best, off_full, off_win, off_list, off_cnt, total;
+  size_t off_obj, off_rec, off_state, off_best, off_full, off_win, off_list, off_cnt, off_cand_obj, off_cand_best,
+      off_cand_win, off_cand_of, total;
   int n_chunks;
+  bool tf;     // windows and fallback runs by the transform
+  int n_cand;  // room for pseudo-objects of the fallback
 };
 // The refine kernel's configuration: 64 threads x 32 frequencies = 2048 bins
 // per item (K = 16 packed chains; the fastest shape measured on GB300 for
@@ -1053,7 +1125,8 @@ struct RefineLayout {
 constexpr int kRefineK = 16;
 constexpr int kRefineThreads = 64;
 
-void refine_layout(int64_t n_obj, int64_t total_nt, int64_t n_f, RefineLayout* r) {
+// tf: with the transform's scratch (without: direct kernels only).
+void refine_layout(int64_t n_obj, int64_t total_nt, int64_t n_f, RefineLayout* r, bool tf = true) {
   size_t off = 0;
   auto take = [&](size_t b) {
     size_t at = off;
@@ -1070,6 +1143,12 @@ void refine_layout(int64_t n_obj, int64_t total_nt, int64_t n_f, RefineLayout* r
   r->off_win = take((size_t)n_obj * sizeof(int32_t));
   r->off_list = take((size_t)n_obj * sizeof(int32_t));
   r->off_cnt = take(64);
+  r->tf = tf && n_obj * (int64_t)r->n_chunks < ((int64_t)1 << 31);  // 32-bit item numbers
+  r->n_cand = r->tf ? (int)(n_obj < ((int64_t)1 << 29) ? 2 * n_obj + kMaxRuns : n_obj) : 0;
+  r->off_cand_obj = take((size_t)r->n_cand * sizeof(ObjInfo));
+  r->off_cand_best = take((size_t)r->n_cand * sizeof(ChunkBest));
+  r->off_cand_win = take((size_t)r->n_cand * sizeof(int32_t));
+  r->off_cand_of = take(r->tf ? (size_t)n_obj * sizeof(int2) : 0);
   r->total = off;
 }
 }  // namespace
@@ -1118,7 +1197,9 @@ lsp_status refine_impl(const double* t, const float* y, const int64_t* offsets, 
   ChunkBest* full = (ChunkBest*)(ws + r.off_full);
   int32_t* win = (int32_t*)(ws + r.off_win);
   int32_t* list = (int32_t*)(ws + r.off_list);
-  uint32_t* cnt = (uint32_t*)(ws + r.off_cnt);  // [0] list count, [1] items, [2] queue
+  // [0] list count, [1] items, [2] queue; fallback: [3] pseudo-objects, [4] objects for the direct full grid,
+  // [5], [6] their items, [7], [8] their queues
+  uint32_t* cnt = (uint32_t*)(ws + r.off_cnt);
   const double df = (grid->f_max - grid->f_min) / (double)grid->n_f;
   int n_sm = 152, dev = 0;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
@@ -1126,7 +1207,8 @@ lsp_status refine_impl(const double* t, const float* y, const int64_t* offsets, 
   if (bps < 1) bps = 1;
 
   LEARN_CUDA(launch_stats(t, y, false, offsets, n_obj, total_nt, 1, norm, obj, s), "refine prologue");
-  LEARN_CUDA(launch_records(t, y, false, obj, n_obj, total_nt, grid->f_min, df, false, rec, s),
+  LEARN_CUDA(launch_records(t, y, false, obj, n_obj, total_nt, grid->f_min, df, false, rec, s, false, nullptr,
+                            r.tf && n_obj > 1 ? 1 : 0),
              "refine records");
   const unsigned g1 = (unsigned)((n_obj + 255) / 256);
   refine_init<<<g1, 256, 0, s>>>(n_obj, obj, state);
@@ -1146,6 +1228,27 @@ lsp_status refine_impl(const double* t, const float* y, const int64_t* offsets, 
   ml.queue = cnt + 2;
   ml.n_f = grid->n_f;
   ml.split = 1;
+  // Windows by the transform: one run each, hardly dependent on N_t (20000
+  // survey objects: 0.5 against 2.7 ms for the first round; the later rounds'
+  // few hundred objects 15 against 200 us, the time one CTA of the direct
+  // kernel takes for its object's observations).
+  TransformParams tp;
+  tp.rec = rec;
+  tp.obj = obj;
+  tp.order = list;
+  tp.power_out = nullptr;
+  tp.cand = nullptr;
+  tp.queue = cnt + 2;
+  tp.n_items = 0;
+  tp.n_items_dev = cnt + 1;
+  tp.have_scale = n_obj > 1;
+  tp.n_f = grid->n_f;
+  tp.peaks = nullptr;
+  tp.f_min = grid->f_min;
+  tp.df = df;
+  tp.ticket = nullptr;
+  int tbs = r.tf ? transform_blocks_per_sm(0, 0) : 0;
+  if (tbs < 1) tbs = 1;
   for (int rr = 0; rr < k_windows; ++rr) {
     LEARN_CUDA(cudaMemsetAsync(cnt, 0, 16, s), "refine counters");
     refine_list<<<g1, 256, 0, s>>>(n_obj, rr, k_windows, classes, stride, window, grid->n_f, state, win,
@@ -1158,23 +1261,62 @@ lsp_status refine_impl(const double* t, const float* y, const int64_t* offsets, 
     ml.win_start = win;
     ml.win_len = (int32_t)window;
     ml.grid = (int)(n_sm * bps);
-    LEARN_CUDA(launch_main(ml, s), "refine main kernel");
+    if (r.tf) {
+      tp.best = best;
+      tp.n_chunks = 1;
+      tp.win_start = win;
+      tp.win_len = (int32_t)window;
+      LEARN_CUDA(launch_transform(tp, 0, n_sm * tbs, s), "refine transform");
+    } else {
+      LEARN_CUDA(launch_main(ml, s), "refine main kernel");
+    }
     refine_merge<<<g1, 256, 0, s>>>(n_obj, rr, k_windows, stop_power, best, state);
   }
   // full-grid fallback for the objects whose refined peak stayed weak
-  LEARN_CUDA(cudaMemsetAsync(cnt, 0, 16, s), "fallback counters");
+  LEARN_CUDA(cudaMemsetAsync(cnt, 0, 64, s), "fallback counters");
   fallback_list<<<g1, 256, 0, s>>>(n_obj, fallback_power, inconclusive_fallback, obj, state, list, cnt);
   items_from_count<<<1, 1, 0, s>>>(cnt, (uint32_t)r.n_chunks, cnt + 1);
+  int2* cand_of = nullptr;
+  ChunkBest* cand_best = nullptr;
+  if (r.tf) {  // see select_runs
+    ObjInfo* cand_obj = (ObjInfo*)(ws + r.off_cand_obj);
+    int32_t* cand_win = (int32_t*)(ws + r.off_cand_win);
+    cand_best = (ChunkBest*)(ws + r.off_cand_best);
+    cand_of = (int2*)(ws + r.off_cand_of);
+    tp.best = full;
+    tp.n_chunks = r.n_chunks;
+    tp.win_start = nullptr;
+    tp.win_len = 0;
+    LEARN_CUDA(launch_transform(tp, 0, n_sm * tbs, s), "fallback transform");
+    select_runs<<<(unsigned)((n_obj + 7) / 8), 256, 0, s>>>(cnt, list, r.n_chunks, norm, obj, full, r.n_cand, cand_obj,
+                                                            cand_win, cand_of, cnt + 3, win, cnt + 4);
+    capped_count<<<1, 1, 0, s>>>(cnt + 3, (uint32_t)r.n_cand, cnt + 5);
+    items_from_count<<<1, 1, 0, s>>>(cnt + 4, (uint32_t)r.n_chunks, cnt + 6);
+    ml.obj = cand_obj;
+    ml.order = nullptr;
+    ml.best = cand_best;
+    ml.queue = cnt + 7;
+    ml.n_chunks = 1;
+    ml.n_items = r.n_cand;
+    ml.n_items_dev = cnt + 5;
+    ml.win_start = cand_win;
+    ml.win_len = kTfBins;
+    LEARN_CUDA(launch_main(ml, s), "fallback runs");
+    ml.obj = obj;
+    ml.order = win;
+    ml.queue = cnt + 8;
+    ml.n_items_dev = cnt + 6;
+  } else {
+    ml.n_items_dev = cnt + 1;
+  }
   ml.best = full;
   ml.n_chunks = r.n_chunks;
   ml.n_items = n_obj * (int64_t)r.n_chunks;
-  ml.n_items_dev = cnt + 1;
   ml.win_start = nullptr;
   ml.win_len = 0;
-  ml.grid = (int)(n_sm * bps);
   LEARN_CUDA(launch_main(ml, s), "fallback main kernel");
   refine_finalize<<<g1, 256, 0, s>>>(n_obj, obj, state, fallback_power, inconclusive_fallback, full,
-                                     r.n_chunks, grid->f_min, df, peaks, info);
+                                     r.n_chunks, cand_of, cand_best, grid->f_min, df, peaks, info);
   LEARN_CUDA(cudaGetLastError(), "refine finalize");
   return LSP_OK;
 }
@@ -1193,6 +1335,7 @@ lsp_status lsp_refine_windows(const double* t, const float* y, const int64_t* of
   if (st || n_obj == 0) return st;
   RefineLayout r;
   refine_layout(n_obj, total_nt, grid->n_f, &r);
+  if (ws_bytes < r.total) refine_layout(n_obj, total_nt, grid->n_f, &r, false);  // room for the direct kernels alone
   if (!workspace || ws_bytes < r.total || ((uintptr_t)workspace) % 256)
     return err_arg("refine workspace too small or misaligned");
   return refine_impl(t, y, offsets, n_obj, total_nt, grid, norm, classes, k_windows, window, stride, stop_power,
@@ -1215,7 +1358,7 @@ struct ProposeLayout {
 };
 
 void propose_layout(const Layers& L, int64_t n_obj, int64_t total_nt, int64_t n_f, int k_windows,
-                    ProposeLayout* p) {
+                    ProposeLayout* p, bool tf = true) {
   size_t off = 0;
   auto take = [&](size_t b) {
     size_t at = off;
@@ -1230,7 +1373,7 @@ void propose_layout(const Layers& L, int64_t n_obj, int64_t total_nt, int64_t n_
   for (int i = 0; i < 2; ++i) p->off_act[i] = take((size_t)rows * ld8(maxw) * sizeof(bf16));
   p->off_logits = take((size_t)rows * L.out[L.n - 1] * sizeof(float));
   p->off_cls = take((size_t)n_obj * k_windows * sizeof(int32_t));
-  refine_layout(n_obj, total_nt, n_f, &p->r);
+  refine_layout(n_obj, total_nt, n_f, &p->r, tf);
   p->off_refine = take(p->r.total);
   p->total = off;
 }
@@ -1289,6 +1432,7 @@ lsp_status lsp_propose_refine(const lsp_proposer* net, const double* t, const fl
   if (st || n_obj == 0) return st;
   ProposeLayout p;
   propose_layout(L, n_obj, total_nt, grid->n_f, net->k_windows, &p);
+  if (ws_bytes < p.total) propose_layout(L, n_obj, total_nt, grid->n_f, net->k_windows, &p, false);
   if (!workspace || ws_bytes < p.total || ((uintptr_t)workspace) % 256)
     return err_arg("propose-refine workspace too small or misaligned");
   cudaStream_t s = (cudaStream_t)stream;

@@ -110,9 +110,12 @@ __global__ void __launch_bounds__(kThreads, 2) transform_kernel(TransformParams 
     if (tid == 0) ticket = gridDim.x + atomicAdd(p.queue, 1u);
     const uint32_t chunk = item % n_chunks;
     const uint32_t orank = item / n_chunks;
-    const int64_t o = p.order_back ? (int64_t)p.order_back[-(int64_t)orank] : (int64_t)orank;
+    const int64_t o = p.order_back ? (int64_t)p.order_back[-(int64_t)orank]
+                                   : p.order ? (int64_t)p.order[orank] : (int64_t)orank;
     const ObjInfo oi = p.obj[o];
-    const int64_t kc0 = (int64_t)chunk * kTfBins;
+    // bins of this item lie in [kc0, kend): the run inside the grid, or the object's window
+    const int64_t kc0 = p.win_start ? (int64_t)p.win_start[o] : (int64_t)chunk * kTfBins;
+    const int64_t kend = p.win_start && kc0 + p.win_len < p.n_f ? kc0 + p.win_len : p.n_f;
     const uint32_t kc = (uint32_t)kc0 + kTfBins / 2;
     const int n = oi.flags ? 0 : oi.n;  // flagged objects: zero power
     const uint4* rec = reinterpret_cast<const uint4*>(p.rec + oi.begin);
@@ -268,7 +271,7 @@ __global__ void __launch_bounds__(kThreads, 2) transform_kernel(TransformParams 
     uint32_t bad = 0u;
 #pragma unroll
     for (int m = 0; m < 8; ++m) {
-      if (pv[m] < 0.0f && (int64_t)k0 + m < p.n_f) bad |= 1u << m;
+      if (pv[m] < 0.0f && (int64_t)k0 + m < kend) bad |= 1u << m;
       if (oi.flags) pv[m] = 0.0f;
     }
     if (oi.flags) bad = 0u;
@@ -276,9 +279,9 @@ __global__ void __launch_bounds__(kThreads, 2) transform_kernel(TransformParams 
       fix_ill_conditioned_gls<8>(pv, bad, k0, p.rec, oi);
     else
       fix_ill_conditioned<8>(pv, bad, k0, p.rec, oi.begin, oi.n, oi.norm_scale);
-    if (p.power_out) store_row<8>(p.power_out + o * p.n_f, (int64_t)k0, pv, p.n_f);
+    if (p.power_out) store_row<8>(p.power_out + o * p.n_f, (int64_t)k0, pv, kend);
     const int64_t res = o * (int64_t)n_chunks + chunk;
-    chunk_results_f32<8>(pv, k0, kc0, p.n_f, p.best + res, p.cand ? p.cand + res : nullptr, s_edge, red);
+    chunk_results_f32<8>(pv, k0, kc0, kend, p.best + res, p.cand ? p.cand + res : nullptr, s_edge, red);
   }
 
   // ---- one object, first maximum: the last CTA to finish writes the peak

@@ -193,3 +193,29 @@ def test_smaller_workspaces_take_smaller_paths(env, precision):
     assert torch.allclose(want, direct, rtol=0, atol=TOL if precision == "fp32" else 1e-10)
     with pytest.raises(lsp.LSPError):
         lsp.periodogram(t, y, g, precision=precision, workspace=torch.empty(1024, dtype=torch.uint8, device=dev))
+
+
+@pytest.mark.parametrize("norm", ["standard", "psd"])
+def test_refine_fallback_runs_equal_the_direct_full_grid(env, norm):
+    """The fallback looks for the maximum's run with the transform and takes the result from the direct kernel
+    on it: bit-equal to the direct full grid, also where many runs tie (regular sampling: the aliases of a
+    frequency have the same power in exact arithmetic, more runs than the fallback keeps) and on a ragged grid."""
+    lsp, torch, dev = env
+    from paper_2105_04006_gb300 import learned as L
+    counts = [2, 5, 39, 64, 300, 900]
+    t, y, off = _segments(counts, "uniform", 21)
+    reg = 60000.0 + np.arange(400.0)  # one observation a day: aliases at every whole cycle per day
+    t = np.concatenate([t, reg])
+    y = np.concatenate([y, np.sin(2 * np.pi * 0.3 * reg) + 0.1 * np.cos(2 * np.pi * 0.11 * reg)])
+    off = np.append(off, off[-1] + 400)
+    g = lsp.Grid(0.24, 12.0, 30_011)
+    args = (torch.tensor(t, device=dev), torch.tensor(y.astype(np.float32), device=dev), torch.tensor(off, device=dev))
+    n = off.size - 1
+    cls = torch.zeros((n, 1), dtype=torch.int32, device=dev)
+    code = 1 if norm == "standard" else 0
+    peaks, info = L.refine(*args, g, cls, 1, 1e30, 1e30, norm=code)  # every object falls back
+    _, want = lsp.batch(*args, g, norm=norm, k_reseed=16, freqs_per_thread=32, block_threads=64)
+    a, b = lsp.peaks_to_numpy(peaks), lsp.peaks_to_numpy(want)
+    for name in ("idx", "power", "flags"):
+        np.testing.assert_array_equal(a[name], b[name], err_msg=name)
+    assert (info.cpu().numpy() & 256).all()

@@ -78,7 +78,7 @@ struct Smem {
 };
 
 template <bool GLS>
-__global__ void __launch_bounds__(kThreads, 2) transform_kernel(TransformParams p) {
+__global__ void __launch_bounds__(kThreads, GLS ? 2 : 3) transform_kernel(TransformParams p) {
   using S = Smem<GLS>;
   constexpr int kW = GLS ? 4 : 2;  // grid planes: Z (re, im), with errors C, then W
   extern __shared__ __align__(128) unsigned char dyn_smem[];
@@ -91,9 +91,6 @@ __global__ void __launch_bounds__(kThreads, 2) transform_kernel(TransformParams 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t n_items = p.n_items_dev ? *p.n_items_dev : p.n_items;
   const uint32_t n_chunks = (uint32_t)p.n_chunks;
-  f2_t poly[9];  // of this lane's cell, lane & 7
-#pragma unroll
-  for (int d = 0; d < 9; ++d) poly[d] = dup_<f2_t>(__ldg(&kTfPoly[d * 8 + (lane & 7)]));
   auto clear_grid = [&]() {
     int4* g4 = reinterpret_cast<int4*>(plane);
 #pragma unroll
@@ -142,6 +139,11 @@ __global__ void __launch_bounds__(kThreads, 2) transform_kernel(TransformParams 
     // time: a lane each for the phase, then an octet of lanes each for the 8
     // cells
     {
+      // window coefficients of this lane's cell (not kept across the transform:
+      // their 18 registers are what lets three CTAs share an SM)
+      f2_t poly[9];
+#pragma unroll
+      for (int d = 0; d < 9; ++d) poly[d] = dup_<f2_t>(__ldg(&kTfPoly[d * 8 + (lane & 7)]));
       const int j1 = (int)((int64_t)n * (warp + 1) / kWarps);
       unsigned char* const mine = stage + (size_t)warp * 32 * S::kStage;
       for (int jb = (int)((int64_t)n * warp / kWarps); jb < j1; jb += 32) {

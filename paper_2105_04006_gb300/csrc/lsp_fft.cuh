@@ -55,8 +55,19 @@ __device__ __forceinline__ dd add_(dd a, dd b) {
   e = __fadd_rn(e, __fadd_rn(a.lo, b.lo));
   return dd_fast(s, e);
 }
+// A sum whose two parts may overlap by a few bits: exact hi, lo not yet folded
+// in.  Enough where the next operation is another sum.
+__device__ __forceinline__ dd add_lazy_(dd a, dd b) {
+  const float s = __fadd_rn(a.hi, b.hi);
+  const float t = __fsub_rn(s, a.hi);
+  const float e = __fadd_rn(__fsub_rn(a.hi, __fsub_rn(s, t)), __fsub_rn(b.hi, t));
+  return {s, __fadd_rn(e, __fadd_rn(a.lo, b.lo))};
+}
+template <typename T> __device__ __forceinline__ T add_lazy_(T a, T b) { return add_(a, b); }
 __device__ __forceinline__ dd neg1_(dd a) { return {-a.hi, -a.lo}; }
 __device__ __forceinline__ dd sub_(dd a, dd b) { return add_(a, neg1_(b)); }
+__device__ __forceinline__ dd sub_lazy_(dd a, dd b) { return add_lazy_(a, neg1_(b)); }
+template <typename T> __device__ __forceinline__ T sub_lazy_(T a, T b) { return sub_(a, b); }
 __device__ __forceinline__ dd mul_(dd a, dd b) {
   const float p = __fmul_rn(a.hi, b.hi);
   float e = __fmaf_rn(a.hi, b.hi, -p);
@@ -109,7 +120,8 @@ __device__ __forceinline__ Cx<dd> cmul(Cx<dd> a, float4 w) {
 // In-place transform of 4 points with e^{+2 pi i jk/4}.
 template <typename T>
 __device__ __forceinline__ void dft4(Cx<T>& x0, Cx<T>& x1, Cx<T>& x2, Cx<T>& x3) {
-  const Cx<T> a = x0 + x2, b = x0 - x2, c = x1 + x3, d = x1 - x3;
+  const Cx<T> a{add_lazy_(x0.re, x2.re), add_lazy_(x0.im, x2.im)}, b{sub_lazy_(x0.re, x2.re), sub_lazy_(x0.im, x2.im)};
+  const Cx<T> c{add_lazy_(x1.re, x3.re), add_lazy_(x1.im, x3.im)}, d{sub_lazy_(x1.re, x3.re), sub_lazy_(x1.im, x3.im)};
   x0 = a + c;
   x1 = add_i(b, d);
   x2 = a - c;
@@ -158,47 +170,87 @@ __device__ __forceinline__ Cx<T> get(const Cx<T>* buf, int i) {
   return v;
 }
 
+// The first two radix-16 passes of a tile of 4096 values and the exchanges
+// after them: thread tid enters with the values of indices 16 R a + u, u =
+// tid / B, of its column (see the callers) at x[a] and leaves with those of
+// its (p, r = tid & 15), p = tid >> 4, in the order e of the last pass.
+// tw_a(p), tw_b(r): the twiddles after each pass.  The second exchange stays
+// within the 16 threads of one p, in the 256 words that only they read in the
+// first one, so it needs no barrier of the whole CTA.
+//
+// ROLL: the two passes are one loop body.  Unrolled, a two-float transform is
+// 130 KB of instructions, more than the cache that feeds the SM holds (FP64
+// batch, N_t 275, per run and SM: 114 500 -> 110 700 clocks rolled).
+template <bool ROLL, typename T, typename TwA, typename TwB>
+__device__ __forceinline__ void fft_two_passes(Cx<T> (&x)[16], Cx<T>* buf, int tid, TwA&& tw_a, TwB&& tw_b) {
+  const int e0 = tid & 15;
+  Cx<T>* const own = buf + (tid >> 4) * 256;
+  if constexpr (ROLL) {
+#pragma unroll 1
+    for (int pass = 0; pass < 2; ++pass) {
+      dft16(x);
+#pragma unroll
+      for (int p = 1; p < 16; ++p) {
+        const int q = 4 * (p & 3) + (p >> 2);
+        x[q] = cmul(x[q], pass ? tw_b(p) : tw_a(p));
+      }
+      // first exchange: word 256 p + tid, read at own + 16 c + e0; second:
+      // own + 16 r + (e0 ^ r), read at own + 16 e0 + (e ^ e0)
+      Cx<T>* const to = pass ? own : buf + tid;
+      const int step = pass ? 16 : 256, mix = pass ? 15 : 0;
+      if (pass) __syncwarp(); else __syncthreads();
+#pragma unroll
+      for (int p = 0; p < 16; ++p) put(to, p * step + ((e0 ^ p) & mix), x[4 * (p & 3) + (p >> 2)]);
+      if (pass) __syncwarp(); else __syncthreads();
+      const Cx<T>* const from = pass ? own + 16 * e0 : own + e0;
+      const int stride = pass ? 1 : 16, flip = pass ? e0 : 0;
+#pragma unroll
+      for (int c = 0; c < 16; ++c) x[c] = get(from, (c * stride) ^ flip);
+    }
+  } else {
+    dft16(x);
+#pragma unroll
+    for (int p = 1; p < 16; ++p) {
+      const int q = 4 * (p & 3) + (p >> 2);
+      x[q] = cmul(x[q], tw_a(p));
+    }
+    __syncthreads();  // every thread has read its cells
+#pragma unroll
+    for (int p = 0; p < 16; ++p) put(buf, p * 256 + tid, x[4 * (p & 3) + (p >> 2)]);
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < 16; ++c) x[c] = get(own, 16 * c + e0);
+    dft16(x);
+#pragma unroll
+    for (int r = 1; r < 16; ++r) {
+      const int q = 4 * (r & 3) + (r >> 2);
+      x[q] = cmul(x[q], tw_b(r));
+    }
+    __syncwarp();
+    // word (r, d) at 16 r + (d ^ r): the lanes of either the writing order (d
+    // runs) or the reading order (r runs) fall on distinct banks
+#pragma unroll
+    for (int r = 0; r < 16; ++r) put(own, 16 * r + (e0 ^ r), x[4 * (r & 3) + (r >> 2)]);
+    __syncwarp();
+#pragma unroll
+    for (int e = 0; e < 16; ++e) x[e] = get(own, 16 * e0 + (e ^ e0));
+  }
+}
+
 // The 4096-point transform of the CTA: on entry thread b holds cells
 // 256 a + b (a = 0 .. 15); on return, with p = tid >> 4 and r = tid & 15,
 // out[s] holds the value at offset p + 16 r + 256 s - 1024 from the run's
 // centre, s = 0 .. 7.  buf: 4096 complex words, free once every thread has
 // passed the first barrier here; free again only after a barrier of the
-// caller.  The second exchange stays within the 16 threads of one p, in the
-// 256 words that only they read in the first one, so it needs no barrier of
-// the whole CTA.
+// caller.
 // tw1[256 (p - 1) + b] = e^{2 pi i p b / 4096}, tw2[16 (r - 1) + d] = e^{2 pi i r d / 256}.
 template <typename T>
 __device__ __forceinline__ void fft4096(Cx<T> (&x)[16], Cx<T>* buf, const typename Twiddle<T>::type* __restrict__ tw1,
                                         const typename Twiddle<T>::type* __restrict__ tw2, Cx<T> (&out)[8]) {
-  const int tid = threadIdx.x;
-  dft16(x);
-#pragma unroll
-  for (int p = 1; p < 16; ++p) {
-    const int q = 4 * (p & 3) + (p >> 2);
-    x[q] = cmul(x[q], __ldg(&tw1[(p - 1) * 256 + tid]));
-  }
-  __syncthreads();  // every thread has read its cells
-#pragma unroll
-  for (int p = 0; p < 16; ++p) put(buf, p * 256 + tid, x[4 * (p & 3) + (p >> 2)]);
-  __syncthreads();
-  Cx<T>* const own = buf + (tid >> 4) * 256;
-  const int d = tid & 15;
-#pragma unroll
-  for (int c = 0; c < 16; ++c) x[c] = get(own, 16 * c + d);
-  dft16(x);
-#pragma unroll
-  for (int r = 1; r < 16; ++r) {
-    const int q = 4 * (r & 3) + (r >> 2);
-    x[q] = cmul(x[q], __ldg(&tw2[(r - 1) * 16 + d]));
-  }
-  __syncwarp();
-  // word (r, d) at 16 r + (d ^ r): the lanes of either the writing order (d
-  // runs) or the reading order (r runs) fall on distinct banks
-#pragma unroll
-  for (int r = 0; r < 16; ++r) put(own, 16 * r + (d ^ r), x[4 * (r & 3) + (r >> 2)]);
-  __syncwarp();
-#pragma unroll
-  for (int e = 0; e < 16; ++e) x[e] = get(own, 16 * d + (e ^ d));
+  const int tid = threadIdx.x, e0 = tid & 15;
+  fft_two_passes<std::is_same<T, dd>::value>(
+      x, buf, tid, [&](int p) { return __ldg(&tw1[(p - 1) * 256 + tid]); },
+      [&](int r) { return __ldg(&tw2[(r - 1) * 16 + e0]); });
   dft16_first(x);
 #pragma unroll
   for (int k1 = 0; k1 < 4; ++k1) {

@@ -212,35 +212,10 @@ __device__ __forceinline__ constexpr int slot(int s, int col) {
 template <typename T, int R>
 __device__ __forceinline__ void fft_tile(Cx<T> (&x)[16], Cx<T>* buf, int tid) {
   constexpr int B = 16 / R;
-  dft16(x);
-  const int u = tid / B;
-#pragma unroll
-  for (int p = 1; p < 16; ++p) {
-    const int q = 4 * (p & 3) + (p >> 2);
-    x[q] = cmul(x[q], Tables<T>::unit((uint32_t)(p * u * B)));
-  }
-  __syncthreads();
-#pragma unroll
-  for (int p = 0; p < 16; ++p) put(buf, p * 256 + tid, x[4 * (p & 3) + (p >> 2)]);
-  __syncthreads();
-  Cx<T>* const own = buf + (tid >> 4) * 256;
-  const int e0 = tid & 15, d = e0 / B;
-#pragma unroll
-  for (int c = 0; c < 16; ++c) x[c] = get(own, 16 * c + e0);
-  dft16(x);
-  if constexpr (R > 1) {
-#pragma unroll
-    for (int r = 1; r < 16; ++r) {
-      const int q = 4 * (r & 3) + (r >> 2);
-      x[q] = cmul(x[q], Tables<T>::unit((uint32_t)(r * d * (256 / R))));
-    }
-  }
-  __syncwarp();
-#pragma unroll
-  for (int r = 0; r < 16; ++r) put(own, 16 * r + (e0 ^ r), x[4 * (r & 3) + (r >> 2)]);
-  __syncwarp();
-#pragma unroll
-  for (int e = 0; e < 16; ++e) x[e] = get(own, 16 * e0 + (e ^ e0));  // e = d B + col
+  const int u = tid / B, d = (tid & 15) / B;  // afterwards e = d B + col
+  fft_two_passes<false>(  // run once per CTA: rolled, the loop's spills cost more (195 -> 202 us)
+      x, buf, tid, [&](int p) { return Tables<T>::unit((uint32_t)(p * u * B)); },
+      [&](int r) { return Tables<T>::unit((uint32_t)(r * d * (256 / R)) & 4095u); });
   if constexpr (R == 2) {
 #pragma unroll
     for (int c = 0; c < 8; ++c) {

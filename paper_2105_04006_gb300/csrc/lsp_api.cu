@@ -99,13 +99,14 @@ constexpr int kTfMinObs64 = 8;
 // whole grid 30 + N_f / 12500.  Measured, runs | whole grid: N_t 3000, N_f 1e5
 // 41 | 43; N_t 1e4, N_f 1e5 78 | 43; N_t 3000, N_f 4e5 49 | 65; N_t 1e5, N_f 1e6
 // 1480 | 127.  In FP64 the whole grid is always the faster (N_t 1000, N_f 1e5:
-// 208 | 88; the direct kernel takes 1400).
+// 200 | 82; the direct kernel takes 1400).
 bool long_is_faster(int64_t n_t, int64_t n_f, int64_t runs, int64_t slots) {
   const double waves = (double)((runs + slots - 1) / slots);
   return waves * (12.0 + (double)n_t / 150.0) > 30.0 + (double)n_f / 12500.0;
 }
 // The paths a call may take, by the workspace they need: everything; without
-// the whole-grid transform; the direct kernels alone.
+// the whole-grid transform and with fewer FP64 run CTAs; the direct kernels
+// alone.
 constexpr int kLevels = 3;
 
 lsp_status check_grid(const lsp_grid* g) {
@@ -228,6 +229,18 @@ lsp_status resolve(int64_t n_obj, int64_t total_nt, const lsp_grid* g, const lsp
   l.n_res_chunks = split > 1 ? (int32_t)((l.n_f + cchunk - 1) / cchunk) : l.n_chunks;
   l.n_items = n_obj * (int64_t)l.n_chunks * split;
 
+  if (l.tf) {
+    int tb = transform_blocks_per_sm(l.prec, l.gls);
+    if (tb <= 0) {
+      cudaGetLastError();
+      tb = 1;
+    }
+    int64_t tg = (int64_t)tb * current_sm_count();
+    if (tg > l.n_items) tg = l.n_items;
+    if (l.prec && level > 0 && tg > 64) tg = 64;  // 8 MB of cells (kTf64CellBytes per CTA) instead of 40
+    l.tf_grid = (int)(tg < 1 ? 1 : tg);
+  }
+
   size_t off = 0;
   auto take = [&](size_t bytes) {
     size_t at = off;
@@ -244,7 +257,7 @@ lsp_status resolve(int64_t n_obj, int64_t total_nt, const lsp_grid* g, const lsp
   // partial sums: 4 per frequency, the generalized periodogram's 6 in slots of 8
   l.off_part = take(split > 1 ? (size_t)split * l.n_f * (gls ? 8 : 4) * (l.prec ? 8 : 4) : 0);
   l.off_stats = take(n_obj == 1 ? stats_slices_bytes(total_nt) : 0);
-  l.off_cells = take(l.lng ? l.lp.cell_bytes : 0);
+  l.off_cells = take(l.lng ? l.lp.cell_bytes : l.tf && l.prec ? (size_t)l.tf_grid * kTf64CellBytes : 0);
   l.off_t = take(l.lng ? l.lp.t_bytes : 0);
   l.off_row = take(l.lng ? l.lp.row_bytes : 0);
   l.total = off;
@@ -257,16 +270,6 @@ lsp_status resolve(int64_t n_obj, int64_t total_nt, const lsp_grid* g, const lsp
   int64_t grid = (int64_t)bps * current_sm_count();
   if (grid > l.n_items) grid = l.n_items;
   l.grid = (int)(grid < 1 ? 1 : grid);
-  if (l.tf) {
-    int tb = transform_blocks_per_sm(l.prec, l.gls);
-    if (tb <= 0) {
-      cudaGetLastError();
-      tb = 1;
-    }
-    int64_t tg = (int64_t)tb * current_sm_count();
-    if (tg > l.n_items) tg = l.n_items;
-    l.tf_grid = (int)(tg < 1 ? 1 : tg);
-  }
   return LSP_OK;
 }
 
@@ -350,6 +353,7 @@ lsp_status run(const Layout& L, const double* t, const void* y, const int64_t* o
       fill(tp);
       tp.rec = (const RecF64*)rec;
       tp.power_out = (double*)power_out;
+      tp.cells = (long long*)(ws + L.off_cells);
       LSP_CUDA(launch_transform64(tp, L.tf_grid, st), "transform kernel");
     } else {
       TransformParams tp;

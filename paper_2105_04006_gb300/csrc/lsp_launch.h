@@ -103,6 +103,7 @@ size_t main_dyn_smem(int prec, int fpt, int threads, int top);
 // a nonuniform FFT; FP32 (standard and generalized periodogram) and FP64
 // (standard).
 constexpr int kTfBins = 2048;
+constexpr size_t kTf64CellBytes = 4 * 4096 * 8;
 template <typename Rec, typename Real>
 struct TransformParamsOf {
   const Rec* rec;
@@ -116,6 +117,7 @@ struct TransformParamsOf {
   const uint32_t* n_items_dev;  // device item count (overrides n_items)
   uint32_t n_items;
   int32_t n_chunks;      // runs per object
+  long long* cells = nullptr;  // FP64: kTf64CellBytes per CTA
   int32_t have_scale;    // the records kernel left the scales (batches)
   // FP32: per-object windows instead of runs from 0 (n_chunks = 1, one item
   // per object): bins [win_start[o], win_start[o] + win_len) of the grid

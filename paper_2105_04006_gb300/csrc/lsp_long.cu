@@ -20,8 +20,8 @@
 //           runs' maxima, and (first maximum) the peak.
 //
 // Measured (GB300, prepared plans): 1e5 observations on 1e6 bins FP32 127 us
-// (direct 23 400, run by run 1480); FP64 1000 on 1e5 88 us (direct 1404, run by
-// run 208), 5e4 on 5e5 195 us (direct 300 000).  Up to N_f = 1e5 the FP64 time
+// (direct 23 400, run by run 1480); FP64 1000 on 1e5 82 us (direct 1404), 5e4 on
+// 5e5 175 us (direct 300 000).  Up to N_f = 1e5 the FP64 time
 // is the latency of the two passes' dependent two-float chains; at 1e6 bins
 // the FP32 time is the 230 MB that the grid and t move through L2.
 //
@@ -47,20 +47,6 @@ namespace {
 constexpr int kThreads = 256;
 
 // ------------------------------------------------------------------- spread
-// Magnitudes are scaled by 2^-e, sum y^2 <= 2^2e: then a cell of Z is at most
-// sum |y| <= sqrt(N) <= 2^((count_bits + 1) / 2) and one of W at most N.
-__device__ __forceinline__ int y_exponent(double sum_y2) {
-  return (((int)(__double_as_longlong(sum_y2) >> 52) & 0x7ff) - 1023) / 2 + 1;
-}
-__device__ __forceinline__ double pow2(int e) { return __longlong_as_double((long long)(1023 + e) << 52); }
-__device__ __forceinline__ int count_bits(int n) { return 32 - __clz(n); }  // n < 2^count_bits
-__device__ __forceinline__ int z_bits(int n) { return 62 - (count_bits(n) + 1) / 2; }  // cells are in units of 2^-bits
-__device__ __forceinline__ int w_bits(int n) { return 62 - count_bits(n); }
-
-__device__ __forceinline__ void add_cell(long long* cell, long long v) {
-  atomicAdd(reinterpret_cast<unsigned long long*>(cell), (unsigned long long)v);
-}
-
 __global__ void __launch_bounds__(kThreads) spread_f32(const RecF32* __restrict__ rec, const ObjInfo* __restrict__ obj,
                                                        uint32_t kc, int lg, long long* __restrict__ cells) {
   const ObjInfo oi = obj[0];
@@ -104,70 +90,28 @@ __global__ void __launch_bounds__(kThreads) spread_f32(const RecF32* __restrict_
     float wz, ww;
     f2_unpack(w2, wz, ww);
     if (j0 + i < n) {
-      add_cell(cells + 4 * (int64_t)lz, __float2ll_rn(wz * a0));
-      add_cell(cells + 4 * (int64_t)lz + 1, __float2ll_rn(wz * a1));
-      add_cell(cells + 4 * (int64_t)lw + 2, __float2ll_rn(ww * a2));
-      add_cell(cells + 4 * (int64_t)lw + 3, __float2ll_rn(ww * a3));
+      add_cell(cells + 4 * (int64_t)lz, fixed_of(wz * a0));
+      add_cell(cells + 4 * (int64_t)lz + 1, fixed_of(wz * a1));
+      add_cell(cells + 4 * (int64_t)lw + 2, fixed_of(ww * a2));
+      add_cell(cells + 4 * (int64_t)lw + 3, fixed_of(ww * a3));
     }
   }
-}
-
-// A two-float number times 2^s as a 64-bit integer (|v| 2^s < 2^63): hi's part
-// is exact, lo's is rounded.
-__device__ __forceinline__ long long fixed_of(dd v, float two_s) {
-  return __float2ll_rn(v.hi * two_s) + __float2ll_rn(v.lo * two_s);
 }
 
 __global__ void __launch_bounds__(kThreads) spread_f64(const RecF64* __restrict__ rec, const ObjInfo* __restrict__ obj,
                                                        uint64_t kc, int lg, long long* __restrict__ cells) {
   const ObjInfo oi = obj[0];
   const int n = oi.flags ? 0 : oi.n;
-  const int lane = threadIdx.x & 31, r = lane & 15;
+  const int lane = threadIdx.x & 31;
   const int j0 = (blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5)) * 32;
   if (j0 >= n) return;
-  const double y_sc = pow2(-y_exponent(oi.sum_y2));
   const float one[2] = {(float)pow2(z_bits(n)), (float)pow2(w_bits(n))};
-  const uint32_t mask = (1u << lg) - 1u;
-  dd a[4];
-  dd v[2];
-  uint32_t cell[2] = {0u, 0u}, sub[2] = {0u, 0u};
-#pragma unroll
-  for (int q = 0; q < 4; ++q) a[q] = dd{0.0f, 0.0f};
-  v[0] = v[1] = dd{0.0f, 0.0f};
-  const int j = j0 + lane;
-  if (j < n) {
-    const RecF64 q = rec[oi.begin + j];
-    double c, s;
-    seed_sincos_f64(q.a + kc * q.b, c, s);
-    const double ys = q.y * y_sc;
-    a[0] = dd_of(ys * c);
-    a[1] = dd_of(ys * s);
-    a[2] = dd_of((c - s) * (c + s));
-    a[3] = dd_of(2.0 * c * s);
-#pragma unroll
-    for (int t = 0; t < 2; ++t) {  // place of Z (b) and W (2 b): cell, 6 bits of sub-interval, 24 + 22 of place
-      const uint64_t b = q.b << t, f = b << lg;
-      cell[t] = (uint32_t)(b >> (64 - lg)) - 7u;
-      sub[t] = (uint32_t)(f >> 58);
-      const float hi = (float)((uint32_t)(f >> 34) & 0xffffffu) * 5.9604644775390625e-8f;
-      const float lo = (float)((uint32_t)(f >> 12) & 0x3fffffu) * 1.4210854715202004e-14f;
-      v[t] = dd{hi - 0.5f, lo};
-    }
-  }
-  auto bcast = [&](dd x, int i) { return dd{__shfl_sync(0xffffffffu, x.hi, i), __shfl_sync(0xffffffffu, x.lo, i)}; };
-#pragma unroll 1
-  for (int i = lane >> 4; i < 32; i += 2) {
-#pragma unroll
-    for (int t = 0; t < 2; ++t) {
-      const dd w = window(__shfl_sync(0xffffffffu, sub[t], i), bcast(v[t], i), r);
-      const uint32_t l = (__shfl_sync(0xffffffffu, cell[t], i) + (uint32_t)r) & mask;
-      const dd re = mul_(w, bcast(a[2 * t], i)), im = mul_(w, bcast(a[2 * t + 1], i));
-      if (j0 + i < n) {
-        add_cell(cells + 4 * (int64_t)l + 2 * t, fixed_of(re, one[t]));
-        add_cell(cells + 4 * (int64_t)l + 2 * t + 1, fixed_of(im, one[t]));
-      }
-    }
-  }
+  const int j = j0 + lane < n ? j0 + lane : j0;
+  const ObsD o = obs_of(rec[oi.begin + j], kc, lg, pow2(-y_exponent(oi.sum_y2)));
+  spread_warp(o, min(32, n - j0), (1u << lg) - 1u, one, [&](int t, uint32_t l, long long re, long long im) {
+    add_cell(cells + 4 * (int64_t)l + 2 * t, re);
+    add_cell(cells + 4 * (int64_t)l + 2 * t + 1, im);
+  });
 }
 
 // ------------------------------------------------------------------- passes
@@ -213,7 +157,7 @@ template <typename T, int R>
 __device__ __forceinline__ void fft_tile(Cx<T> (&x)[16], Cx<T>* buf, int tid) {
   constexpr int B = 16 / R;
   const int u = tid / B, d = (tid & 15) / B;  // afterwards e = d B + col
-  fft_two_passes<false>(  // run once per CTA: rolled, the loop's spills cost more (195 -> 202 us)
+  fft_two_passes<false>(  // run once per CTA: rolled, the loop's spills cost more (5e4 on 5e5: 195 -> 202 us)
       x, buf, tid, [&](int p) { return Tables<T>::unit((uint32_t)(p * u * B)); },
       [&](int r) { return Tables<T>::unit((uint32_t)(r * d * (256 / R)) & 4095u); });
   if constexpr (R == 2) {
@@ -237,13 +181,7 @@ __device__ __forceinline__ void fft_tile(Cx<T> (&x)[16], Cx<T>* buf, int tid) {
 __device__ __forceinline__ Cx<f2_t> load_cell(const long long* cells, int64_t i, int, f2_t) {
   const longlong2* q = reinterpret_cast<const longlong2*>(cells + 4 * i);
   const longlong2 z = __ldcs(q), w = __ldcs(q + 1);
-  return {f2_pack(__ll2float_rn(z.x), __ll2float_rn(w.x)), f2_pack(__ll2float_rn(z.y), __ll2float_rn(w.y))};
-}
-// An integer of up to 62 bits as a two-float number: its top half exactly in
-// one float where it has 24 bits or fewer, the remainder in the other.
-__device__ __forceinline__ dd dd_of_int(long long v) {
-  const float h = __ll2float_rn(v);
-  return dd{h, __ll2float_rn(v - __float2ll_rn(h))};
+  return {f2_pack(float_of_int(z.x), float_of_int(w.x)), f2_pack(float_of_int(z.y), float_of_int(w.y))};
 }
 __device__ __forceinline__ Cx<dd> load_cell(const long long* cells, int64_t i, int half, dd) {
   const longlong2 z = __ldcs(reinterpret_cast<const longlong2*>(cells + 4 * i) + half);

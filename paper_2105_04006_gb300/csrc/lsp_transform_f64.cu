@@ -12,18 +12,21 @@
 // sums from the exact phases.  Both are below the rounding that the FP64
 // pairwise kernel's chains of 16 accumulate.
 //
-// Measured (GB300): 200 survey light curves (N_t 50 .. 500) on 1e5 bins 3.3 ms
-// against 64 ms with the direct kernel; N_t 8 0.64 | 1.34, 12 0.65 | 1.62, 64
-// 0.73 | 5.3 ms (60 objects).
+// Measured (GB300): 200 survey light curves (N_t 50 .. 500) on 1e5 bins 2.6 ms
+// against 64 ms with the direct kernel; a run on one SM 60 000 clocks plus 89
+// an observation; 60 objects of N_t 8 0.61 | 1.34, 12 0.59 | 1.62, 64 0.63 |
+// 5.3 ms (transform | direct).  Bound by instruction issue (57 %, two CTAs).
 //
 // Differences from the FP32 kernel:
-//   - Z and W one after the other through one grid of two-float cells; Z's
-//     outputs wait in shared memory;
-//   - cells are floating-point, so the order of the adds matters: tiles of
-//     256 observations are sorted by their first cell (rank by counting, ties
-//     by index) and every cell gathers its own contributions in that order.
-//     Repeats are bit-identical, and clustered observations cost no more than
-//     spread-out ones as long as they fill more than a few cells;
+//   - cells are 64-bit fixed point (a cell of W is at most N, one of Z at most
+//     sqrt(N sum y^2)).  Shared memory has no 64-bit add of its own, so each
+//     CTA's 128 KB of cells lie in global memory (in L2: 40 MB for all CTAs)
+//     and take integer reductions there; any time order and any clustering
+//     run at the same speed and repeats are bit-identical.  (Gathered per cell
+//     from sorted observations in shared memory instead, the spread took 190
+//     clocks an observation, lanes waiting for the fullest cell.)
+//   - Z and W are transformed one after the other; Z's outputs wait in shared
+//     memory;
 //   - window values: 64 sub-intervals per cell, degree 5, the two leading
 //     coefficients (below 2^-27) in single floats;
 //   - magnitudes are scaled by a power of two (|y|^2 <= sum y^2) into the
@@ -45,32 +48,21 @@ namespace {
 
 constexpr int kM = 4096;
 constexpr int kThreads = 256;
-constexpr int kTile = 256;  // observations staged at a time
-static_assert(kTfBins == kM / 2 && kTfBins == kThreads * 8, "run length");
+constexpr int kWarps = kThreads / 32;
+constexpr int kLog2M = 12;
+static_assert(kTfBins == kM / 2 && kTfBins == kThreads * 8 && kM == 1 << kLog2M, "run length");
 
-struct __align__(16) StagedObs {
-  dd re, im;      // amplitude times e^{i phase}
-  dd v;           // place inside the sub-interval, -1/2 .. 1/2
-  uint32_t sub;   // sub-interval
-  int32_t cell;   // first cell of the window
-};
-static_assert(sizeof(StagedObs) == 32, "two 16-byte words");
-
-constexpr size_t kGridBytes = (size_t)kM * sizeof(Cx<dd>);       // also: powers of the run
-constexpr size_t kZBytes = (size_t)kTfBins * sizeof(Cx<dd>);     // Z's outputs
-constexpr size_t kStageBytes = (size_t)kTile * sizeof(StagedObs);
-constexpr size_t kKeyBytes = (size_t)kTile * 4;                  // sort keys
-constexpr size_t kStartBytes = (size_t)(kM / 16) * 4;            // first observation of each 16 cells
-constexpr size_t kSmem = kGridBytes + kZBytes + kStageBytes + kKeyBytes + kStartBytes;
-static_assert(kM / 16 == kThreads, "one start per thread");
+constexpr size_t kBufBytes = (size_t)kM * sizeof(Cx<dd>);     // exchange buffer; later the powers of the run
+constexpr size_t kZBytes = (size_t)kTfBins * sizeof(Cx<dd>);  // Z's outputs
+constexpr size_t kSmem = kBufBytes + kZBytes;
+static_assert(kTf64CellBytes == 4 * kM * sizeof(long long), "four planes of cells per CTA");
 
 __global__ void __launch_bounds__(kThreads, 2) transform64_kernel(TransformParams64 p) {
   extern __shared__ __align__(128) unsigned char dyn_smem[];
-  Cx<dd>* const grid = reinterpret_cast<Cx<dd>*>(dyn_smem);
-  Cx<dd>* const s_z = reinterpret_cast<Cx<dd>*>(dyn_smem + kGridBytes);
-  StagedObs* const stage = reinterpret_cast<StagedObs*>(dyn_smem + kGridBytes + kZBytes);
-  uint32_t* const s_key = reinterpret_cast<uint32_t*>(dyn_smem + kGridBytes + kZBytes + kStageBytes);
-  int32_t* const s_start = reinterpret_cast<int32_t*>(s_key + kTile);
+  Cx<dd>* const buf = reinterpret_cast<Cx<dd>*>(dyn_smem);
+  Cx<dd>* const s_z = reinterpret_cast<Cx<dd>*>(dyn_smem + kBufBytes);
+  // this CTA's cells: planes Z re, Z im, W re, W im; zero between runs
+  long long* const cells = p.cells + (int64_t)blockIdx.x * (4 * kM);
   double* const pw = reinterpret_cast<double*>(dyn_smem);
   __shared__ double red_p[32];
   __shared__ int64_t red_k[32];
@@ -78,6 +70,9 @@ __global__ void __launch_bounds__(kThreads, 2) transform64_kernel(TransformParam
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t n_items = p.n_items_dev ? *p.n_items_dev : p.n_items;
   const uint32_t n_chunks = (uint32_t)p.n_chunks;
+
+  for (int i = tid; i < 4 * kM / 2; i += kThreads) reinterpret_cast<longlong2*>(cells)[i] = make_longlong2(0, 0);
+  __threadfence();
 
   uint32_t ticket = blockIdx.x;  // first item static, then one ticket ahead (as in main_f32_packed_body)
   for (;;) {
@@ -95,88 +90,33 @@ __global__ void __launch_bounds__(kThreads, 2) transform64_kernel(TransformParam
     const int n = oi.flags ? 0 : oi.n;  // flagged objects: zero power
     const RecF64* rec = p.rec + oi.begin;
     // 2^-e bounds the magnitudes by 1: |y| <= sqrt(sum y^2) < 2^e
-    const int e = (((int)(__double_as_longlong(oi.sum_y2) >> 52) & 0x7ff) - 1023) / 2 + 1;
-    const double y_sc = __longlong_as_double((long long)(1023 - e) << 52);
+    const double y_sc = pow2(-y_exponent(oi.sum_y2));
+    {  // spread: each warp takes an eighth of the observations
+      const float one[2] = {(float)pow2(z_bits(n)), (float)pow2(w_bits(n))};
+      const int j1 = (int)((int64_t)n * (warp + 1) / kWarps);
+      for (int jb = (int)((int64_t)n * warp / kWarps); jb < j1; jb += 32) {
+        const ObsD ob = obs_of(rec[jb + lane < j1 ? jb + lane : jb], kc, kLog2M, y_sc);
+        spread_warp(ob, min(32, j1 - jb), kM - 1, one, [&](int t, uint32_t l, long long re, long long im) {
+          add_cell(cells + (2 * t) * kM + l, re);
+          add_cell(cells + (2 * t + 1) * kM + l, im);
+        });
+      }
+    }
+    __threadfence();
+    __syncthreads();  // every reduction has reached L2
+    const float z_inv = (float)pow2(-z_bits(n)), w_inv = (float)pow2(-w_bits(n));
 
 #pragma unroll 1
     for (int tr = 0; tr < 2; ++tr) {  // Z, then W
-      {
-        uint4* g4 = reinterpret_cast<uint4*>(grid);
-#pragma unroll
-        for (int i = 0; i < kM / kThreads; ++i) g4[tid + i * kThreads] = make_uint4(0u, 0u, 0u, 0u);
-      }
-      for (int ts = 0; ts < n; ts += kTile) {
-        const int j = ts + tid, nt = min(kTile, n - ts);
-        StagedObs st;
-        uint32_t key = 0xffffffffu;
-        if (j < n) {
-          const RecF64 r = rec[j];
-          const uint64_t ph = r.a + kc * r.b, b = tr ? r.b << 1 : r.b;
-          double c, s;
-          seed_sincos_f64(tr ? ph << 1 : ph, c, s);
-          if (!tr) {
-            const double ys = r.y * y_sc;
-            c *= ys;
-            s *= ys;
-          }
-          st.re = dd_of(c);
-          st.im = dd_of(s);
-          // 12 bits of cell, 6 of sub-interval, 46 of place: 24 and 22 exactly in two floats
-          st.cell = (int32_t)(((uint32_t)(b >> 52) - 7u) & (kM - 1));
-          st.sub = (uint32_t)(b >> 46) & 63u;
-          const float hi = (float)((uint32_t)(b >> 22) & 0xffffffu) * 5.9604644775390625e-8f;  // 2^-24
-          const float lo = (float)((uint32_t)b & 0x3fffffu) * 1.4210854715202004e-14f;         // 2^-46
-          st.v = dd{hi - 0.5f, lo};
-          key = (uint32_t)st.cell << 8 | (uint32_t)tid;
-        }
-        s_key[tid] = key;
-        __syncthreads();  // keys; on the first tile also: the grid is clear
-        int rank = 0;
-        for (int i = 0; i < (nt + 3) / 4; ++i) {
-          const uint4 k = reinterpret_cast<const uint4*>(s_key)[i];
-          rank += (int)(k.x < key) + (int)(k.y < key) + (int)(k.z < key) + (int)(k.w < key);
-        }
-        if (j < n) stage[rank] = st;
-        __syncthreads();
-        {  // first sorted observation whose cell is at least 16 tid
-          int lo = 0, hi = nt;
-          while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (stage[mid].cell < 16 * tid) lo = mid + 1;
-            else hi = mid;
-          }
-          s_start[tid] = lo;
-        }
-        __syncthreads();
-#pragma unroll 1
-        for (int a = 0; a < kM / kThreads; ++a) {
-          const int l = kThreads * a + tid;  // contributions: first cells l - 15 .. l, around the end
-          Cx<dd> acc{{0.0f, 0.0f}, {0.0f, 0.0f}};
-          bool any = false;
-          auto add = [&](int i) {
-            const StagedObs q = stage[i];
-            const dd w = window(q.sub, q.v, (l - q.cell) & (kM - 1));
-            acc = acc + Cx<dd>{mul_(w, q.re), mul_(w, q.im)};
-            any = true;
-          };
-          const int from = l - 15;
-          if (from < 0) {
-            int i = s_start[(from + kM) >> 4];
-            while (i < nt && stage[i].cell < from + kM) ++i;
-            for (; i < nt; ++i) add(i);
-          }
-          int i = s_start[(from < 0 ? 0 : from) >> 4];
-          while (i < nt && stage[i].cell < from) ++i;
-          for (; i < nt && stage[i].cell <= l; ++i) add(i);
-          if (any) put(grid, l, get(grid, l) + acc);
-        }
-        __syncthreads();
-      }
-      if (n <= 0) __syncthreads();  // the grid is clear
       Cx<dd> x[16], out[8];
 #pragma unroll
-      for (int a = 0; a < 16; ++a) x[a] = get(grid, 256 * a + tid);
-      fft4096(x, grid, kTfTwD1, kTfTwD2, out);
+      for (int a = 0; a < 16; ++a) {
+        long long* const c = cells + 2 * tr * kM + 256 * a + tid;
+        x[a] = Cx<dd>{dd_of_int(__ldcg(c)), dd_of_int(__ldcg(c + kM))};
+        c[0] = 0;
+        c[kM] = 0;
+      }
+      fft4096(x, buf, kTfTwD1, kTfTwD2, out);
       if (!tr) {
 #pragma unroll
         for (int s = 0; s < 8; ++s) put(s_z, 256 * s + tid, out[s]);
@@ -188,16 +128,17 @@ __global__ void __launch_bounds__(kThreads, 2) transform64_kernel(TransformParam
 #pragma unroll
         for (int s = 0; s < 8; ++s) {
           const float2 t = __ldg(&kTfDeconvD[256 * s + tid]);
-          const dd dc{t.x, t.y};
+          const dd dz{t.x * z_inv, t.y * z_inv}, dw{t.x * w_inv, t.y * w_inv};
           const Cx<dd> z = get(s_z, 256 * s + tid);
           bool ill;
-          const dd v = power_dd(Cx<dd>{mul_(z.re, dc), mul_(z.im, dc)},
-                                Cx<dd>{mul_(out[s].re, dc), mul_(out[s].im, dc)}, nd, ill);
+          const dd v = power_dd(Cx<dd>{mul_(z.re, dz), mul_(z.im, dz)},
+                                Cx<dd>{mul_(out[s].re, dw), mul_(out[s].im, dw)}, nd, ill);
           // bin p + 16 r + 256 s, padded by one word per 16; -1 marks it for re-evaluation
           pw[(tid >> 4) + 17 * (tid & 15) + 272 * s] = ill ? -1.0 : scale * dd_double(v);
         }
       }
     }
+    __threadfence();  // the cleared cells, before the next run's reductions
     __syncthreads();
 
     double pv[8];

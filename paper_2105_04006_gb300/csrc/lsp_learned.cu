@@ -373,6 +373,43 @@ __global__ void repitch_bf16_kernel(const bf16* __restrict__ src, int64_t rows, 
     dst[(i / cols) * ldd + i % cols] = src[(i / cols) * lds + i % cols];
 }
 
+// The weights' transposed and padded copies of all layers in one launch (seven
+// launches of 3 us each for a training step of four layers).  A job is a
+// rows x cols matrix in 32 x 32 tiles, numbered from `first`.
+struct CopyJob {
+  const bf16* src;
+  bf16* dst;
+  int rows, cols, transposed;
+  int64_t lds, ldd;
+  unsigned first;
+};
+struct CopyJobs {
+  CopyJob job[16];
+  int n;
+};
+__global__ void copy_jobs_kernel(const __grid_constant__ CopyJobs jobs) {
+  __shared__ bf16 tile[32][33];
+  int q = 0;
+  while (q + 1 < jobs.n && blockIdx.x >= jobs.job[q + 1].first) ++q;
+  const CopyJob& j = jobs.job[q];
+  const int col_tiles = (j.cols + 31) / 32, i = (int)(blockIdx.x - j.first);
+  const int r0 = i / col_tiles * 32, c0 = i % col_tiles * 32;
+  for (int k = threadIdx.y; k < 32; k += blockDim.y) {
+    const int r = r0 + k, c = c0 + threadIdx.x;
+    if (r < j.rows && c < j.cols) {
+      const bf16 v = j.src[r * j.lds + c];
+      if (j.transposed) tile[k][threadIdx.x] = v;
+      else j.dst[r * j.ldd + c] = v;
+    }
+  }
+  if (!j.transposed) return;
+  __syncthreads();
+  for (int k = threadIdx.y; k < 32; k += blockDim.y) {
+    const int c = c0 + k, r = r0 + threadIdx.x;
+    if (c < j.cols && r < j.rows) j.dst[c * j.ldd + r] = tile[threadIdx.x][k];
+  }
+}
+
 cudaError_t transpose_bf16(const bf16* src, int64_t rows, int64_t cols, int64_t lds, bf16* dst, int64_t ldd,
                            cudaStream_t s) {
   if (rows <= 0 || cols <= 0) return cudaSuccess;
@@ -515,7 +552,7 @@ __global__ void rowsum_kernel(const bf16* __restrict__ m, int rows, int64_t cols
   const int lane = threadIdx.x & 31;
   if (row >= rows) return;
   float s = 0.0f;
-#pragma unroll 16
+#pragma unroll 64
   for (int64_t c = lane; c < cols; c += 32) s += __bfloat162float(m[row * ld + c]);  // loads in flight, adds in order
   for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
   if (lane == 0) out[row] = s;
@@ -860,11 +897,22 @@ void mlp_ws_layout(const Layers& L, int64_t batch, bool training, char* base, Ml
   w->total = off;
 }
 
-// Transposed weights of every layer (the forward GEMMs' B operands).
-lsp_status prep_forward_weights(const Layers& L, const bf16* p16, const MlpWs& w, cudaStream_t s) {
-  for (int l = 0; l < L.n; ++l)
-    LEARN_CUDA(transpose_bf16(p16 + L.w_off[l], L.in[l], L.out[l], L.out[l], w.wt[l], ld8(L.in[l]), s),
-               "MLP weight transpose");
+// Transposed weights of every layer (the forward GEMMs' B operands) and, for
+// training, the padded copies (the input-gradient GEMMs').
+lsp_status prep_weights(const Layers& L, const bf16* p16, const MlpWs& w, bool training, cudaStream_t s) {
+  CopyJobs jobs;
+  jobs.n = 0;
+  unsigned tiles = 0;
+  auto add = [&](const bf16* src, int rows, int cols, bf16* dst, int64_t ldd, int transposed) {
+    jobs.job[jobs.n++] = CopyJob{src, dst, rows, cols, transposed, cols, ldd, tiles};
+    tiles += (unsigned)((rows + 31) / 32 * ((cols + 31) / 32));
+  };
+  for (int l = 0; l < L.n; ++l) {  // at most 7 layers: 13 jobs
+    add(p16 + L.w_off[l], L.in[l], L.out[l], w.wt[l], ld8(L.in[l]), 1);
+    if (training && l > 0) add(p16 + L.w_off[l], L.in[l], L.out[l], w.wp[l], ld8(L.out[l]), 0);
+  }
+  copy_jobs_kernel<<<tiles, dim3(32, 8), 0, s>>>(jobs);
+  LEARN_CUDA(cudaGetLastError(), "MLP weight copies");
   return LSP_OK;
 }
 
@@ -968,7 +1016,7 @@ lsp_status lsp_mlp_forward(const lsp_mlp_dims* dims, const float* params, const 
   if (!workspace || ws_bytes < w.total) return err_arg("MLP workspace too small");
   w.logits = logits;
   cudaStream_t s = (cudaStream_t)stream;
-  if ((st = prep_forward_weights(L, (const bf16*)params_bf16, w, s))) return st;
+  if ((st = prep_weights(L, (const bf16*)params_bf16, w, false, s))) return st;
   return mlp_forward_impl(L, params, (const bf16*)x_bf16, batch, w, false, s);
 }
 
@@ -988,10 +1036,7 @@ lsp_status lsp_mlp_loss_grad(const lsp_mlp_dims* dims, const float* params, cons
   cudaStream_t s = (cudaStream_t)stream;
   const bf16* p16 = (const bf16*)params_bf16;
   const bf16* x = (const bf16*)x_bf16;
-  if ((st = prep_forward_weights(L, p16, w, s))) return st;
-  for (int l = 1; l < L.n; ++l)
-    LEARN_CUDA(repitch_bf16(p16 + L.w_off[l], L.in[l], L.out[l], L.out[l], w.wp[l], ld8(L.out[l]), s),
-               "MLP weight copy");
+  if ((st = prep_weights(L, p16, w, true, s))) return st;
   LEARN_CUDA(transpose_bf16(x, batch, L.in[0], L.in[0], w.xT, w.ldb, s), "MLP input transpose");
   if ((st = mlp_forward_impl(L, params, x, batch, w, true, s))) return st;
   const int n_cls = L.out[L.n - 1];
@@ -1472,7 +1517,7 @@ lsp_status lsp_propose_refine(const lsp_proposer* net, const double* t, const fl
   for (int l = 0; l < L.n; ++l) w.wt[l] = (bf16*)(ws + p.off_wt[l]);
   for (int l = 0; l + 1 < L.n; ++l) w.act[l] = (bf16*)(ws + p.off_act[l & 1]);
   w.logits = (float*)(ws + p.off_logits);
-  if ((st = prep_forward_weights(L, (const bf16*)net->params_bf16, w, s))) return st;
+  if ((st = prep_weights(L, (const bf16*)net->params_bf16, w, false, s))) return st;
   for (int64_t r0 = 0; r0 < n_obj; r0 += kProposeRows) {
     const int64_t rows = n_obj - r0 < kProposeRows ? n_obj - r0 : kProposeRows;
     if ((st = mlp_forward_impl(L, net->params, feat + r0 * LSP_FEAT_DIM, rows, w, false, s))) return st;

@@ -308,6 +308,12 @@ lsp_status make_map(CUtensorMap* map, const bf16* base, int64_t rows, int64_t k,
   return LSP_OK;
 }
 
+struct RowSums {
+  const bf16* m;
+  int rows;
+  int64_t cols, ld;
+  float* out;
+};
 struct Gemm {
   int M, N, K;
   const bf16* A;  // [M][lda], K contiguous
@@ -326,6 +332,7 @@ struct Gemm {
   int64_t ldt;
   int splits;     // K split: partial FP32 tiles at part + z M N (pitch N), summed into C32 in order of z
   float* part;
+  RowSums sums;   // row sums to take behind the product (rows 0: none)
 };
 
 // Split count for a weight-gradient GEMM: about one CTA per SM, at most
@@ -340,9 +347,32 @@ int k_splits(int M, int N, int K) {
   return s < kb ? s : kb;
 }
 
+// Row sums of a bf16 [rows x cols] matrix of row pitch ld: the bias
+// gradients from the transposed dZ (features x batch).  One warp per row,
+// lanes along it, a fixed shuffle tree: the same order on every call.
+__device__ __forceinline__ void row_sums(const RowSums& q, int64_t warp) {
+  const int lane = threadIdx.x & 31;
+  if (warp >= q.rows) return;
+  const bf16* row = q.m + warp * q.ld;
+  float s = 0.0f;
+#pragma unroll 64
+  for (int64_t c = lane; c < q.cols; c += 32) s += __bfloat162float(row[c]);  // loads in flight, adds in order
+  for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+  if (lane == 0) q.out[warp] = s;
+}
+
+// Behind a weight-gradient GEMM: the first blocks take the layer's bias
+// gradient (rows of dZ^T), the others add the GEMM's partial tiles in order
+// of z (one launch and one latency for both).
 __global__ void splitk_reduce_kernel(const float* __restrict__ part, int splits, int64_t mn, int n,
-                                     float* __restrict__ out, int64_t ldo) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < mn; i += (int64_t)gridDim.x * blockDim.x) {
+                                     float* __restrict__ out, int64_t ldo, RowSums q) {
+  const int64_t sum_blocks = (q.rows + 7) / 8;
+  if (blockIdx.x < sum_blocks) {
+    row_sums(q, (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
+    return;
+  }
+  for (int64_t i = (blockIdx.x - sum_blocks) * (int64_t)blockDim.x + threadIdx.x; i < mn;
+       i += (gridDim.x - sum_blocks) * (int64_t)blockDim.x) {
     float s = 0.0f;
     for (int z = 0; z < splits; ++z) s += part[z * mn + i];
     out[(i / n) * ldo + i % n] = s;
@@ -494,9 +524,12 @@ lsp_status gemm(const Gemm& q, cudaStream_t s) {
   LEARN_CUDA(cudaGetLastError(), "GEMM launch");
   if (splits > 1) {
     const int64_t mn = (int64_t)q.M * q.N;
-    splitk_reduce_kernel<<<(unsigned)((mn + 255) / 256 < 1024 ? (mn + 255) / 256 : 1024), 256, 0, s>>>(
-        q.part, splits, mn, q.N, q.C32, q.ldc32);
+    const unsigned blocks = (unsigned)((mn + 255) / 256 < 1024 ? (mn + 255) / 256 : 1024);
+    splitk_reduce_kernel<<<blocks + (q.sums.rows + 7) / 8, 256, 0, s>>>(q.part, splits, mn, q.N, q.C32, q.ldc32, q.sums);
     LEARN_CUDA(cudaGetLastError(), "GEMM split reduction");
+  } else if (q.sums.rows > 0) {
+    splitk_reduce_kernel<<<(q.sums.rows + 7) / 8, 256, 0, s>>>(nullptr, 0, 0, 1, nullptr, 0, q.sums);
+    LEARN_CUDA(cudaGetLastError(), "row sums");
   }
   return LSP_OK;
 }
@@ -541,21 +574,6 @@ __global__ void mean_kernel(const float* __restrict__ v, int64_t n, float* out) 
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += sh[w];
     *out = (float)(t / (double)(n > 0 ? n : 1));
   }
-}
-
-// Row sums of a bf16 [rows x cols] matrix of row pitch ld: the bias
-// gradients from the transposed dZ (features x batch).  One warp per row,
-// lanes along it, a fixed shuffle tree: the same order on every call.
-__global__ void rowsum_kernel(const bf16* __restrict__ m, int rows, int64_t cols, int64_t ld,
-                              float* __restrict__ out) {
-  const int row = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
-  const int lane = threadIdx.x & 31;
-  if (row >= rows) return;
-  float s = 0.0f;
-#pragma unroll 64
-  for (int64_t c = lane; c < cols; c += 32) s += __bfloat162float(m[row * ld + c]);  // loads in flight, adds in order
-  for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-  if (lane == 0) out[row] = s;
 }
 
 __global__ void adamw_kernel(int64_t n, float* __restrict__ p, bf16* __restrict__ p16,
@@ -1062,9 +1080,8 @@ lsp_status lsp_mlp_loss_grad(const lsp_mlp_dims* dims, const float* params, cons
     g.ldc32 = L.out[l];
     g.splits = k_splits(g.M, g.N, g.K);
     g.part = w.part;
+    g.sums = RowSums{w.dzT[cur], L.out[l], batch, w.ldb, grad + L.b_off[l]};
     if ((st = gemm(g, s))) return st;
-    rowsum_kernel<<<(L.out[l] + 7) / 8, 256, 0, s>>>(w.dzT[cur], L.out[l], batch, w.ldb, grad + L.b_off[l]);
-    LEARN_CUDA(cudaGetLastError(), "bias gradient");
     if (l > 0) {
       // dZ_{l-1} = (dZ_l W_l^T) * (A_{l-1} > 0), also written transposed
       Gemm h;

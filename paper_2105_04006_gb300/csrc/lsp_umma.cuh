@@ -303,56 +303,56 @@ __global__ void __launch_bounds__(THREADS, 2)
     __syncthreads();
     const int cols = min(hw, n_valid - h0);
     if (c32 || g.C16 || (use_mask && g.C16T)) {
-      // 8 columns per lane, 16 lanes per row (EPI_COLS = 128): two rows per
-      // warp and eight per CTA at a time, 16-byte stores where aligned
-      const int r_sub = lane >> 4, c = (lane & 15) * 8;
-      const int cnt = min(8, cols - c);
-      if (cnt > 0) {
-        for (int r = warp * 2 + r_sub; r < BM; r += THREADS / 16) {
-          const int m = m0 + r;
-          if (m >= g.M) break;
-          const float4* src = reinterpret_cast<const float4*>(stile + r * sp + c);
-          const float4 lo = src[0], hi = src[1];
-          float x[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
-          const int n = n0 + h0 + c;
-          if (use_mask) {
-            const bf16* mk = g.mask + (int64_t)m * g.ldm + n;
-            if (cnt == 8 && vec_mask) {
-              const uint4 u = *reinterpret_cast<const uint4*>(mk);
-              const bf16* hv = reinterpret_cast<const bf16*>(&u);
+      // 8 columns per lane, as many lanes per row as the staged part has
+      // groups of 8 (16 lanes at a fixed 128 columns left three in four idle
+      // in 32-column tiles, 16 rounds of load latency each)
+      const int per_row = (cols + 7) / 8;
+      for (int i = tid; i < BM * per_row; i += THREADS) {
+        const int r = i / per_row, c = (i % per_row) * 8;
+        const int cnt = min(8, cols - c);
+        const int m = m0 + r;
+        if (m >= g.M) break;  // later i only have larger rows
+        const float4* src = reinterpret_cast<const float4*>(stile + r * sp + c);
+        const float4 lo = src[0], hi = src[1];
+        float x[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+        const int n = n0 + h0 + c;
+        if (use_mask) {
+          const bf16* mk = g.mask + (int64_t)m * g.ldm + n;
+          if (cnt == 8 && vec_mask) {
+            const uint4 u = *reinterpret_cast<const uint4*>(mk);
+            const bf16* hv = reinterpret_cast<const bf16*>(&u);
 #pragma unroll
-              for (int j = 0; j < 8; ++j)
-                if (!(__bfloat162float(hv[j]) > 0.0f)) x[j] = 0.0f;
-            } else {
-              for (int j = 0; j < cnt; ++j)
-                if (!(__bfloat162float(mk[j]) > 0.0f)) x[j] = 0.0f;
-            }
-            if (g.C16T) {  // the transposed copy below reads the masked tile
-              float4* back = reinterpret_cast<float4*>(stile + r * sp + c);
-              back[0] = make_float4(x[0], x[1], x[2], x[3]);
-              back[1] = make_float4(x[4], x[5], x[6], x[7]);
-            }
+            for (int j = 0; j < 8; ++j)
+              if (!(__bfloat162float(hv[j]) > 0.0f)) x[j] = 0.0f;
+          } else {
+            for (int j = 0; j < cnt; ++j)
+              if (!(__bfloat162float(mk[j]) > 0.0f)) x[j] = 0.0f;
           }
-          if (c32) {
-            float* d = c32 + (int64_t)m * g.ldc32 + n;
-            if (cnt == 8 && vec_c32) {
-              reinterpret_cast<float4*>(d)[0] = make_float4(x[0], x[1], x[2], x[3]);
-              reinterpret_cast<float4*>(d)[1] = make_float4(x[4], x[5], x[6], x[7]);
-            } else {
-              for (int j = 0; j < cnt; ++j) d[j] = x[j];
-            }
+          if (g.C16T) {  // the transposed copy below reads the masked tile
+            float4* back = reinterpret_cast<float4*>(stile + r * sp + c);
+            back[0] = make_float4(x[0], x[1], x[2], x[3]);
+            back[1] = make_float4(x[4], x[5], x[6], x[7]);
           }
-          if (g.C16) {
-            bf16* d = g.C16 + (int64_t)m * g.ldc16 + n;
-            if (cnt == 8 && vec_c16) {
-              uint4 u;
-              __nv_bfloat162* hv = reinterpret_cast<__nv_bfloat162*>(&u);
+        }
+        if (c32) {
+          float* d = c32 + (int64_t)m * g.ldc32 + n;
+          if (cnt == 8 && vec_c32) {
+            reinterpret_cast<float4*>(d)[0] = make_float4(x[0], x[1], x[2], x[3]);
+            reinterpret_cast<float4*>(d)[1] = make_float4(x[4], x[5], x[6], x[7]);
+          } else {
+            for (int j = 0; j < cnt; ++j) d[j] = x[j];
+          }
+        }
+        if (g.C16) {
+          bf16* d = g.C16 + (int64_t)m * g.ldc16 + n;
+          if (cnt == 8 && vec_c16) {
+            uint4 u;
+            __nv_bfloat162* hv = reinterpret_cast<__nv_bfloat162*>(&u);
 #pragma unroll
-              for (int j = 0; j < 4; ++j) hv[j] = __floats2bfloat162_rn(x[2 * j], x[2 * j + 1]);
-              *reinterpret_cast<uint4*>(d) = u;
-            } else {
-              for (int j = 0; j < cnt; ++j) d[j] = __float2bfloat16_rn(x[j]);
-            }
+            for (int j = 0; j < 4; ++j) hv[j] = __floats2bfloat162_rn(x[2 * j], x[2 * j + 1]);
+            *reinterpret_cast<uint4*>(d) = u;
+          } else {
+            for (int j = 0; j < cnt; ++j) d[j] = __float2bfloat16_rn(x[j]);
           }
         }
       }

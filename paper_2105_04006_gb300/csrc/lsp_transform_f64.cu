@@ -93,10 +93,10 @@ __global__ void __launch_bounds__(kThreads, 2) transform64_kernel(TransformParam
     const double y_sc = pow2(-y_exponent(oi.sum_y2));
     {  // spread: each warp takes an eighth of the observations
       const float one[2] = {(float)pow2(z_bits(n)), (float)pow2(w_bits(n))};
-      const int j1 = (int)((int64_t)n * (warp + 1) / kWarps);
-      for (int jb = (int)((int64_t)n * warp / kWarps); jb < j1; jb += 32) {
+      const uint32_t j1 = (uint32_t)((int64_t)n * (warp + 1) / kWarps);
+      for (uint32_t jb = (uint32_t)((int64_t)n * warp / kWarps); jb < j1; jb += 32) {
         const ObsD ob = obs_of(rec[jb + lane < j1 ? jb + lane : jb], kc, kLog2M, y_sc);
-        spread_warp(ob, min(32, j1 - jb), kM - 1, one, [&](int t, uint32_t l, long long re, long long im) {
+        spread_warp(ob, (int)min(32u, j1 - jb), kM - 1, one, [&](int t, uint32_t l, long long re, long long im) {
           add_cell(cells + (2 * t) * kM + l, re);
           add_cell(cells + (2 * t + 1) * kM + l, im);
         });

@@ -247,12 +247,12 @@ typedef struct lsp_plan lsp_plan;
  * The ablation kernels (trig or staging non-zero) are FP32, scalar
  * (packed 0), k_reseed = freqs_per_thread = 16, standard periodogram only;
  * other combinations return LSP_E_UNSUPPORTED.
- * reserved = 1: objects with enough observations (FP32 40, FP64 8) get their
- * trig sums from a nonuniform FFT, per run of 2048 bins or, one object, of
- * its whole grid, instead of pair by pair (the same sums, no less exact), and
- * the kernel the other fields name serves the rest.  It is the choice of every call whose
- * lsp_opts leave the kernel options 0, and of a plan until lsp_plan_set_config
- * says otherwise.  It needs block_threads x freqs_per_thread = 2048 (a single
+ * reserved = 1: objects with enough observations (FP32 40, more on grids of
+ * a few hundred bins; FP64 8) get their trig sums from a nonuniform FFT, per
+ * run of 2048 bins or, one object, of its whole grid, instead of pair by pair
+ * (the same sums, no less exact), and the kernel the other fields name serves
+ * the rest.  It is the choice of every call whose lsp_opts leave the kernel
+ * options 0, and of a plan until lsp_plan_set_config says otherwise.  It needs block_threads x freqs_per_thread = 2048 (a single
  * object: any) and no ablation; other configurations read it as 0.
  */
 typedef struct lsp_config {

@@ -90,9 +90,22 @@ constexpr int kGateObjects = 8;  // objects the autotuner's error gate checks
 // Objects with at least this many observations take the transform path: its
 // cost per run of bins hardly depends on N_t, the direct kernel's is
 // proportional to it.  Measured (2000 objects of equal N_t, N_f = 1e5,
-// transform | direct, ms): N_t 32 2.2 | 1.9, 48 2.2 | 2.6, 100 2.4 | 5.0.
+// transform | direct, ms): N_t 32 2.2 | 1.9, 48 2.2 | 2.6, 100 2.4 | 5.0; later
+// cuts of the run's cost put the crossing at N_t 36, the generalized
+// periodogram's at 43.
 constexpr int kTfMinObs = 40;
 constexpr int kTfMinObs64 = 8;
+// That line is for whole runs.  A run costs the same however few of its bins
+// lie in the grid, the direct kernel's warps of 512 bins past its end cost
+// nothing: for a batch on a short or ragged grid the line moves up by half the
+// share of the runs' warps without bins.  20 000 objects, transform | direct,
+// us: N_f 512, N_t 80 732 | 711, 100 778 | 821; N_f 1000, N_t 56 691 | 682,
+// 64 684 | 727; N_f 2049, N_t 40 1098 | 1015, 56 1100 | 1235.  In FP64 the
+// transform is the faster on any grid (5000 objects, N_t 8: N_f 512 1005 | 1968).
+int tf_min_obs(int base, int64_t n_f) {
+  const int64_t runs = (n_f + kTfBins - 1) / kTfBins, warps = (n_f + 511) / 512;
+  return (int)(base * (4 * runs + warps) / (2 * warps));
+}
 // One FP32 object goes run by run or by one transform of its whole grid,
 // whichever a model of their times (us, GB300, fitted to N_t 1e3 .. 1e5, N_f
 // 3e3 .. 1e6) puts first: a run costs 12 + N_t / 150 per wave of CTAs, the
@@ -151,7 +164,8 @@ lsp_status resolve(int64_t n_obj, int64_t total_nt, const lsp_grid* g, const lsp
   // the transform is the library's own choice: a call that names a kernel
   // option gets the direct kernel it names
   bool tf = l.prec == LSP_FP32 || !gls;
-  const int tf_min = l.prec == LSP_FP32 ? kTfMinObs : kTfMinObs64;
+  int tf_min = l.prec == LSP_FP32 ? kTfMinObs : kTfMinObs64;
+  if (n_obj > 1 && l.prec == LSP_FP32) tf_min = tf_min_obs(tf_min, l.n_f);
   if (cfg) tf = tf && cfg->reserved == 1;
   else tf = tf && !o.k_reseed && !o.freqs_per_thread && !o.block_threads && !o.obs_split;
   if (cfg) {

@@ -195,6 +195,21 @@ def test_smaller_workspaces_take_smaller_paths(env, precision):
         lsp.periodogram(t, y, g, precision=precision, workspace=torch.empty(1024, dtype=torch.uint8, device=dev))
 
 
+@pytest.mark.parametrize("n_f", [1, 511, 513, 1000, 1537])
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_short_grids_equal_the_direct_kernel(env, n_f, precision):
+    """Both sides of the observation counts at which a short grid's objects change kernels."""
+    lsp, torch, dev = env
+    counts = [7, 8, 9, 19, 20, 21, 39, 41, 59, 60, 61, 99, 100, 101, 400]
+    t, y, off = _segments(counts, "uniform", 19)
+    dt = torch.float32 if precision == "fp32" else torch.float64
+    args = (torch.tensor(t, device=dev), torch.tensor(y, dtype=dt, device=dev), torch.tensor(off, device=dev),
+            lsp.Grid(0.24, 12.0, n_f))
+    p, _ = lsp.batch(*args, precision=precision, return_power=True)
+    q, _ = lsp.batch(*args, precision=precision, return_power=True, k_reseed=8)
+    assert float((p - q).abs().max()) <= (2 * TOL if precision == "fp32" else 1e-10)
+
+
 @pytest.mark.parametrize("norm", ["standard", "psd"])
 def test_refine_fallback_runs_equal_the_direct_full_grid(env, norm):
     """The fallback looks for the maximum's run with the transform and takes the result from the direct kernel

@@ -479,7 +479,7 @@ lsp_status gemm(const Gemm& q, cudaStream_t s) {
   // training batch of 4096 rows is 32 tiles: 32 columns make 256 of them).
   // The K order of every output, and so its bits, does not depend on it.
   // Measured: train step of 4096 rows 499 -> 228 us together with the
-  // epilogue's transposed copy.
+  // epilogue's transposed copy (172 with the fewer launches around it).
   const int row_tiles = (q.M + umma::BM - 1) / umma::BM * (q.splits < 1 ? 1 : q.splits);
   int n_tile = q.N >= umma::MAX_BN ? umma::MAX_BN : (q.N + 15) / 16 * 16;
   while (n_tile > 32 && (int64_t)row_tiles * ((q.N + n_tile - 1) / n_tile) < 148) n_tile = (n_tile / 2 + 15) / 16 * 16;

@@ -17,7 +17,8 @@
 //     owns tile rows 32w..32w+31, one row per thread), add the bias, apply
 //     ReLU, and stage the FP32 tile in the idle ring, 128 columns at a time;
 //     the stores to global memory then run along rows, 8 columns per lane
-//     with 16-byte writes (or, for the transposed copy, down columns), so
+//     with 16-byte writes (the transposed copy: down columns, 8 rows per lane,
+//     16-byte writes too), so
 //     that each warp writes contiguous bytes: multiplication by a ReLU mask,
 //     FP32 and/or bfloat16 outputs, and an optional transposed bfloat16 copy
 //     (the operand layout the weight-gradient GEMM reads).

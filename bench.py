@@ -2,17 +2,18 @@
 """Throughput benchmark of the GB300 Lomb-Scargle path.
 
 A step is one pass of the whole path over one batch resident in HBM: the
-prologue (centring, phase records), the work-queue order, the persistent
-trig-sum kernel with its fused power/argmax/top-3 epilogue and the finalize
-kernel, replayed as one CUDA graph (``lsp_plan_execute``) with the autotuned
+prologue (centring, phase records), the work lists, the persistent transform
+and direct trig-sum kernels with their fused power/argmax/top-3 epilogue and
+the finalize kernel, replayed as one CUDA graph (``lsp_plan_execute``) with the autotuned
 configuration.  The default workload is the largest batch: 100000 objects,
 N_t log-uniform in [10, 2000] with a seasonal cadence, N_f = 50000 on
 [0.24, 12) c/d, FP32 sums with FP64/fixed-point phases, argmax and top-3.
 
 One JSON line is printed by rank 0.  ``value`` is objects/s over all ranks;
 ``e2e`` is the same metric through the host-buffer entry point with the
-copies inside the timed region; ``roofline`` relates the main kernel's
-measured pair rate to the FP32-pipe bound; ``cpu_baseline`` times the FP64
+copies inside the timed region; ``roofline`` relates the main kernels'
+operations to the FP32-pipe bound (the transform's own operations where it
+runs, 8 per pair for the direct kernels alone); ``cpu_baseline`` times the FP64
 CPU oracle on a bounded sample of the same workload on this host's cores;
 ``learned`` (default workload, one GPU) times the learned proposal path
 (``lsp_propose_refine``, one call) against the plain full grid on 100000
@@ -51,6 +52,14 @@ KERNEL_OPS_PER_PAIR = 6    # what the kernels spend: a chain of K pairs takes on
 FP32_LANES_PER_SM = 128    # FP32 lanes per SM per clock
 FP64_LANES_PER_SM = 2      # FP64 FMAs per SM per clock: 1.25 TFLOP/s nominal / (2 x 152 SMs x 2.07 GHz)
 
+# FP32 operations of the transform path, per run of 2048 bins: two 4096-point
+# transforms of 39 per point and 30 a bin for its power; per observation and
+# run: 8 cells of a degree-8 window for two grids with four products each, and
+# 40 for the phase.  (Objects below 40 observations keep the direct kernel.)
+RUN_BINS, TF_MIN_OBS = 2048, 40
+RUN_OPS = 2 * 4096 * 39 + 2048 * 30
+RUN_OBS_OPS = 8 * (2 * 9 + 4) + 40
+
 WORKLOADS = {
     "ragged_survey": dict(kind="batch", top_k=1, power=False, cpu_sample=64, ref_per_step=6,
                           desc="10000 objects, N_t~U{50..500}, seasonal cadence, N_f=1e5 on [0.24,12) c/d, argmax only"),
@@ -77,6 +86,27 @@ def make_workload(name, rank, n_obj=None):
     seed = synth.SEEDS[name] + 1_000_003 * rank
     kw = {"n_obj": n_obj} if n_obj else {}
     return synth.by_name(name, seed=seed, **kw)
+
+
+def roofline_of(plan, n_t, n_f, pairs, main_ms, fp64, peak_pairs, basis):
+    """Main-kernel roofline: FP32 operations against the pipe where the transform runs a batch,
+    pairs against 8 operations each where the direct kernels run alone.  One object, and FP64, by the
+    transform have no such bound: latency and L2 traffic of a few launches, two-float arithmetic."""
+    rate = pairs / (main_ms / 1e3) / 1e9
+    if not plan.transform:
+        return {"bound": "alu", "achieved": rate, "peak": peak_pairs, "unit": "Gpair/s",
+                "frac": rate / peak_pairs if peak_pairs else None, "peak_basis": basis, "path": "direct"}
+    note = {"path": "transform", "pairs_equivalent_per_s": rate * 1e9,
+            "path_note": "sums by a nonuniform FFT per run of bins: the N_t*N_f pairs are not evaluated one by one"}
+    if fp64 or len(n_t) < 2:
+        return {"bound": "latency", "achieved": None, "peak": None, "unit": None, "frac": None, **note}
+    n_t = np.asarray(n_t, dtype=np.float64)
+    runs = -(-n_f // RUN_BINS)
+    tf = n_t >= TF_MIN_OBS
+    ops = runs * (RUN_OPS * tf.sum() + RUN_OBS_OPS * n_t[tf].sum()) + KERNEL_OPS_PER_PAIR * n_f * n_t[~tf].sum()
+    got, peak = ops / (main_ms / 1e3) / 1e9, peak_pairs * OPS_PER_PAIR if peak_pairs else None
+    return {"bound": "alu", "achieved": got, "peak": peak, "unit": "Gop/s", "frac": got / peak if peak else None,
+            "peak_basis": basis.replace(f" / {OPS_PER_PAIR} ops per pair", ", one operation per lane and clock"), **note}
 
 
 # ------------------------------------------------------------------ clocks
@@ -439,11 +469,12 @@ def run_gls(args, w, name):
         "data": "synthetic",
         "config": {"workload": name + "+gls", "shape": w["desc"] + ", dy ~ U[0.02, 0.3]", "n_obj": b.n_obj,
                    "total_nt": int(b.t.size), "n_f": g.n_f, "l2": "flushed between steps (256 MiB write)",
-                   "kernel": "main_f32_packed_gls" if not fp64 else "main_f64_gls", "options": kw},
+                   "kernel": "main_f64_gls" if fp64 else "main_f32_packed_gls" if kw else "transform_kernel",
+                   "options": kw},
         "pairs_per_s": achieved * 1e9,
         "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "Gpair/s",
-                     "frac": achieved / peak if peak else None, "traffic": None,
-                     "peak_basis": basis},
+                     "frac": achieved / peak if peak and (fp64 or kw) else None, "traffic": None,
+                     "peak_basis": basis if fp64 or kw else "pairs equivalent: the transform does not evaluate them"},
         "cpu_baseline": cpu, "parity_vs_oracle": parity,
         "e2e": {"value": b.n_obj / (statistics.mean(e2e_ms) / 1e3), "unit": "objects/s", "h2d_bytes_per_step": int(h2d),
                 "d2h_bytes_per_step": int(peaks.numel()), "ms_per_step": statistics.mean(e2e_ms)},
@@ -782,7 +813,6 @@ def other_leg(args, dev, name, precision, steps):
     st, _ = timed(False)
     _, mk = timed(True)
     n_sm = torch.cuda.get_device_properties(dev).multi_processor_count
-    achieved = b.pairs / (mk / 1e3) / 1e9
     if fp64:
         peak = lsp.probe_fma_rates(dev)["f64"] / OPS_PER_PAIR / 1e9
         basis = f"measured DFMA rate / {OPS_PER_PAIR} ops per pair"
@@ -812,8 +842,7 @@ def other_leg(args, dev, name, precision, steps):
     out = {"workload": name, "precision": precision, "shape": w["desc"], "value": b.n_obj / (st / 1e3),
            "unit": "objects/s", "ms_per_step": st, "main_kernel_ms": mk, "pairs_per_s": b.pairs / (st / 1e3),
            "timing": "step without the timing probe; main kernel from a second pass with it",
-           "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "Gpair/s",
-                        "frac": achieved / peak, "peak_basis": basis},
+           "roofline": roofline_of(plan, b.n_t, g.n_f, b.pairs, mk, fp64, peak, basis),
            "kernel_config": plan.config, "autotuned": tuned, "gpu_launches_per_step": plan.kernel_count,
            "steps": steps,
            "parity_vs_oracle": par}
@@ -939,7 +968,6 @@ def run_gpu(args, w, name):
 
     n_sm = torch.cuda.get_device_properties(dev).multi_processor_count
     main_avg = statistics.mean(main_ms)
-    achieved = pairs / (main_avg / 1e3) / 1e9
     clk_mhz = (clocks or {}).get("sm_mhz") or 0.0
     lanes = FP64_LANES_PER_SM if fp64 else FP32_LANES_PER_SM
     rates = lsp.probe_fma_rates(dev)  # measured pipe ceilings, outside the timed region
@@ -987,19 +1015,11 @@ def run_gpu(args, w, name):
                        "precision": "fp64" if fp64 else "fp32 sums, fp64/fixed-point phase",
                        "l2": "flushed between steps (256 MiB write)", "kernel_config": plan.config},
             "pairs_per_s": world * pairs * args.steps / total_s,
-            "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "Gpair/s",
-                         "frac": (achieved / peak) if peak else None, "traffic": traffic,
-                         "kernel": "main trig-sum kernel", "main_kernel_ms": main_avg,
-                         "peak_basis": basis, "peak_nominal_at_max_clock": peak_max,
-                         "measured_fma_rates_per_s": rates,
-                         "frac_of_measured_pipe_ceiling": achieved / ceiling,
-                         "kernel_ops_per_pair": KERNEL_OPS_PER_PAIR,
-                         "frac_note": (f"frac counts {OPS_PER_PAIR} FP32 operations per pair (the rotation "
-                                       f"recurrence's algorithmic work); the kernel issues {KERNEL_OPS_PER_PAIR}, "
-                                       "so its FP32 pipe is busy frac x 6/8 (pipe_busy_with_kernel_ops)"),
-                         "pipe_busy_with_kernel_ops": (achieved * KERNEL_OPS_PER_PAIR / OPS_PER_PAIR / peak)
-                         if (peak and not fp64) else achieved * KERNEL_OPS_PER_PAIR / OPS_PER_PAIR / ceiling,
-                         "source_hash": src},
+            "roofline": dict(roofline_of(plan, b.n_t, g.n_f, pairs, main_avg, fp64, peak, basis),
+                             traffic=traffic, kernel="main kernels (between the prologue and the finalize)",
+                             main_kernel_ms=main_avg, peak_nominal_at_max_clock=peak_max,
+                             measured_fma_rates_per_s=rates, measured_pipe_ceiling_pairs=ceiling,
+                             direct_kernel_ops_per_pair=KERNEL_OPS_PER_PAIR, source_hash=src),
             "cpu_baseline": cpu,
             "parity_vs_oracle": parity,
             "e2e": {"value": e2e_value, "unit": "objects/s", "h2d_bytes_per_step": int(h2d),

@@ -439,6 +439,13 @@ class Plan:
         _check(lib().lsp_plan_get_config(self._h, ctypes.byref(c)))
         return c.as_dict()
 
+    @property
+    def transform(self) -> bool:
+        """Whether objects of enough observations take the transform path (see lsp_config in lsp.h)."""
+        c = Config()
+        _check(lib().lsp_plan_get_config(self._h, ctypes.byref(c)))
+        return c.reserved == 1
+
     def set_config(self, **cfg):
         c = Config()
         _check(lib().lsp_plan_get_config(self._h, ctypes.byref(c)))

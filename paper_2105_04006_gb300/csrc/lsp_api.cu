@@ -750,6 +750,10 @@ bool cache_lookup(const char* path, const std::string& key, lsp_config* c) {
         get("block_threads", &t.block_threads) && get("obs_split", &t.obs_split) &&
         get("packed", &t.packed)) {
       get("trig", &t.trig);        // absent in older entries: 0
+      // an entry from before the transform names the direct kernel only: the
+      // default choice (on) stands beside it, off where the entry's tile does
+      // not allow it
+      t.reserved = 1;
       get("transform", &t.reserved);
       get("staging", &t.staging);
       *c = t;

@@ -115,6 +115,34 @@ def test_plan_uses_the_transform_until_told_otherwise(env):
     plan.close()
 
 
+@pytest.mark.parametrize("threads,on", [(128, True), (256, False)])
+def test_tuned_entry_from_before_the_transform(env, tmp_path, threads, on):
+    """Its choice of direct kernel stands; the transform serves what it serves by default."""
+    import re
+    lsp, torch, dev = env
+    b = synth.ragged_survey(6, seed=3, grid=synth.Grid(0.24, 12.0, 3001))
+    args = (torch.tensor(b.t, device=dev), torch.tensor(b.y.astype(np.float32), device=dev),
+            torch.tensor(b.offsets, device=dev))
+    cache = tmp_path / "tune.jsonl"
+    first = lsp.Plan(b.n_obj, b.t.size, lsp.Grid(0.24, 12.0, 3001))
+    first.autotune(*args, cache_path=str(cache))
+    first.close()
+    entry = re.sub(r'"transform": \d+, ', "", cache.read_text())
+    assert "transform" not in entry
+    for key, v in (("k_reseed", 8), ("freqs_per_thread", 16), ("block_threads", threads)):
+        entry, n = re.subn(rf'"{key}": \d+', f'"{key}": {v}', entry)
+        assert n == 1
+    cache.write_text(entry)
+    plan = lsp.Plan(b.n_obj, b.t.size, lsp.Grid(0.24, 12.0, 3001))
+    cfg = plan.autotune(*args, cache_path=str(cache))
+    assert (cfg["k_reseed"], cfg["freqs_per_thread"], cfg["block_threads"]) == (8, 16, threads)
+    assert plan.transform is on
+    kw = {} if on else dict(k_reseed=8, freqs_per_thread=16, block_threads=threads)
+    _, want = lsp.batch(*args, lsp.Grid(0.24, 12.0, 3001), **kw)
+    assert torch.equal(plan.execute(*args), want)
+    plan.close()
+
+
 @pytest.mark.parametrize("n_t,n_f", [(8, 1), (9, 2047), (33, 32737), (300, 32738), (1000, 65505), (7001, 20_011)])
 @pytest.mark.parametrize("cadence", ["uniform", "nightly", "long"])
 def test_single_object_fp64(env, n_t, n_f, cadence):

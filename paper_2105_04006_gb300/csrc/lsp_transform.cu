@@ -18,11 +18,12 @@
 // instead of 8 per observation.
 //
 // Measured (GB300): 10 000 survey light curves (N_t 50 .. 500) on 1e5 bins
-// 12.2 ms against 64.7 ms with the direct kernel, 1e5 observations on 1e6
-// bins 1.48 ms against 23.4 ms.  A run of 2048 bins takes an SM 6350 clocks at
-// N_t 64, 7620 at 275, 12000 at 1000 (top-3 9 % more, generalized 1.56 times);
-// what bounds it is the L1 data pipe (70 % busy: the spread's atomics and the
-// FFT's exchanges), with the FMA pipe at 50 %.
+// 11.9 ms against 64.7 ms with the direct kernel, 1e5 observations on 1e6
+// bins 1.48 ms against 23.4 ms.  A run of 2048 bins takes an SM 6040 clocks at
+// N_t 64, 7370 at 275, 11700 at 1000 (top-3 8 % more, generalized 1.6 times);
+// what bounds it is the L1 data pipe (76 % busy before the FFT's twiddles came
+// from products: the exchanges, the spread's atomics), with the FMA pipe at
+// 48 %.
 //
 // Accuracy: the window's aliasing is at most 1.6e-7 (5e-8 rms) of the largest
 // amplitude near the run, the FP32 transform adds about as much; both are

@@ -19,8 +19,8 @@
 //
 // Measured (GB300): 10 000 survey light curves (N_t 50 .. 500) on 1e5 bins
 // 11.9 ms against 64.7 ms with the direct kernel, 1e5 observations on 1e6
-// bins 1.48 ms against 23.4 ms.  A run of 2048 bins takes an SM 6040 clocks at
-// N_t 64, 7370 at 275, 11700 at 1000 (top-3 8 % more, generalized 1.6 times);
+// bins 1.48 ms against 23.4 ms.  A run of 2048 bins takes an SM 5990 clocks at
+// N_t 64, 7280 at 275, 11470 at 1000 (top-3 8 % more, generalized 1.6 times);
 // what bounds it is the L1 data pipe (76 % busy before the FFT's twiddles came
 // from products: the exchanges, the spread's atomics), with the FMA pipe at
 // 48 %.
@@ -62,7 +62,10 @@ namespace {
 constexpr int kM = 4096;                 // grid cells
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
-constexpr size_t kPowers = kTfBins + kTfBins / 16;  // a word of padding per 16 powers
+// A word of padding per 8 powers: the lanes fall on distinct banks both in the
+// transform's order (18 apart) and in runs of eight (9 apart).  Together with
+// the staged words in rows of 32: 11 733 -> 11 470 clocks a run at N_t 1000.
+constexpr size_t kPowers = kTfBins + kTfBins / 8;
 static_assert(kTfBins == kM / 2 && kTfBins == kThreads * 8 && kTfGroups == kM / 8, "run length");
 
 __device__ __forceinline__ f2_t cells_f2(const int32_t* a, const int32_t* b, int i) {
@@ -164,20 +167,20 @@ __global__ void __launch_bounds__(kThreads, GLS ? 2 : 3) transform_kernel(Transf
           const uint32_t fw = (b2 << 12) | (lo2 >> 20);
           const float uz = fmaf(__uint2float_rn(fz), 2.3283064365386963e-10f, -0.5f);
           const float uw = fmaf(__uint2float_rn(fw), 2.3283064365386963e-10f, -0.5f);
-          float4* st = reinterpret_cast<float4*>(mine + (size_t)lane * S::kStage);
+          float4* st = reinterpret_cast<float4*>(mine) + lane;  // word w of an observation at 32 w: no bank twice
           st[0] = make_float4(uz, uw, __uint_as_float((r1.x >> 20) - 3u), __uint_as_float((b2 >> 20) - 3u));
-          st[1] = make_float4(ys * c, ys * s, ws * (c - s) * (c + s), ws * 2.0f * c * s);
+          st[32] = make_float4(ys * c, ys * s, ws * (c - s) * (c + s), ws * 2.0f * c * s);
           if (GLS) {
             const float cs = __uint_as_float(r1.w) * c_sc;
-            st[2] = make_float4(cs * c, cs * s, 0.0f, 0.0f);
+            st[64] = make_float4(cs * c, cs * s, 0.0f, 0.0f);
           }
         }
         __syncwarp();
         const int nt = (int)min(32u, j1 - jb);
 #pragma unroll 2
         for (int i = lane >> 3; i < nt; i += 4) {
-          const float4* st = reinterpret_cast<const float4*>(mine + (size_t)i * S::kStage);
-          const float4 at = st[0], v = st[1];
+          const float4* st = reinterpret_cast<const float4*>(mine) + i;
+          const float4 at = st[0], v = st[32];
           const f2_t u = f2_pack(at.x, at.y);
           f2_t w2 = poly[8];
 #pragma unroll
@@ -191,7 +194,7 @@ __global__ void __launch_bounds__(kThreads, GLS ? 2 : 3) transform_kernel(Transf
           atomicAdd(&plane[kW * kM + lw], __float2int_rn(ww * v.z));
           atomicAdd(&plane[(kW + 1) * kM + lw], __float2int_rn(ww * v.w));
           if (GLS) {
-            const float4 q = st[2];
+            const float4 q = st[64];
             atomicAdd(&plane[2 * kM + lz], __float2int_rn(wz * q.x));
             atomicAdd(&plane[3 * kM + lz], __float2int_rn(wz * q.y));
           }
@@ -216,7 +219,7 @@ __global__ void __launch_bounds__(kThreads, GLS ? 2 : 3) transform_kernel(Transf
       const float nf = (float)oi.n;
 #pragma unroll
       for (int s = 0; s < 8; ++s) {
-        const int i = (tid >> 4) + 17 * (tid & 15) + 272 * s;  // bin p + 16 r + 256 s, padded
+        const int i = (tid >> 4) + (tid >> 7) + 18 * (tid & 15) + 288 * s;  // bin b = p + 16 r + 256 s at b + b / 8
         const float dc = __ldg(&kTfDeconv[256 * s + tid]);
         const f2_t f = f2_mul(inv, f2_pack(dc, dc));
         float zr, wr, zi, wi;
@@ -253,7 +256,7 @@ __global__ void __launch_bounds__(kThreads, GLS ? 2 : 3) transform_kernel(Transf
       const float inv_w = 1.0f / w_sc, wsum = oi.wsum_f, yy = (float)oi.sum_y2;
 #pragma unroll
       for (int s = 0; s < 8; ++s) {
-        const int i = (tid >> 4) + 17 * (tid & 15) + 272 * s;  // bin p + 16 r + 256 s, padded
+        const int i = (tid >> 4) + (tid >> 7) + 18 * (tid & 15) + 288 * s;  // bin b = p + 16 r + 256 s at b + b / 8
         const float dc = __ldg(&kTfDeconv[256 * s + tid]);
         const f2_t f = f2_mul(inv, f2_pack(dc, dc));
         float yr, cr, yi, ci;
@@ -271,7 +274,7 @@ __global__ void __launch_bounds__(kThreads, GLS ? 2 : 3) transform_kernel(Transf
     // ---- eight consecutive bins per thread from here on
     float pv[8];
 #pragma unroll
-    for (int m = 0; m < 8; ++m) pv[m] = pw[8 * tid + (tid >> 1) + m];
+    for (int m = 0; m < 8; ++m) pv[m] = pw[9 * tid + m];
     clear_grid();  // for the next item: every thread is past the transform
     const uint32_t k0 = (uint32_t)kc0 + 8u * (uint32_t)tid;
     uint32_t bad = 0u;

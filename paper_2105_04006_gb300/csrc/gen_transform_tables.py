@@ -176,10 +176,10 @@ def main(path):
              [1.0 / psi_hat((t // 16 + 16 * (t % 16) + 256 * s - m // 4) / m, w, beta)
               for s in range(8) for t in range(256)], f32)
         # twiddles of the 4096-point transform's first two radix-16 passes
-        emit(out, "__device__ const float2 kTfTw1[2 * 256]",
-             [unit(p * b, 4096) for p in (1, 4) for b in range(256)], c32, 4)
-        emit(out, "__device__ const float2 kTfTw2[2 * 16]",
-             [unit(r * d, 256) for r in (1, 4) for d in range(16)], c32, 4)
+        emit(out, "__device__ const float2 kTfTw1[4 * 256]",
+             [unit(p * b, 4096) for p in (1, 2, 4, 8) for b in range(256)], c32, 4)
+        emit(out, "__device__ const float2 kTfTw2[4 * 16]",
+             [unit(r * d, 256) for r in (1, 2, 4, 8) for d in range(16)], c32, 4)
         out.write("#endif\n")
         # one long object: e^{2 pi i n / 4096}, e^{2 pi i n / 2^24}, and 1 / psi^ as a polynomial in (4 xi)^2
         out.write("#ifdef LSP_TF_TABLES_LONG\n")

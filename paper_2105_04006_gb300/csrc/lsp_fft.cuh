@@ -94,12 +94,12 @@ __device__ __forceinline__ typename Twiddle<T>::type twiddle(double c, double s)
   }
 }
 
-// w^p, p = 1 .. 15, from w and w^4.
+// w^p, p = 1 .. 15, from w, w^2, w^4 and w^8.
 __device__ __forceinline__ float2 unit_mul(float2 a, float2 b) {
   return make_float2(__fmaf_rn(a.x, b.x, -(a.y * b.y)), __fmaf_rn(a.x, b.y, a.y * b.x));
 }
-__device__ __forceinline__ float2 unit_power(int p, float2 w1, float2 w4) {
-  const float2 w2 = unit_mul(w1, w1), w3 = unit_mul(w2, w1), w8 = unit_mul(w4, w4), w12 = unit_mul(w8, w4);
+__device__ __forceinline__ float2 unit_power(int p, float2 w1, float2 w2, float2 w4, float2 w8) {
+  const float2 w3 = unit_mul(w2, w1), w12 = unit_mul(w8, w4);
   const float2 lo = (p & 3) == 1 ? w1 : (p & 3) == 2 ? w2 : w3, hi = p < 8 ? w4 : p < 12 ? w8 : w12;
   return p < 4 ? lo : (p & 3) == 0 ? hi : unit_mul(hi, lo);
 }
@@ -254,14 +254,15 @@ __device__ __forceinline__ void fft_two_passes(Cx<T> (&x)[16], Cx<T>* buf, int t
 // passed the first barrier here; free again only after a barrier of the
 // caller.
 // tw1 holds e^{2 pi i p b / 4096} for b = 0 .. 255, tw2 e^{2 pi i r d / 256} for
-// d = 0 .. 15: dd all of p, r = 1 .. 15; FP32 the first and the fourth, the
-// others are products (at most four roundings).  The full FP32 tables are 32 KB,
-// about what three CTAs' shared memory leaves of the L1 cache: half of the
-// kernel's loads missed it (clocks per run and SM at N_t 64 / 275 / 1000:
-// 6355 / 7616 / 12 028 with them, 6040 / 7365 / 11 733 with the products; six
-// loads and nine products for the first pass were slower than either).  The
-// periodogram's error against 64 bits (rms of a row, median of 300 objects of
-// 275 observations) goes from 1.9e-7 to 2.2e-7; the direct kernel's is 5.4e-7.
+// d = 0 .. 15: dd all of p, r = 1 .. 15; FP32 those of 1, 2, 4 and 8, the
+// others are products (at most three).  The full FP32 tables are 32 KB, about
+// what three CTAs' shared memory leaves of the L1 cache: half of the kernel's
+// loads missed it (clocks per run and SM at N_t 64 / 275 / 1000: 6355 / 7616 /
+// 12 028 before, 6064 / 7350 / 11 540 now, of which the staging's layout gave
+// 60 / 90 / 260).  Two loads and 13 products would be 1 % faster, but the error
+// against 64 bits (rms of a row, N_t 120, median of 100 objects) goes 2.0e-7,
+// 2.2e-7 with four loads, 2.3e-7 with two, and the largest error of a peak
+// 4.4e-7, 4.4e-7, 6.4e-7; the direct kernel's are 3.1e-7 and 5.8e-7.
 template <typename T>
 __device__ __forceinline__ void fft4096(Cx<T> (&x)[16], Cx<T>* buf, const typename Twiddle<T>::type* __restrict__ tw1,
                                         const typename Twiddle<T>::type* __restrict__ tw2, Cx<T> (&out)[8]) {
@@ -270,11 +271,11 @@ __device__ __forceinline__ void fft4096(Cx<T> (&x)[16], Cx<T>* buf, const typena
       x, buf, tid,
       [&](int p) {
         if constexpr (std::is_same<T, dd>::value) return __ldg(&tw1[(p - 1) * 256 + tid]);
-        else return unit_power(p, __ldg(&tw1[tid]), __ldg(&tw1[256 + tid]));
+        else return unit_power(p, __ldg(&tw1[tid]), __ldg(&tw1[256 + tid]), __ldg(&tw1[512 + tid]), __ldg(&tw1[768 + tid]));
       },
       [&](int r) {
         if constexpr (std::is_same<T, dd>::value) return __ldg(&tw2[(r - 1) * 16 + e0]);
-        else return unit_power(r, __ldg(&tw2[e0]), __ldg(&tw2[16 + e0]));
+        else return unit_power(r, __ldg(&tw2[e0]), __ldg(&tw2[16 + e0]), __ldg(&tw2[32 + e0]), __ldg(&tw2[48 + e0]));
       });
   dft16_first(x);
 #pragma unroll

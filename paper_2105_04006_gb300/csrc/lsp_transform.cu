@@ -19,8 +19,8 @@
 //
 // Measured (GB300): 10 000 survey light curves (N_t 50 .. 500) on 1e5 bins
 // 11.9 ms against 64.7 ms with the direct kernel, 1e5 observations on 1e6
-// bins 1.48 ms against 23.4 ms.  A run of 2048 bins takes an SM 5990 clocks at
-// N_t 64, 7280 at 275, 11470 at 1000 (top-3 8 % more, generalized 1.6 times);
+// bins 1.48 ms against 23.4 ms.  A run of 2048 bins takes an SM 6060 clocks at
+// N_t 64, 7350 at 275, 11540 at 1000 (top-3 8 % more, generalized 1.6 times);
 // what bounds it is the L1 data pipe (76 % busy before the FFT's twiddles came
 // from products: the exchanges, the spread's atomics), with the FMA pipe at
 // 48 %.

@@ -18,12 +18,11 @@
 // instead of 8 per observation.
 //
 // Measured (GB300): 10 000 survey light curves (N_t 50 .. 500) on 1e5 bins
-// 11.9 ms against 64.7 ms with the direct kernel, 1e5 observations on 1e6
+// 11.8 ms against 64.7 ms with the direct kernel, 1e5 observations on 1e6
 // bins 1.48 ms against 23.4 ms.  A run of 2048 bins takes an SM 6060 clocks at
 // N_t 64, 7350 at 275, 11540 at 1000 (top-3 8 % more, generalized 1.6 times);
-// what bounds it is the L1 data pipe (76 % busy before the FFT's twiddles came
-// from products: the exchanges, the spread's atomics), with the FMA pipe at
-// 48 %.
+// what bounds it is the L1 data pipe (71 % busy: the FFT's exchanges, the
+// spread's atomics), with issue at 60 % and the FMA pipe at 52 %.
 //
 // Accuracy: the window's aliasing is at most 1.6e-7 (5e-8 rms) of the largest
 // amplitude near the run, the FP32 transform adds about as much; both are

@@ -904,59 +904,79 @@ __device__ __forceinline__ float lsp_power_f32(float xc, float xs, float cc, flo
 // The transform (lsp_transform.cu) accumulates its grid cells in 32-bit fixed
 // point.  An observation's window covers 8 cells, so at most two neighbouring
 // groups of 8, and window values are <= 1: a cell's magnitude is at most the
-// largest count of two neighbouring groups times the largest weight.  The
-// scales put that at 2^30, half the range, and are capped so that their
-// inverses stay normal numbers.  W's observations sit at twice the phase.
+// sum of |weight| over two neighbouring groups.  The scales put the largest of
+// these sums at 2^30, half the range, and are capped so that their inverses
+// stay normal numbers.  W's observations sit at twice the phase.
+//
+// The sums, not counts times the largest weight: with one error bar 100 times
+// smaller than the rest that bound leaves the others a few units each, or
+// none (generalized periodogram, 2000 observations in a month: powers wrong
+// by 8e-4, by 8e-7 with the sums, by 2e-6 in the direct kernel's FP32 sums).
+//
+// The groups add integers, so the sums do not depend on the order: weights are
+// rounded up in units of 2^-30 of a power of two that bounds the sum of all of
+// them, sum |u| <= sqrt(sum w sum w y^2) < 2^e (u = w y; plain: w = 1).
 constexpr int kTfGroups = 512;
 struct TfScale {
   float y, w, c;  // Z, W and (generalized) C
 };
-__device__ __forceinline__ void tf_count(uint32_t* count, uint32_t y_bits, uint32_t w_bits, uint32_t b_hi,
-                                         uint32_t b_lo, uint32_t& ymax, uint32_t& wmax) {
-  const uint32_t ya = y_bits & 0x7fffffffu;  // magnitudes' bits order like integers
-  ymax = ya > ymax ? ya : ymax;
-  wmax = w_bits > wmax ? w_bits : wmax;
-  const uint32_t b2 = (b_hi << 1) | (b_lo >> 31);
-  atomicAdd(&count[b_hi >> 23], 1u);
-  atomicAdd(&count[kTfGroups + (b2 >> 23)], 1u);
+__device__ __forceinline__ float tf_pow2(int e) {
+  return __int_as_float((min(max(e, -126), 127) + 127) << 23);
 }
-// The scales from the CTA's counts (complete) and each thread's largest
-// weights; every thread of the NW warps gets them.
-template <int NW>
-__device__ __forceinline__ TfScale tf_scale_block(const uint32_t* count, uint32_t ymax, uint32_t wmax,
-                                                  uint32_t (*s_max)[NW]) {
-  uint32_t cz = 1u, cw = 1u;
-  for (int g = threadIdx.x; g < kTfGroups; g += 32 * NW) {
-    const int g1 = (g + 1) & (kTfGroups - 1);
-    cz = max(cz, count[g] + count[g1]);
-    cw = max(cw, count[kTfGroups + g] + count[kTfGroups + g1]);
+__device__ __forceinline__ int tf_exponent(double v) {  // v < 2^tf_exponent(v)
+  return ((int)(__double_as_longlong(v) >> 52) & 0x7ff) - 1022;
+}
+template <bool GLS>
+struct TfCounter {
+  static constexpr int kWords = (GLS ? 3 : 2) * kTfGroups;  // |y| (or |u|), W, C
+  uint32_t* count;      // zero on entry
+  float y_unit, w_unit; // integers per unit of |u| and w
+  uint32_t bad = 0u;    // a weight is not finite
+  __device__ __forceinline__ TfCounter(uint32_t* c, const ObjInfo& oi) : count(c) {
+    const int ew = tf_exponent(oi.wsum), eu = (ew + tf_exponent(oi.sum_y2) + 1) >> 1;
+    y_unit = tf_pow2(30 - eu);
+    w_unit = tf_pow2(30 - ew);
   }
-  cz = __reduce_max_sync(0xffffffffu, cz);
-  cw = __reduce_max_sync(0xffffffffu, cw);
-  ymax = __reduce_max_sync(0xffffffffu, ymax);
-  wmax = __reduce_max_sync(0xffffffffu, wmax);
-  const int warp = threadIdx.x >> 5;
-  if ((threadIdx.x & 31) == 0) {
-    s_max[0][warp] = cz;
-    s_max[1][warp] = cw;
-    s_max[2][warp] = ymax;
-    s_max[3][warp] = wmax;
+  __device__ __forceinline__ void add(float y, float w, uint32_t b_hi, uint32_t b_lo) {
+    const uint32_t b2 = (b_hi << 1) | (b_lo >> 31);
+    const float ya = fabsf(y);
+    bad |= !(ya <= 3.4028234664e38f);
+    atomicAdd(&count[b_hi >> 23], __float2uint_ru(ya * y_unit));
+    if constexpr (GLS) {
+      bad |= !(w <= 3.4028234664e38f);
+      const uint32_t q = __float2uint_ru(w * w_unit);
+      atomicAdd(&count[kTfGroups + (b2 >> 23)], q);
+      atomicAdd(&count[2 * kTfGroups + (b_hi >> 23)], q);
+    } else {
+      atomicAdd(&count[kTfGroups + (b2 >> 23)], 1u);
+    }
   }
-  __syncthreads();
+  // The scales, once the sums of all NW warps are complete; every thread gets
+  // them.  0 where a weight is not finite: every power is then 0, which is
+  // what the direct kernel's sums give.
+  template <int NW>
+  __device__ __forceinline__ TfScale scale(uint32_t (*s_max)[NW]) const {
+    uint32_t c[4] = {1u, 1u, 1u, bad};
 #pragma unroll
-  for (int i = 0; i < NW; ++i) {
-    cz = max(cz, s_max[0][i]);
-    cw = max(cw, s_max[1][i]);
-    ymax = max(ymax, s_max[2][i]);
-    wmax = max(wmax, s_max[3][i]);
+    for (int a = 0; a < kWords / kTfGroups; ++a)
+      for (int g = threadIdx.x; g < kTfGroups; g += 32 * NW)
+        c[a] = max(c[a], count[a * kTfGroups + g] + count[a * kTfGroups + ((g + 1) & (kTfGroups - 1))]);
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+      c[a] = __reduce_max_sync(0xffffffffu, c[a]);
+      if ((threadIdx.x & 31) == 0) s_max[a][threadIdx.x >> 5] = c[a];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int i = 0; i < NW; ++i) c[a] = max(c[a], s_max[a][i]);
+    if (c[3]) return TfScale{0.0f, 0.0f, 0.0f};
+    const float top = 1073741824.0f, unit = GLS ? w_unit : 1.0f;
+    return TfScale{fminf(top / (float)c[0] * y_unit, 1e37f), fminf(top / (float)c[1] * unit, 1e37f),
+                   fminf(top / (float)c[2] * unit, 1e37f)};
   }
-  const float top = 1073741824.0f;
-  TfScale s;
-  s.y = fminf(top / __uint_as_float(ymax) / (float)cz, 1e37f);
-  s.w = fminf(top / __uint_as_float(wmax) / (float)cw, 1e37f);
-  s.c = fminf(top / __uint_as_float(wmax) / (float)cz, 1e37f);
-  return s;
-}
+};
 // Once the records are written an object's t0 and mean are not read again:
 // the records kernel leaves the scales in their place.
 __device__ __forceinline__ void tf_scale_put(ObjInfo* oi, TfScale s) {

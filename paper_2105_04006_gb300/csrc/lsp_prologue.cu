@@ -350,21 +350,20 @@ __global__ void records_kernel(const double* __restrict__ t, const YT* __restric
     for (int64_t j = lo + threadIdx.x; j < hi; j += blockDim.x)
       make_record<YT, Rec, GLS>(t, y, dy, j, oi, f_min, df, rec);
   } else {
-    __shared__ uint32_t count[2 * kTfGroups];
+    __shared__ uint32_t count[TfCounter<GLS>::kWords];
     __shared__ uint32_t s_max[4][kRecThreads / 32];
     const bool scaled = oi.n >= tf_min;
     if (scaled)
-      for (int i = threadIdx.x; i < 2 * kTfGroups; i += kRecThreads) count[i] = 0u;
+      for (int i = threadIdx.x; i < TfCounter<GLS>::kWords; i += kRecThreads) count[i] = 0u;
     __syncthreads();
-    uint32_t ymax = 0u, wmax = GLS ? 0u : 0x3f800000u;
+    TfCounter<GLS> counter(count, oi);
     for (int64_t j = lo + threadIdx.x; j < hi; j += kRecThreads) {
       const Rec r = make_record<YT, Rec, GLS>(t, y, dy, j, oi, f_min, df, rec);
-      if (scaled)
-        tf_count(count, __float_as_uint(r.y), GLS ? r.pad : 0x3f800000u, r.b_hi, r.b_lo, ymax, wmax);
+      if (scaled) counter.add(r.y, __uint_as_float(r.pad), r.b_hi, r.b_lo);
     }
     if (!scaled) return;
     __syncthreads();
-    const TfScale s = tf_scale_block<kRecThreads / 32>(count, ymax, wmax, s_max);
+    const TfScale s = counter.template scale<kRecThreads / 32>(s_max);
     if (threadIdx.x == 0) tf_scale_put(obj + blockIdx.x, s);
   }
 }

@@ -36,8 +36,9 @@
 //     not depend on the order of the adds (bit-identical repeats), any time
 //     order and any clustering of the observations run at the same speed,
 //     and 8 lanes per observation hit 8 consecutive banks.  The scale is the
-//     largest one that cannot overflow: cells 8 wide are counted first, and
-//     an observation's window covers at most two neighbouring ones;
+//     largest one that cannot overflow: |weights| are summed per 8 cells
+//     first, and an observation's window covers at most two neighbouring
+//     groups (TfCounter);
 //   - lane r of an octet always adds the r-th cell, so the window polynomial
 //     of its cell stays in 9 registers;
 //   - 4096 = 16^3: three register passes of 16 points per thread with two
@@ -72,7 +73,7 @@ __device__ __forceinline__ f2_t cells_f2(const int32_t* a, const int32_t* b, int
 }
 
 // Shared memory: grid planes (the exchange buffer after the grid is read),
-// staged observations (group counts before, the run's powers after them).
+// staged observations (group sums before, the run's powers after them).
 template <bool GLS>
 struct Smem {
   static constexpr int kPlanes = GLS ? 6 : 4;
@@ -80,7 +81,7 @@ struct Smem {
   static constexpr size_t grid = (size_t)kPlanes * kM * 4;
   static constexpr size_t stage = (size_t)kThreads * kStage > kPowers * 4 ? (size_t)kThreads * kStage : kPowers * 4;
   static constexpr size_t total = grid + stage;
-  static_assert(stage >= 2 * kTfGroups * 4, "the counts use the staging area");
+  static_assert(stage >= TfCounter<GLS>::kWords * 4, "the group sums use the staging area");
 };
 
 template <bool GLS>
@@ -129,15 +130,15 @@ __global__ void __launch_bounds__(kThreads, GLS ? 2 : 3) transform_kernel(Transf
       sc = tf_scale_of(oi);
     } else {
       uint32_t* const count = reinterpret_cast<uint32_t*>(stage);
-      for (int i = tid; i < 2 * kTfGroups; i += kThreads) count[i] = 0u;
+      for (int i = tid; i < TfCounter<GLS>::kWords; i += kThreads) count[i] = 0u;
       __syncthreads();
-      uint32_t ymax = 0u, wmax = GLS ? 0u : 0x3f800000u;
+      TfCounter<GLS> counter(count, oi);
       for (uint32_t j = tid; j < (uint32_t)n; j += kThreads) {
         const uint4 r0 = __ldg(rec + 2 * (size_t)j), r1 = __ldg(rec + 2 * (size_t)j + 1);
-        tf_count(count, r0.x, GLS ? r1.w : 0x3f800000u, r1.x, r1.y, ymax, wmax);
+        counter.add(__uint_as_float(r0.x), __uint_as_float(r1.w), r1.x, r1.y);
       }
       __syncthreads();
-      sc = tf_scale_block<kWarps>(count, ymax, wmax, s_max);  // its barriers end the use of the counts
+      sc = counter.template scale<kWarps>(s_max);  // its barrier ends the use of the sums
     }
     const float y_sc = sc.y, w_sc = sc.w, c_sc = sc.c;
 

@@ -68,6 +68,33 @@ constexpr int kWarps = kThreads / 32;
 constexpr size_t kPowers = kTfBins + kTfBins / 8;
 static_assert(kTfBins == kM / 2 && kTfBins == kThreads * 8 && kTfGroups == kM / 8, "run length");
 
+// Objects of many observations add their window values with an offset in
+// (-1/2, 1/2) before the rounding, different for every value and set by its
+// index alone.  A unit of a cell is up to N 2^-30 of one observation's weight:
+// rounded to nearest, the window's tails lose up to half a unit each, in the
+// same direction where the observations share few cells, and the error of a
+// sum grows like N / 2^30 of it; with the offsets the errors cancel and it
+// grows like sqrt(N).  Emulated, 1e6 observations in a month: error of a power
+// 3.8e-5 without, 1.7e-6 with the offsets (direct kernel 1.2e-5; generalized,
+// lognormal errors: 8.4e-5, 1.6e-6, 2.3e-3).  At 4096 the two are level.
+constexpr int kTfOffsets = 4096;
+__device__ __forceinline__ uint32_t scramble(uint32_t x) {
+  x *= 0x9e3779b1u;  // 2^32 / golden ratio
+  x ^= x >> 16;
+  x *= 0x9e3779b1u;
+  return x ^ (x >> 15);
+}
+__device__ __forceinline__ void rounding_offsets(uint32_t i, float (&d)[6]) {
+  const uint32_t x = scramble(i), z = scramble(x + 1u);
+  auto byte = [](uint32_t v) { return __uint_as_float(0x3f800000u | (v & 0xffu) << 15) - 1.498046875f; };
+  d[0] = byte(x);
+  d[1] = byte(x >> 8);
+  d[2] = byte(x >> 16);
+  d[3] = byte(x >> 24);
+  d[4] = byte(z);
+  d[5] = byte(z >> 8);
+}
+
 __device__ __forceinline__ f2_t cells_f2(const int32_t* a, const int32_t* b, int i) {
   return f2_pack(__int2float_rn(a[i]), __int2float_rn(b[i]));
 }
@@ -153,54 +180,60 @@ __global__ void __launch_bounds__(kThreads, GLS ? 2 : 3) transform_kernel(Transf
       for (int d = 0; d < 9; ++d) poly[d] = dup_<f2_t>(__ldg(&kTfPoly[d * 8 + (lane & 7)]));
       const uint32_t j1 = (uint32_t)((int64_t)n * (warp + 1) / kWarps);
       unsigned char* const mine = stage + (size_t)warp * 32 * S::kStage;
-      for (uint32_t jb = (uint32_t)((int64_t)n * warp / kWarps); jb < j1; jb += 32) {
-        const uint32_t j = jb + lane;
-        if (j < j1) {
-          const uint4 r0 = __ldg(rec + 2 * (size_t)j), r1 = __ldg(rec + 2 * (size_t)j + 1);
-          const uint32_t ph = phase_hi32(r0.w, r1.x, r1.y, kc);
-          float s, c;
-          sincospif(__int2float_rn((int)ph) * 4.656612873077393e-10f, &s, &c);  // 2^-31 half-cycles
-          const float ys = __uint_as_float(r0.x) * y_sc;
-          const float ws = GLS ? __uint_as_float(r1.w) * w_sc : w_sc;
-          // position in cells, 12 bits of cell and 32 of fraction
-          const uint32_t fz = (r1.x << 12) | (r1.y >> 20), b2 = (r1.x << 1) | (r1.y >> 31), lo2 = r1.y << 1;
-          const uint32_t fw = (b2 << 12) | (lo2 >> 20);
-          const float uz = fmaf(__uint2float_rn(fz), 2.3283064365386963e-10f, -0.5f);
-          const float uw = fmaf(__uint2float_rn(fw), 2.3283064365386963e-10f, -0.5f);
-          float4* st = reinterpret_cast<float4*>(mine) + lane;  // word w of an observation at 32 w: no bank twice
-          st[0] = make_float4(uz, uw, __uint_as_float((r1.x >> 20) - 3u), __uint_as_float((b2 >> 20) - 3u));
-          st[32] = make_float4(ys * c, ys * s, ws * (c - s) * (c + s), ws * 2.0f * c * s);
-          if (GLS) {
-            const float cs = __uint_as_float(r1.w) * c_sc;
-            st[64] = make_float4(cs * c, cs * s, 0.0f, 0.0f);
+      auto spread = [&](auto offsets) {
+        for (uint32_t jb = (uint32_t)((int64_t)n * warp / kWarps); jb < j1; jb += 32) {
+          const uint32_t j = jb + lane;
+          if (j < j1) {
+            const uint4 r0 = __ldg(rec + 2 * (size_t)j), r1 = __ldg(rec + 2 * (size_t)j + 1);
+            const uint32_t ph = phase_hi32(r0.w, r1.x, r1.y, kc);
+            float s, c;
+            sincospif(__int2float_rn((int)ph) * 4.656612873077393e-10f, &s, &c);  // 2^-31 half-cycles
+            const float ys = __uint_as_float(r0.x) * y_sc;
+            const float ws = GLS ? __uint_as_float(r1.w) * w_sc : w_sc;
+            // position in cells, 12 bits of cell and 32 of fraction
+            const uint32_t fz = (r1.x << 12) | (r1.y >> 20), b2 = (r1.x << 1) | (r1.y >> 31), lo2 = r1.y << 1;
+            const uint32_t fw = (b2 << 12) | (lo2 >> 20);
+            const float uz = fmaf(__uint2float_rn(fz), 2.3283064365386963e-10f, -0.5f);
+            const float uw = fmaf(__uint2float_rn(fw), 2.3283064365386963e-10f, -0.5f);
+            float4* st = reinterpret_cast<float4*>(mine) + lane;  // word w of an observation at 32 w: no bank twice
+            st[0] = make_float4(uz, uw, __uint_as_float((r1.x >> 20) - 3u), __uint_as_float((b2 >> 20) - 3u));
+            st[32] = make_float4(ys * c, ys * s, ws * (c - s) * (c + s), ws * 2.0f * c * s);
+            if (GLS) {
+              const float cs = __uint_as_float(r1.w) * c_sc;
+              st[64] = make_float4(cs * c, cs * s, 0.0f, 0.0f);
+            }
           }
-        }
-        __syncwarp();
-        const int nt = (int)min(32u, j1 - jb);
+          __syncwarp();
+          const int nt = (int)min(32u, j1 - jb);
 #pragma unroll 2
-        for (int i = lane >> 3; i < nt; i += 4) {
-          const float4* st = reinterpret_cast<const float4*>(mine) + i;
-          const float4 at = st[0], v = st[32];
-          const f2_t u = f2_pack(at.x, at.y);
-          f2_t w2 = poly[8];
+          for (int i = lane >> 3; i < nt; i += 4) {
+            const float4* st = reinterpret_cast<const float4*>(mine) + i;
+            const float4 at = st[0], v = st[32];
+            const f2_t u = f2_pack(at.x, at.y);
+            f2_t w2 = poly[8];
 #pragma unroll
-          for (int d = 7; d >= 0; --d) w2 = f2_fma(w2, u, poly[d]);
-          float wz, ww;
-          f2_unpack(w2, wz, ww);
-          const int lz = (int)(__float_as_uint(at.z) + (uint32_t)(lane & 7)) & (kM - 1);
-          const int lw = (int)(__float_as_uint(at.w) + (uint32_t)(lane & 7)) & (kM - 1);
-          atomicAdd(&plane[0 * kM + lz], __float2int_rn(wz * v.x));
-          atomicAdd(&plane[1 * kM + lz], __float2int_rn(wz * v.y));
-          atomicAdd(&plane[kW * kM + lw], __float2int_rn(ww * v.z));
-          atomicAdd(&plane[(kW + 1) * kM + lw], __float2int_rn(ww * v.w));
-          if (GLS) {
-            const float4 q = st[64];
-            atomicAdd(&plane[2 * kM + lz], __float2int_rn(wz * q.x));
-            atomicAdd(&plane[3 * kM + lz], __float2int_rn(wz * q.y));
+            for (int d = 7; d >= 0; --d) w2 = f2_fma(w2, u, poly[d]);
+            float wz, ww;
+            f2_unpack(w2, wz, ww);
+            const int lz = (int)(__float_as_uint(at.z) + (uint32_t)(lane & 7)) & (kM - 1);
+            const int lw = (int)(__float_as_uint(at.w) + (uint32_t)(lane & 7)) & (kM - 1);
+            float d[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+            if constexpr (decltype(offsets)::value) rounding_offsets(8u * (jb + i) + (lane & 7), d);
+            atomicAdd(&plane[0 * kM + lz], __float2int_rn(fmaf(wz, v.x, d[0])));
+            atomicAdd(&plane[1 * kM + lz], __float2int_rn(fmaf(wz, v.y, d[1])));
+            atomicAdd(&plane[kW * kM + lw], __float2int_rn(fmaf(ww, v.z, d[2])));
+            atomicAdd(&plane[(kW + 1) * kM + lw], __float2int_rn(fmaf(ww, v.w, d[3])));
+            if (GLS) {
+              const float4 q = st[64];
+              atomicAdd(&plane[2 * kM + lz], __float2int_rn(fmaf(wz, q.x, d[4])));
+              atomicAdd(&plane[3 * kM + lz], __float2int_rn(fmaf(wz, q.y, d[5])));
+            }
           }
+          __syncwarp();
         }
-        __syncwarp();
-      }
+      };
+      if (n < kTfOffsets) spread(std::false_type{});  // two loops: the test inside one took 0.5 % of a batch's time
+      else spread(std::true_type{});
     }
     __syncthreads();
 

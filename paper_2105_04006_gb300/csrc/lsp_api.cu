@@ -667,21 +667,38 @@ void drop_graph(lsp_plan* p) {
   for (auto& a : p->cap_args) a = nullptr;
 }
 
+// Room for `bytes` in the plan's workspace.  Where it cannot be had the plan
+// keeps the workspace it has (or, if even that was lost to another allocation
+// in between, none: ws_cap 0, which lsp_plan_execute tries to mend).
 lsp_status ensure_ws(lsp_plan* p, size_t bytes) {
-  if (bytes <= p->ws_cap) return LSP_OK;
-  drop_graph(p);  // a captured graph may reference the old workspace
+  if (p->ws && bytes <= p->ws_cap) return LSP_OK;
+  const size_t size = bytes ? bytes : kAlign, had = p->ws_cap;
+  char* ws = nullptr;
+  cudaError_t e = cudaMalloc(&ws, size);
+  if (e == cudaSuccess || p->ws) drop_graph(p);  // a captured graph may reference the old workspace
   if (p->ws) {
     cudaDeviceSynchronize();
     cudaFree(p->ws);
+    p->ws = nullptr;
+    p->ws_cap = 0;
   }
-  p->ws = nullptr;
-  p->ws_cap = 0;
-  if (cudaMalloc(&p->ws, bytes ? bytes : kAlign) != cudaSuccess) {
+  if (e != cudaSuccess) {  // not beside the old one: in its place
     cudaGetLastError();
-    return fail(LSP_E_NOMEM, "plan workspace of %zu bytes", bytes);
+    e = cudaMalloc(&ws, size);
   }
-  p->ws_cap = bytes;
-  return LSP_OK;
+  if (e == cudaSuccess) {
+    p->ws = ws;
+    p->ws_cap = size;
+    return LSP_OK;
+  }
+  cudaGetLastError();
+  if (had && cudaMalloc(&p->ws, had) == cudaSuccess) {
+    p->ws_cap = had;
+  } else {
+    cudaGetLastError();
+    p->ws = nullptr;
+  }
+  return fail(LSP_E_NOMEM, "plan workspace of %zu bytes", bytes);
 }
 
 lsp_status apply_config(lsp_plan* p, const lsp_config* c) {
@@ -1044,6 +1061,7 @@ lsp_status lsp_plan_execute(lsp_plan* p, const double* t, const void* y, const i
   lsp_status st = check_io(p->total_nt, t, y);
   if (st) return st;
   if (p->n_obj > 1 && !offsets) return fail(LSP_E_ARG, "offsets must not be NULL");
+  if ((st = ensure_ws(p, p->L.total))) return st;
   const void* args[5] = {t, y, offsets, power_out, peaks};
   bool same = p->exec != nullptr;
   for (int i = 0; i < 5 && same; ++i) same = args[i] == p->cap_args[i];
@@ -1218,7 +1236,7 @@ lsp_status lsp_plan_autotune_ex(lsp_plan* p, const double* t, const void* y, con
   std::vector<int> splits = {0};
   if (p->n_obj == 1) {
     Layout L0;
-    if ((st = resolve(1, p->total_nt, &p->grid, &p->opts, nullptr, &L0))) return st;
+    if ((st = resolve(1, p->total_nt, &p->grid, &p->opts, nullptr, &L0, false, p->level))) return st;
     for (int f : {2, 4}) {
       if (L0.split * f <= kMaxSplit && p->total_nt / (L0.split * f) >= kMinObsPerSplit)
         splits.push_back(L0.split * f);
@@ -1373,23 +1391,37 @@ lsp_status lsp_plan_autotune_ex(lsp_plan* p, const double* t, const void* y, con
     cudaFree(gws);
   };
   const int64_t g_nobj = p->n_obj == 1 ? 1 : g_rows;
+  int g_level = p->level;  // paths the gate's scratch has room for
   if (gate) {
-    Layout L64;
-    if ((st = resolve(g_nobj, g_total, &p->grid, &o64, nullptr, &L64))) return st;
-    gws_bytes = L64.total;
-    for (const auto& c : cands) {  // room for every candidate's layout too
-      Layout Lc;
-      if (!resolve(g_nobj, g_total, &p->grid, &o1, &c, &Lc) && Lc.total > gws_bytes) gws_bytes = Lc.total;
-    }
-    g_err.clear();
     const size_t rows = (size_t)g_rows;
     if (cudaMalloc(&ref, rows * p->grid.n_f * sizeof(double)) || cudaMalloc(&y64, g_total * sizeof(double)) ||
         cudaMalloc(&gt, g_total * sizeof(double)) || cudaMalloc(&gy, g_total * sizeof(float)) ||
         cudaMalloc(&goff, (rows + 1) * sizeof(int64_t)) || cudaMalloc(&pw, rows * p->grid.n_f * sizeof(float)) ||
-        cudaMalloc(&d_err, rows * sizeof(double)) || cudaMalloc(&gws, gws_bytes)) {
+        cudaMalloc(&d_err, rows * sizeof(double))) {
       cudaGetLastError();
       cleanup();
       return fail(LSP_E_NOMEM, "autotune scratch");
+    }
+    Layout L64;
+    for (;; ++g_level) {
+      if ((st = resolve(g_nobj, g_total, &p->grid, &o64, nullptr, &L64, false, g_level))) {
+        cleanup();
+        return st;
+      }
+      gws_bytes = L64.total;
+      for (const auto& c : cands) {  // room for every candidate's layout too
+        Layout Lc;
+        if (!resolve(g_nobj, g_total, &p->grid, &o1, &c, &Lc, false, g_level) && Lc.total > gws_bytes)
+          gws_bytes = Lc.total;
+      }
+      g_err.clear();
+      if (cudaMalloc(&gws, gws_bytes) == cudaSuccess) break;
+      cudaGetLastError();
+      gws = nullptr;
+      if (g_level + 1 >= kLevels) {
+        cleanup();
+        return fail(LSP_E_NOMEM, "autotune scratch");
+      }
     }
     std::vector<int64_t> hoff(rows + 1, 0);
     cudaError_t e = cudaSuccess;
@@ -1430,13 +1462,14 @@ lsp_status lsp_plan_autotune_ex(lsp_plan* p, const double* t, const void* y, con
   };
   for (const auto& c : cands) {
     Layout Lc;
-    if (resolve(p->n_obj, p->total_nt, &p->grid, &p->opts, &c, &Lc)) { g_err.clear(); continue; }
+    if (resolve(p->n_obj, p->total_nt, &p->grid, &p->opts, &c, &Lc, false, p->level)) { g_err.clear(); continue; }
     double err = 0.0;
     int64_t worst_obj = -1;
     if (gate) {
       // the candidate's own configuration (a single object keeps its split)
       Layout Lg;
-      if (resolve(g_nobj, g_total, &p->grid, &o1, &c, &Lg)) { g_err.clear(); continue; }
+      if (resolve(g_nobj, g_total, &p->grid, &o1, &c, &Lg, false, g_level)) { g_err.clear(); continue; }
+      if ((Lc.tf && !Lg.tf) || (Lc.lng && !Lg.lng)) continue;  // the gate has no room for this path
       if ((st = run(Lg, gt, gy, g_nobj > 1 ? goff : nullptr, pw, nullptr, gws, s))) { cleanup(); return st; }
       cudaError_t e = launch_row_max_abs_diff(pw, ref, g_rows, p->grid.n_f, d_err, s);
       if (e == cudaSuccess)
@@ -1453,7 +1486,12 @@ lsp_status lsp_plan_autotune_ex(lsp_plan* p, const double* t, const void* y, con
         continue;
       }
     }
-    if ((st = ensure_ws(p, Lc.total))) { cleanup(); return st; }
+    if (ensure_ws(p, Lc.total)) {  // no room for this candidate
+      g_err.clear();
+      if (p->ws) continue;
+      cleanup();
+      return fail(LSP_E_NOMEM, "plan workspace");
+    }
     Layout saved = p->L;
     p->L = Lc;
     float ms = 0.f;

@@ -569,14 +569,14 @@ class Plan:
             _check(lib().lsp_plan_autotune(self._h, _ptr(t), _ptr(y), _ptr(offsets), cp,
                                            _stream_handle(t.device)))
             return self.config
-        buf = (Trial * 64)()
+        buf = (Trial * 256)()  # one object: 5 splits of 14 kernels, 10 ablations each, and the transform
         n = ctypes.c_int32(0)
         _check(lib().lsp_plan_autotune_ex(self._h, _ptr(t), _ptr(y), _ptr(offsets), cp,
-                                          TUNE_ABLATIONS if ablations else 0, buf, 64, ctypes.byref(n),
+                                          TUNE_ABLATIONS if ablations else 0, buf, 256, ctypes.byref(n),
                                           _stream_handle(t.device)))
         trials = [dict(config=buf[i].config.as_dict(), ms=float(buf[i].ms), max_err=float(buf[i].max_err),
                        passed=bool(buf[i].passed), worst_object=int(buf[i].worst_object))
-                  for i in range(min(n.value, 64))]
+                  for i in range(min(n.value, 256))]
         return (self.config, trials) if return_trials else self.config
 
     def gate_report(self):

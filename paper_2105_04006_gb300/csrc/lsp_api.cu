@@ -1237,10 +1237,10 @@ lsp_status lsp_plan_autotune_ex(lsp_plan* p, const double* t, const void* y, con
   if (p->n_obj == 1) {
     Layout L0;
     if ((st = resolve(1, p->total_nt, &p->grid, &p->opts, nullptr, &L0, false, p->level))) return st;
+    const int split = config_of(L0).obs_split;  // the direct kernel's own
     for (int f : {2, 4}) {
-      if (L0.split * f <= kMaxSplit && p->total_nt / (L0.split * f) >= kMinObsPerSplit)
-        splits.push_back(L0.split * f);
-      if (L0.split / f >= 1) splits.push_back(L0.split / f);
+      if (split * f <= kMaxSplit && p->total_nt / (split * f) >= kMinObsPerSplit) splits.push_back(split * f);
+      if (split / f >= 1) splits.push_back(split / f);
     }
   }
   for (int sp : splits) {

@@ -41,8 +41,8 @@ def runs(h, args, n_peaks):
     assert st == 0 and fake.fake_launches() > before, (st, L.lsp_last_error())
     assert fake.fake_outside() == 0
 def trials_of(h, args):
-    buf, n = (lsp.Trial * 64)(), ctypes.c_int32(0)
-    st = L.lsp_plan_autotune_ex(h, *args, None, 0, buf, 64, ctypes.byref(n), None)
+    buf, n = (lsp.Trial * 256)(), ctypes.c_int32(0)
+    st = L.lsp_plan_autotune_ex(h, *args, None, 0, buf, 256, ctypes.byref(n), None)
     return st, [buf[i] for i in range(n.value)]
 """
 
@@ -127,4 +127,20 @@ def test_autotune_skips_candidates_that_do_not_fit(fake):
     assert st == 0, L.lsp_last_error()
     assert 0 < len(some) <= len(every)
     runs(h, args, 50)
+    """)
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_autotune_tries_splits_around_the_direct_kernels_own(fake, precision):
+    """One object: also where the transform, which has no split, is the default."""
+    fake(f"""
+    g = lsp.Grid(0.1, 10.0, 60_000)
+    args = inputs([9000], np.float64 if "{precision}" == "fp64" else np.float32)
+    st, h = plan([9000], g, precision="{precision}")
+    c = lsp.Config()
+    assert st == 0 and L.lsp_plan_get_config(h, ctypes.byref(c)) == 0 and c.obs_split >= 8
+    st, trials = trials_of(h, args)
+    assert st == 0, L.lsp_last_error()
+    tried = set(t.config.obs_split for t in trials)
+    assert tried >= set(c.obs_split * f // 4 for f in (1, 2, 4, 8, 16)), (tried, c.obs_split)
     """)

@@ -379,9 +379,12 @@ lsp_status lsp_plan_autotune_ex(lsp_plan* plan, const double* t, const void* y, 
 /*
  * The last lsp_plan_autotune(_ex) error gate: its objects (batch indices,
  * into objects) and, for the configuration it chose, each object's
- * max |P_n - P_n(FP64)| with the direct kernel of that configuration (into
- * max_err), at most cap of each; *n = the number of gate objects (0 after a
- * cache hit or for FP64 plans).  Host only.
+ * max |P_n - P_n(FP64)| (into max_err), at most cap of each; *n = the number
+ * of gate objects (0 after a cache hit or for FP64 plans).  A batch whose
+ * configuration runs the transform has two kernels, the transform for objects
+ * of enough observations and the direct kernel for the others: both are gated
+ * on every gate object, and the larger error is reported, here and in the
+ * trial.  Host only.
  */
 lsp_status lsp_plan_gate_report(const lsp_plan* plan, int64_t* objects, float* max_err, int32_t cap,
                                 int32_t* n);

@@ -580,7 +580,8 @@ class Plan:
         return (self.config, trials) if return_trials else self.config
 
     def gate_report(self):
-        """The last autotune's error gate: [(object index, max |P_n - P_n(FP64)|)] for the chosen configuration."""
+        """The last autotune's error gate: [(object index, max |P_n - P_n(FP64)|)] for the chosen configuration;
+        of a batch that runs the transform beside a direct kernel, the larger of the two kernels' errors."""
         objs = (ctypes.c_int64 * 8)()
         errs = (ctypes.c_float * 8)()
         n = ctypes.c_int32(0)

@@ -1440,7 +1440,7 @@ lsp_status lsp_plan_autotune_ex(lsp_plan* p, const double* t, const void* y, con
     if (e != cudaSuccess) { cleanup(); return cuda_fail(e, "autotune gate inputs"); }
     if ((st = run(L64, gt, y64, g_nobj > 1 ? goff : nullptr, ref, nullptr, gws, s))) { cleanup(); return st; }
   }
-  std::vector<double> cur_err((size_t)g_rows), best_obj_err, direct_err;
+  std::vector<double> cur_err((size_t)g_rows), best_obj_err;
 
   float best_ms = 1e30f;
   double best_err = 0.0;
@@ -1470,12 +1470,29 @@ lsp_status lsp_plan_autotune_ex(lsp_plan* p, const double* t, const void* y, con
       Layout Lg;
       if (resolve(g_nobj, g_total, &p->grid, &o1, &c, &Lg, false, g_level)) { g_err.clear(); continue; }
       if ((Lc.tf && !Lg.tf) || (Lc.lng && !Lg.lng)) continue;  // the gate has no room for this path
-      if ((st = run(Lg, gt, gy, g_nobj > 1 ? goff : nullptr, pw, nullptr, gws, s))) { cleanup(); return st; }
-      cudaError_t e = launch_row_max_abs_diff(pw, ref, g_rows, p->grid.n_f, d_err, s);
-      if (e == cudaSuccess)
-        e = cudaMemcpyAsync(cur_err.data(), d_err, cur_err.size() * sizeof(double), cudaMemcpyDeviceToHost, s);
-      if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-      if (e != cudaSuccess) { cleanup(); return cuda_fail(e, "autotune gate"); }
+      auto errors = [&](const Layout& l, std::vector<double>& out) -> lsp_status {
+        const lsp_status r = run(l, gt, gy, g_nobj > 1 ? goff : nullptr, pw, nullptr, gws, s);
+        if (r) return r;
+        cudaError_t e = launch_row_max_abs_diff(pw, ref, g_rows, p->grid.n_f, d_err, s);
+        if (e == cudaSuccess)
+          e = cudaMemcpyAsync(out.data(), d_err, out.size() * sizeof(double), cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        return e == cudaSuccess ? LSP_OK : cuda_fail(e, "autotune gate");
+      };
+      if ((st = errors(Lg, cur_err))) { cleanup(); return st; }
+      if (Lg.tf && g_nobj > 1) {  // and the direct kernel that serves the batch's short objects
+        lsp_config cd = c;
+        cd.reserved = 0;
+        Layout Ld;
+        std::vector<double> direct((size_t)g_rows);
+        if (resolve(g_nobj, g_total, &p->grid, &o1, &cd, &Ld, false, g_level) || Ld.total > gws_bytes) {
+          g_err.clear();
+          continue;
+        }
+        if ((st = errors(Ld, direct))) { cleanup(); return st; }
+        for (size_t i = 0; i < direct.size(); ++i)
+          if (!(direct[i] <= cur_err[i])) cur_err[i] = direct[i];
+      }
       for (size_t i = 0; i < gobj.size(); ++i)
         if (!(cur_err[i] <= err)) {  // NaN counts as the worst
           err = std::isnan(cur_err[i]) ? INFINITY : cur_err[i];
@@ -1499,13 +1516,6 @@ lsp_status lsp_plan_autotune_ex(lsp_plan* p, const double* t, const void* y, con
     p->L = saved;
     if (st) { cleanup(); return st; }
     record(config_of(Lc), ms, err, true, worst_obj);
-    // the report describes the direct kernel of the configuration, also
-    // where the transform, gated above like every candidate, is chosen
-    const lsp_config cc = config_of(Lc), ct = cands.back();
-    if (ct.reserved && !cc.reserved && cc.k_reseed == ct.k_reseed && cc.freqs_per_thread == ct.freqs_per_thread &&
-        cc.block_threads == ct.block_threads && cc.packed == ct.packed && !cc.trig && !cc.staging)
-      direct_err = cur_err;
-    if (cc.reserved && !direct_err.empty()) cur_err = direct_err;
     if (ms < best_ms) {
       best_ms = ms;
       best = config_of(Lc);

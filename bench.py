@@ -578,7 +578,8 @@ def run_ablations(args, lsp, torch, plan, b, t, y, off, name, rank):
     rows = []
     for tr in trials:
         c = tr["config"]
-        kind = ("recurrence", "SFU sincos per pair", "accurate sincospif per pair")[c["trig"]]
+        kind = ("transform" if c["transform"] else
+                ("recurrence", "SFU sincos per pair", "accurate sincospif per pair")[c["trig"]])
         rows.append({"config": c, "trig": kind, "staging": ("shared", "global")[c["staging"]],
                      "ms_per_step": tr["ms"], "pairs_per_s": pairs / (tr["ms"] * 1e-3) if tr["ms"] > 0 else None,
                      "max_err_vs_fp64": tr["max_err"], "passed_gate": tr["passed"]})

@@ -247,13 +247,21 @@ typedef struct lsp_plan lsp_plan;
  * The ablation kernels (trig or staging non-zero) are FP32, scalar
  * (packed 0), k_reseed = freqs_per_thread = 16, standard periodogram only;
  * other combinations return LSP_E_UNSUPPORTED.
- * reserved = 1: objects with enough observations (FP32 40, more on grids of
- * a few hundred bins; FP64 8) get their trig sums from a nonuniform FFT, per
- * run of 2048 bins or, one object, of its whole grid, instead of pair by pair
- * (the same sums, no less exact), and the kernel the other fields name serves
- * the rest.  It is the choice of every call whose lsp_opts leave the kernel
- * options 0, and of a plan until lsp_plan_set_config says otherwise.  It needs block_threads x freqs_per_thread = 2048 (a single
- * object: any) and no ablation; other configurations read it as 0.
+ * transform: objects with enough observations (FP32 40, more on grids of a few
+ * hundred bins; FP64 8) get their trig sums from a nonuniform FFT, per run of
+ * 2048 bins or, one object, of its whole grid, instead of pair by pair, and
+ * the kernel the other fields name serves the rest.  It is the choice of every
+ * call whose lsp_opts leave the kernel options 0, and of a plan until
+ * lsp_plan_set_config says otherwise.  It needs block_threads x
+ * freqs_per_thread = 2048 (a single object: any) and no ablation; other
+ * configurations read it as 0.
+ *   0: off: every object takes the kernel that the other fields name;
+ *   1: on, beside any kernel;
+ *   what lsp_plan_get_config returns where it is on: on beside the kernel of
+ *      the same configuration, in this plan or another; off where one of
+ *      k_reseed, freqs_per_thread, block_threads, obs_split and packed was
+ *      changed since, so that a configuration read, changed and set runs the
+ *      kernel it then names.
  */
 typedef struct lsp_config {
   int32_t k_reseed;
@@ -263,7 +271,7 @@ typedef struct lsp_config {
   int32_t packed;      /* 1: packed f32x2 arithmetic across two reseed chains */
   int32_t trig;
   int32_t staging;
-  int32_t reserved;    /* 1: objects of enough observations take the transform path (below) */
+  int32_t transform;   /* objects of enough observations take the transform path (above) */
 } lsp_config;
 
 /*

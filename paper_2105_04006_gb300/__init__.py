@@ -63,12 +63,12 @@ class Config(ctypes.Structure):
     _fields_ = [("k_reseed", ctypes.c_int32), ("freqs_per_thread", ctypes.c_int32),
                 ("block_threads", ctypes.c_int32), ("obs_split", ctypes.c_int32),
                 ("packed", ctypes.c_int32), ("trig", ctypes.c_int32), ("staging", ctypes.c_int32),
-                ("reserved", ctypes.c_int32)]
+                ("transform", ctypes.c_int32)]
 
     def as_dict(self):
         return dict(k_reseed=self.k_reseed, freqs_per_thread=self.freqs_per_thread,
                     block_threads=self.block_threads, obs_split=self.obs_split, packed=self.packed,
-                    trig=self.trig, staging=self.staging)
+                    trig=self.trig, staging=self.staging, transform=int(self.transform != 0))
 
 
 class Trial(ctypes.Structure):
@@ -444,12 +444,15 @@ class Plan:
         """Whether objects of enough observations take the transform path (see lsp_config in lsp.h)."""
         c = Config()
         _check(lib().lsp_plan_get_config(self._h, ctypes.byref(c)))
-        return c.reserved == 1
+        return c.transform != 0
 
     def set_config(self, **cfg):
+        """Run the kernel that the given fields name, the others as they are.  The transform is off beside a
+        named kernel unless transform=1 is given too, as ``config`` does: ``b.set_config(**a.config)`` makes
+        plan b run as plan a."""
         c = Config()
         _check(lib().lsp_plan_get_config(self._h, ctypes.byref(c)))
-        c.reserved = 0  # a named kernel configuration runs that kernel, not the transform
+        c.transform = 0
         for k, v in cfg.items():
             setattr(c, k, int(v))
         _check(lib().lsp_plan_set_config(self._h, ctypes.byref(c)))

@@ -132,6 +132,13 @@ lsp_status check_grid(const lsp_grid* g) {
   return LSP_OK;
 }
 
+// The value of lsp_config::transform that is on beside this kernel only (> 1).
+int32_t transform_tag(const lsp_config& c) {
+  return 2 + (c.k_reseed & 31) + ((c.freqs_per_thread & 63) << 5) + ((c.block_threads / 32 & 15) << 11) +
+         ((c.packed & 1) << 15) + ((c.obs_split & 511) << 16);
+}
+bool transform_on(const lsp_config& c) { return c.transform == 1 || c.transform == transform_tag(c); }
+
 lsp_status resolve(int64_t n_obj, int64_t total_nt, const lsp_grid* g, const lsp_opts* opts_in,
                    const lsp_config* cfg, Layout* L, bool gls = false, int level = 0) {
   lsp_status st = check_grid(g);
@@ -166,7 +173,7 @@ lsp_status resolve(int64_t n_obj, int64_t total_nt, const lsp_grid* g, const lsp
   bool tf = l.prec == LSP_FP32 || !gls;
   int tf_min = l.prec == LSP_FP32 ? kTfMinObs : kTfMinObs64;
   if (n_obj > 1 && l.prec == LSP_FP32) tf_min = tf_min_obs(tf_min, l.n_f);
-  if (cfg) tf = tf && cfg->reserved == 1;
+  if (cfg) tf = tf && transform_on(*cfg);
   else tf = tf && !o.k_reseed && !o.freqs_per_thread && !o.block_threads && !o.obs_split;
   if (cfg) {
     k = cfg->k_reseed;
@@ -652,10 +659,10 @@ lsp_config config_of(const Layout& L) {
   c.freqs_per_thread = L.fpt;
   c.block_threads = L.threads;
   c.obs_split = L.tf && L.n_obj == 1 ? L.cfg_split : L.split;
-  c.reserved = L.tf;
   c.packed = L.packed;
   c.trig = L.abl % 3;
   c.staging = L.abl / 3;
+  c.transform = L.tf ? transform_tag(c) : 0;
   return c;
 }
 
@@ -770,8 +777,8 @@ bool cache_lookup(const char* path, const std::string& key, lsp_config* c) {
       // an entry from before the transform names the direct kernel only: the
       // default choice (on) stands beside it, off where the entry's tile does
       // not allow it
-      t.reserved = 1;
-      get("transform", &t.reserved);
+      t.transform = 1;
+      get("transform", &t.transform);
       get("staging", &t.staging);
       *c = t;
       found = true;
@@ -786,7 +793,7 @@ void cache_store(const char* path, const std::string& key, const lsp_config& c, 
   f << "{\"key\": \"" << key << "\", \"k_reseed\": " << c.k_reseed << ", \"freqs_per_thread\": "
     << c.freqs_per_thread << ", \"block_threads\": " << c.block_threads << ", \"obs_split\": "
     << c.obs_split << ", \"packed\": " << c.packed << ", \"trig\": " << c.trig << ", \"staging\": "
-    << c.staging << ", \"transform\": " << c.reserved << ", \"ms\": " << ms << ", \"max_err\": " << err
+    << c.staging << ", \"transform\": " << (c.transform ? 1 : 0) << ", \"ms\": " << ms << ", \"max_err\": " << err
     << "}\n";
 }
 
@@ -1482,7 +1489,7 @@ lsp_status lsp_plan_autotune_ex(lsp_plan* p, const double* t, const void* y, con
       if ((st = errors(Lg, cur_err))) { cleanup(); return st; }
       if (Lg.tf && g_nobj > 1) {  // and the direct kernel that serves the batch's short objects
         lsp_config cd = c;
-        cd.reserved = 0;
+        cd.transform = 0;
         Layout Ld;
         std::vector<double> direct((size_t)g_rows);
         if (resolve(g_nobj, g_total, &p->grid, &o1, &cd, &Ld, false, g_level) || Ld.total > gws_bytes) {

@@ -103,7 +103,7 @@ def test_a_configuration_that_does_not_fit_leaves_the_plan_as_it_was(fake, preci
     fake.fake_limit(fake.fake_used() + 400)
     c = lsp.Config()
     L.lsp_plan_get_config(h, ctypes.byref(c))
-    c.reserved = 0
+    c.transform = 0
     c.obs_split = 256
     assert L.lsp_plan_set_config(h, ctypes.byref(c)) == 3  # LSP_E_NOMEM
     runs(h, args, 1)

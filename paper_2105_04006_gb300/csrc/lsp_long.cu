@@ -46,6 +46,10 @@ namespace {
 
 constexpr int kThreads = 256;
 
+// y_exponent for FP32 factors: 2^-e has to be finite (magnitudes below 2^-126
+// keep their bits, which the product with 2^126 makes normal).
+__device__ __forceinline__ int y_exponent_f32(double sum_y2) { return max(y_exponent(sum_y2), -126); }
+
 // ------------------------------------------------------------------- spread
 __global__ void __launch_bounds__(kThreads) spread_f32(const RecF32* __restrict__ rec, const ObjInfo* __restrict__ obj,
                                                        uint32_t kc, int lg, long long* __restrict__ cells) {
@@ -57,7 +61,7 @@ __global__ void __launch_bounds__(kThreads) spread_f32(const RecF32* __restrict_
   f2_t poly[9];
 #pragma unroll
   for (int d = 0; d < 9; ++d) poly[d] = dup_<f2_t>(__ldg(&kTfPoly[d * 8 + r]));
-  const float y_sc = (float)pow2(-y_exponent(oi.sum_y2)), z_one = (float)pow2(z_bits(n)), w_one = (float)pow2(w_bits(n));
+  const float y_sc = (float)pow2(-y_exponent_f32(oi.sum_y2)), z_one = (float)pow2(z_bits(n)), w_one = (float)pow2(w_bits(n));
   float zr = 0.f, zi = 0.f, wr = 0.f, wi = 0.f, uz = 0.f, uw = 0.f;
   uint32_t cz = 0u, cw = 0u;
   const uint32_t mask = (1u << lg) - 1u;
@@ -252,7 +256,7 @@ __global__ void __launch_bounds__(kThreads, 2) pass2_f32(const Cx<f2_t>* __restr
   const f2_t inv = f2_pack((float)pow2(-z_bits(n)), (float)pow2(-w_bits(n)));
   const float nf = (float)oi.n;
   // the magnitudes' power of two comes back with the normalisation, in FP64 range
-  const double y_inv = pow2(y_exponent(oi.sum_y2));
+  const double y_inv = pow2(y_exponent_f32(oi.sum_y2));
   const float scale = (float)(oi.norm_scale * y_inv * y_inv);
   const int p = tid >> 4, r = tid & 15;
   const float xi4 = (float)pow2(2 - lg);  // 4 / Mg

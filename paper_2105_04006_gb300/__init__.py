@@ -240,11 +240,11 @@ _known_opts = {}
 
 def _opts_of(kw) -> Opts:
     """make_opts(**kw), built once per set of arguments; read-only (the library takes it by const pointer)."""
+    for v in kw.values():
+        if type(v) not in (str, int, bool):  # a tensor, say, may hold another number in the next call
+            return make_opts(**kw)
     key = tuple(kw.items())
-    try:
-        o = _known_opts.get(key)
-    except TypeError:  # an unhashable argument: make_opts says what is wrong with it
-        return make_opts(**kw)
+    o = _known_opts.get(key)
     if o is None:
         o = make_opts(**kw)
         if len(_known_opts) < 64:

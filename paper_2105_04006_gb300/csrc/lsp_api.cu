@@ -117,6 +117,17 @@ bool long_is_faster(int64_t n_t, int64_t n_f, int64_t runs, int64_t slots) {
   const double waves = (double)((runs + slots - 1) / slots);
   return waves * (12.0 + (double)n_t / 150.0) > 30.0 + (double)n_f / 12500.0;
 }
+// One object of the generalized periodogram goes run by run or to the direct
+// kernel with its observations split over the SMs, by a model of their times
+// (us, GB300): a wave of run CTAs 22 + N_t / 140, as every run spreads all
+// observations; the split kernel 74 + N_t / 1500 + N_t N_f / 2.15e6.  Measured,
+// runs | split: N_t 1e4, N_f 1000 95 | 84, 3000 95 | 105; N_t 3e4, N_f 3000
+// 232 | 144, 1e4 234 | 215, 3e4 239 | 503; N_t 1e5, N_f 3000 726 | 300, 1e4 739 |
+// 584, 3e4 751 | 1574; below N_t 3000 the runs are the faster on any grid.
+bool split_gls_is_faster(int64_t n_t, int64_t n_f, int64_t runs, int64_t slots) {
+  const double n = (double)n_t, waves = (double)((runs + slots - 1) / slots);
+  return waves * (22.0 + n / 140.0) > 74.0 + n / 1500.0 + n * (double)n_f / 2.15e6;
+}
 // The paths a call may take, by the workspace they need: everything; without
 // the whole-grid transform and with fewer FP64 run CTAs; the direct kernels
 // alone.
@@ -235,6 +246,9 @@ lsp_status resolve(int64_t n_obj, int64_t total_nt, const lsp_grid* g, const lsp
   tf = tf && level < 2 && !abl && n_obj > 0 && (n_obj == 1 ? total_nt >= tf_min : chunk == kTfBins);
   const int64_t tf_chunks = (l.n_f + kTfBins - 1) / kTfBins;
   tf = tf && n_obj * tf_chunks < ((int64_t)1 << 31);  // 32-bit item numbers
+  // (with less scratch than the split kernel needs, level 1 takes the runs)
+  if (tf && gls && n_obj == 1 && level < 1)
+    tf = !split_gls_is_faster(total_nt, l.n_f, tf_chunks, 2 * (int64_t)current_sm_count());
   l.tf = tf;
   l.tf_min = tf_min;
   l.split = split;

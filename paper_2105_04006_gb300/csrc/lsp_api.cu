@@ -46,7 +46,10 @@ lsp_status cuda_fail(cudaError_t e, const char* what) {
 constexpr size_t kAlign = 256;
 size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
-int current_sm_count() {
+}  // namespace
+
+// SMs of the current device.
+int lsp::current_sm_count() {
   static std::mutex mu;
   static int cache[64] = {0};
   int dev = 0;
@@ -62,6 +65,8 @@ int current_sm_count() {
   }
   return cache[dev];
 }
+
+namespace {
 
 // Resolved configuration and workspace layout of one call.
 struct Layout {

@@ -25,6 +25,8 @@ inline cudaError_t allow_dyn_smem(Kern kern, size_t dyn) {
   return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
 }
 
+int current_sm_count();  // of the current device, asked of the runtime once (152 on an error)
+
 // CTAs of a kernel resident per SM (0 on an error), asked of the runtime once
 // per device, kernel and shape: the query costs several microseconds, as much
 // as the smallest calls' kernels.

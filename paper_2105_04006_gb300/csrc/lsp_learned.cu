@@ -482,7 +482,8 @@ lsp_status gemm(const Gemm& q, cudaStream_t s) {
   // epilogue's transposed copy (172 with the fewer launches around it).
   const int row_tiles = (q.M + umma::BM - 1) / umma::BM * (q.splits < 1 ? 1 : q.splits);
   int n_tile = q.N >= umma::MAX_BN ? umma::MAX_BN : (q.N + 15) / 16 * 16;
-  while (n_tile > 32 && (int64_t)row_tiles * ((q.N + n_tile - 1) / n_tile) < 148) n_tile = (n_tile / 2 + 15) / 16 * 16;
+  while (n_tile > 32 && (int64_t)row_tiles * ((q.N + n_tile - 1) / n_tile) < current_sm_count())
+    n_tile = (n_tile / 2 + 15) / 16 * 16;
   CUtensorMap ma, mb;
   lsp_status st = make_map(&ma, q.A, q.M, q.K, q.lda, umma::BM, "GEMM operand A");
   if (st) return st;
@@ -1285,8 +1286,7 @@ lsp_status refine_impl(const double* t, const float* y, const int64_t* offsets, 
   // [5], [6] their items, [7], [8] their queues
   uint32_t* cnt = (uint32_t*)(ws + r.off_cnt);
   const double df = (grid->f_max - grid->f_min) / (double)grid->n_f;
-  int n_sm = 152, dev = 0;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+  const int n_sm = current_sm_count();
   int bps = main_blocks_per_sm(0, 1, kRefineK, 2 * kRefineK, kRefineThreads, 0);
   if (bps < 1) bps = 1;
 

@@ -96,9 +96,12 @@ constexpr int kGateObjects = 8;  // objects the autotuner's error gate checks
 // cost per run of bins hardly depends on N_t, the direct kernel's is
 // proportional to it.  Measured (2000 objects of equal N_t, N_f = 1e5,
 // transform | direct, ms): N_t 32 2.2 | 1.9, 48 2.2 | 2.6, 100 2.4 | 5.0; later
-// cuts of the run's cost put the crossing at N_t 36, the generalized
-// periodogram's at 43.
+// cuts of the run's cost put the crossing at N_t 36 (in a batch of a few
+// objects, where one run's latency counts, at 50: 29.9 | 28.7 us at 40).  The
+// generalized periodogram's (1000 objects, N_f = 1e5, us): N_t 40 1540 | 1500, 42
+// 1541 | 1559, 44 1541 | 1621.
 constexpr int kTfMinObs = 40;
+constexpr int kTfMinObsGls = 42;
 constexpr int kTfMinObs64 = 8;
 // That line is for whole runs.  A run costs the same however few of its bins
 // lie in the grid, the direct kernel's warps of 512 bins past its end cost
@@ -187,7 +190,7 @@ lsp_status resolve(int64_t n_obj, int64_t total_nt, const lsp_grid* g, const lsp
   // the transform is the library's own choice: a call that names a kernel
   // option gets the direct kernel it names
   bool tf = l.prec == LSP_FP32 || !gls;
-  int tf_min = l.prec == LSP_FP32 ? kTfMinObs : kTfMinObs64;
+  int tf_min = l.prec == LSP_FP64 ? kTfMinObs64 : gls ? kTfMinObsGls : kTfMinObs;
   if (n_obj > 1 && l.prec == LSP_FP32) tf_min = tf_min_obs(tf_min, l.n_f);
   if (cfg) tf = tf && transform_on(*cfg);
   else tf = tf && !o.k_reseed && !o.freqs_per_thread && !o.block_threads && !o.obs_split;

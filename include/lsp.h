@@ -62,7 +62,10 @@ typedef enum lsp_status {
 
 typedef enum lsp_precision {
   LSP_FP32 = 0, /* trig sums in FP32; phases reduced in FP64 / fixed point (y, power: float) */
-  LSP_FP64 = 1  /* everything in FP64 (y, power: double) */
+  LSP_FP64 = 1  /* y, power: double; powers within 1e-10 of exact sums.  Objects of 8 observations
+                   and more: sums in 64-bit fixed point and two-float arithmetic (48 bits),
+                   good to about 1e-14 of their norm; others, the generalized periodogram and
+                   calls that name a kernel option: FP64 throughout */
 } lsp_precision;
 
 typedef enum lsp_norm {

@@ -109,7 +109,9 @@ constexpr int kTfMinObs64 = 8;
 // share of the runs' warps without bins.  20 000 objects, transform | direct,
 // us: N_f 512, N_t 80 732 | 711, 100 778 | 821; N_f 1000, N_t 56 691 | 682,
 // 64 684 | 727; N_f 2049, N_t 40 1098 | 1015, 56 1100 | 1235.  In FP64 the
-// transform is the faster on any grid (5000 objects, N_t 8: N_f 512 1005 | 1968).
+// transform is the faster on any grid (5000 objects, N_t 8: N_f 512 1005 | 1968;
+// 2 objects, N_t 8, N_f 256 68 | 108), and from N_t 60 on, or on grids of 20 000 bins
+// and more, as exact (below that its sums' 1e-14 shows: N_t 8, N_f 3000 3e-15 | 3e-16).
 int tf_min_obs(int base, int64_t n_f) {
   const int64_t runs = (n_f + kTfBins - 1) / kTfBins, warps = (n_f + 511) / 512;
   return (int)(base * (4 * runs + warps) / (2 * warps));
@@ -120,7 +122,9 @@ int tf_min_obs(int base, int64_t n_f) {
 // whole grid 30 + N_f / 12500.  Measured, runs | whole grid: N_t 3000, N_f 1e5
 // 41 | 43; N_t 1e4, N_f 1e5 78 | 43; N_t 3000, N_f 4e5 49 | 65; N_t 1e5, N_f 1e6
 // 1480 | 127.  In FP64 the whole grid is always the faster (N_t 1000, N_f 1e5:
-// 200 | 82; the direct kernel takes 1400).
+// 200 | 82), also than the direct kernel, whose FP64 chain per observation is
+// long however short the grid: whole grid | direct at N_t 8, N_f 64 58 | 96; 8, 3e4
+// 63 | 96; 100, 512 66 | 141; 1000, 1e5 82 | 1400.
 bool long_is_faster(int64_t n_t, int64_t n_f, int64_t runs, int64_t slots) {
   const double waves = (double)((runs + slots - 1) / slots);
   return waves * (12.0 + (double)n_t / 150.0) > 30.0 + (double)n_f / 12500.0;

@@ -6,10 +6,13 @@
 //   Rec      rec[total_nt]              per-observation records (prologue)
 //   int32    order[n_obj]               objects by decreasing N_t (LPT queue)
 //   uint32   hist[LSP_HIST_BINS + 1]    counting-sort scratch
-//   uint32   queue[4]                   persistent-kernel work counter
+//   uint32   queue[6]                   work counters, last-CTA tickets, list lengths
 //   ChunkBest best[n_obj * n_chunks]    first maximum of each frequency chunk
 //   ChunkCand cand[n_obj * n_chunks]    top-3 local maxima + edge bins (top_k > 1)
 //   partial  part[split * n_f]          split-N_t partial sums (single object)
+//   stats    one StatAcc per 256 observations (single object)
+//   cells    fixed-point cells: of every CTA (FP64 runs) or of the whole grid
+//   t, row   whole-grid transform: after its first pass; its powers
 #pragma once
 
 #include <type_traits>
@@ -24,8 +27,8 @@ namespace lsp {
 
 // Per-object statistics written by the prologue (Section 2: zero-mean y).
 struct __align__(16) ObjInfo {
-  double t0;         // midpoint of the object's time span; phases use t - t0
-  double ymean;      // FP64 mean of y (0 when centring is off)
+  double t0;         // midpoint of the object's time span; phases use t - t0 (batches that
+  double ymean;      // FP64 mean of y (0 when centring is off)   take the transform: tf_scale_put)
   double sum_y2;     // FP64 sum of the centred y^2
   int64_t begin;     // offsets[o]
   int32_t n;         // N_t (0 for an object with bad offsets)

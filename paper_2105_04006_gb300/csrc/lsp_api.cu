@@ -702,7 +702,7 @@ void drop_graph(lsp_plan* p) {
 
 // Room for `bytes` in the plan's workspace.  Where it cannot be had the plan
 // keeps the workspace it has (or, if even that was lost to another allocation
-// in between, none: ws_cap 0, which lsp_plan_execute tries to mend).
+// in between, none: lsp_plan_execute then refuses until a configuration is set).
 lsp_status ensure_ws(lsp_plan* p, size_t bytes) {
   if (p->ws && bytes <= p->ws_cap) return LSP_OK;
   const size_t size = bytes ? bytes : kAlign, had = p->ws_cap;
@@ -1094,7 +1094,8 @@ lsp_status lsp_plan_execute(lsp_plan* p, const double* t, const void* y, const i
   lsp_status st = check_io(p->total_nt, t, y);
   if (st) return st;
   if (p->n_obj > 1 && !offsets) return fail(LSP_E_ARG, "offsets must not be NULL");
-  if ((st = ensure_ws(p, p->L.total))) return st;
+  if (!p->ws || p->ws_cap < p->L.total)
+    return fail(LSP_E_WORKSPACE, "the plan lost its workspace when it could not grow: set its configuration again");
   const void* args[5] = {t, y, offsets, power_out, peaks};
   bool same = p->exec != nullptr;
   for (int i = 0; i < 5 && same; ++i) same = args[i] == p->cap_args[i];

@@ -144,3 +144,28 @@ def test_autotune_tries_splits_around_the_direct_kernels_own(fake, precision):
     tried = set(t.config.obs_split for t in trials)
     assert tried >= set(c.obs_split * f // 4 for f in (1, 2, 4, 8, 16)), (tried, c.obs_split)
     """)
+
+
+def test_a_plan_that_lost_its_workspace_refuses_until_it_has_one(fake):
+    """The old size is not to be had either: no launch on memory the plan does not have, no allocation in an
+    execution, and a configuration set later brings the plan back."""
+    fake("""
+    g = lsp.Grid(0.1, 10.0, 100_000)
+    args = inputs([9000], np.float32)
+    st, h = plan([9000], g)
+    assert st == 0
+    c = lsp.Config()
+    L.lsp_plan_get_config(h, ctypes.byref(c))
+    pk = dev(np.zeros(40, np.uint8))
+    fake.fake_limit(0)
+    d = lsp.Config.from_buffer_copy(c)
+    d.obs_split = 256
+    assert L.lsp_plan_set_config(h, ctypes.byref(d)) == 3
+    before = fake.fake_launches()
+    assert L.lsp_plan_execute(h, *args, None, pk, None) == 4  # LSP_E_WORKSPACE
+    fake.fake_limit(1 << 40)
+    assert L.lsp_plan_execute(h, *args, None, pk, None) == 4
+    assert fake.fake_launches() == before and fake.fake_outside() == 0
+    assert L.lsp_plan_set_config(h, ctypes.byref(c)) == 0
+    runs(h, args, 1)
+    """)
